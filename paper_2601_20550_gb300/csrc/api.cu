@@ -733,12 +733,12 @@ heom_status heom_response_2d(heom_hier *h, const heom_state *rho_eq, const heom_
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     check_tc_error(h);
     PhaseRange phase("heom: 2D DFT");
+    DeviceBuffer work((size_t)dft2d_work(n1, n3) * 16);
     const double dtau = g->dt_fs * g->steps_per_sample;
     for (int it = 0; it < nt2; ++it) {
       double2 *RI = (double2 *)Rdev.p + (int64_t)it * 2 * n1 * n3;
-      dft2d_sc_kernel<<<(n1 * n3 + 255) / 256, 256, 0, h->stream>>>(RI, RI + (int64_t)n1 * n3, n1, n3, dtau,
-                                                                     (double *)SCdev.p + (int64_t)it * n1 * n3);
-      count_launch(1);
+      dft2d_sc(RI, RI + (int64_t)n1 * n3, n1, n3, dtau, (double *)SCdev.p + (int64_t)it * n1 * n3, (double2 *)work.p,
+               h->stream);
       LAUNCH_CHECK();
     }
     std::vector<double> Rh((size_t)nt2 * 2 * n1 * n3 * 2);
@@ -791,7 +791,7 @@ heom_status heom_spectrum_2d(const double *R_I, const double *R_II, int n_t2, in
     return fail(HEOM_EINVAL, "bad spectrum arguments");
   return guarded([&]() -> heom_status {
     const size_t blk = (size_t)n1 * n3;
-    DeviceBuffer R((size_t)n_t2 * 2 * blk * 16), S((size_t)n_t2 * blk * 8);
+    DeviceBuffer R((size_t)n_t2 * 2 * blk * 16), S((size_t)n_t2 * blk * 8), work((size_t)dft2d_work(n1, n3) * 16);
     for (int it = 0; it < n_t2; ++it) {
       CUDA_TRY(cudaMemcpy((char *)R.p + (size_t)it * 2 * blk * 16, R_I + it * blk * 2, blk * 16, cudaMemcpyHostToDevice));
       CUDA_TRY(cudaMemcpy((char *)R.p + ((size_t)it * 2 + 1) * blk * 16, R_II + it * blk * 2, blk * 16,
@@ -799,8 +799,7 @@ heom_status heom_spectrum_2d(const double *R_I, const double *R_II, int n_t2, in
     }
     for (int it = 0; it < n_t2; ++it) {
       const double2 *RI = (const double2 *)R.p + (size_t)it * 2 * blk;
-      dft2d_sc_kernel<<<(unsigned)((blk + 255) / 256), 256>>>(RI, RI + blk, n1, n3, dtau_fs, (double *)S.p + it * blk);
-      count_launch(1);
+      dft2d_sc(RI, RI + blk, n1, n3, dtau_fs, (double *)S.p + it * blk, (double2 *)work.p, 0);
       LAUNCH_CHECK();
     }
     CUDA_TRY(cudaMemcpy(S_C, S.p, S.bytes, cudaMemcpyDeviceToHost));

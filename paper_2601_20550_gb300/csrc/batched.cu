@@ -321,12 +321,11 @@ heom_status heom_response_2d_batched(heom_hier *const *hs, const heom_state *con
       response_2d_multi(hs, eqs, n_sets, g, Rdev);
     }
     const double dtau = g->dt_fs * g->steps_per_sample;
+    DeviceBuffer work((size_t)dft2d_work(n1, n3) * 16);
     for (int i = 0; i < n_sets; ++i)
       for (int it = 0; it < nt2; ++it) {
         double2 *RI = Rdev[i] + (int64_t)it * 2 * one;
-        dft2d_sc_kernel<<<(unsigned)((one + 255) / 256), 256, 0, st>>>(RI, RI + one, n1, n3, dtau,
-                                                                       (double *)SCall.p + (size_t)i * blk + it * one);
-        count_launch(1);
+        dft2d_sc(RI, RI + one, n1, n3, dtau, (double *)SCall.p + (size_t)i * blk + it * one, (double2 *)work.p, st);
         LAUNCH_CHECK();
       }
     std::vector<double> Rh(Rall.bytes / 8);

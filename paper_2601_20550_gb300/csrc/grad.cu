@@ -222,7 +222,7 @@ static void backprop_span(AdjCtx &c, const double2 *start, int64_t N, int B, dou
   }
 }
 
-// Adjoint of the 2D Fourier sums of dft2d_sc_kernel: Rbar = i conj(F) Sbar for
+// Adjoint of the 2D Fourier sums of dft2d_sc: Rbar = i conj(F) Sbar for
 // S = Im(F R), per t2 and pathway ([n1][n3] each).
 static void dft2d_adjoint(const double *Sbar, int n1, int n3, double dtau, std::vector<double> &RbarI,
                           std::vector<double> &RbarII) {
@@ -326,14 +326,12 @@ extern "C" heom_status heom_response_2d_grad(heom_hier *h, const heom_state *rho
     }
     // ---- forward: R and S_C, loss and the adjoint of S_C (host)
     const size_t blk = (size_t)n1 * n3;
-    DeviceBuffer Rdev((size_t)nt2 * 2 * blk * 16), SCdev((size_t)nt2 * blk * 8);
+    DeviceBuffer Rdev((size_t)nt2 * 2 * blk * 16), SCdev((size_t)nt2 * blk * 8), work((size_t)dft2d_work(n1, n3) * 16);
     CUDA_TRY(cudaMemsetAsync(Rdev.p, 0, Rdev.bytes, st));
     response_2d_rows_impl<double>(h, rho_eq, g, 0, n1, (double2 *)Rdev.p);
     for (int it = 0; it < nt2; ++it) {
       double2 *RI = (double2 *)Rdev.p + (int64_t)it * 2 * blk;
-      dft2d_sc_kernel<<<(unsigned)((blk + 255) / 256), 256, 0, st>>>(RI, RI + blk, n1, n3, dtau,
-                                                                     (double *)SCdev.p + (int64_t)it * blk);
-      count_launch(1);
+      dft2d_sc(RI, RI + blk, n1, n3, dtau, (double *)SCdev.p + (int64_t)it * blk, (double2 *)work.p, st);
       LAUNCH_CHECK();
     }
     std::vector<double> SC((size_t)nt2 * blk);

@@ -3,32 +3,68 @@
 
 namespace heom {
 
-__global__ void dft2d_sc_kernel(const double2 *__restrict__ RI, const double2 *__restrict__ RII,
-                                int n1, int n3, double dtau, double *__restrict__ SC) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n1 * n3) return;
-  const int q = idx / n3, p = idx % n3;
-  const int qf = (n1 - q) % n1;   // -Omega1 for the rephasing part
-  double sr = 0, snr = 0;         // imaginary parts only
-  for (int j = 0; j < n1; ++j) {
-    const double wj = j == 0 ? 0.5 : 1.0;
-    double s1r, c1r, s1n, c1n;
-    sincospi(2.0 * (double)((long long)qf * j % n1) / n1, &s1r, &c1r);
-    sincospi(2.0 * (double)((long long)q * j % n1) / n1, &s1n, &c1n);
-    for (int k = 0; k < n3; ++k) {
-      const double w = wj * (k == 0 ? 0.5 : 1.0);
-      double s3, c3;
-      sincospi(2.0 * (double)((long long)p * k % n3) / n3, &s3, &c3);
-      const double2 a = RI[(long long)j * n3 + k];
-      const double2 b = RII[(long long)j * n3 + k];
-      // Im[(cos + i sin)(x + i y)] = sin x + cos y, phase = phase1 + phase3
-      const double cr = c1r * c3 - s1r * s3, sr_ = s1r * c3 + c1r * s3;
-      const double cn = c1n * c3 - s1n * s3, sn = s1n * c3 + c1n * s3;
-      sr += w * (sr_ * a.x + cr * a.y);
-      snr += w * (sn * b.x + cn * b.y);
-    }
+void count_launch(uint64_t n);
+
+__global__ void __launch_bounds__(256) dft_twiddle_kernel(double2 *__restrict__ tw, int n1, int n3) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n1 + n3) return;
+  const int k = i < n1 ? i : i - n1, n = i < n1 ? n1 : n3;
+  double s, c;
+  sincospi(2.0 * (double)k / n, &s, &c);
+  tw[i] = make_double2(c, s);
+}
+
+__global__ void __launch_bounds__(128) dft_rows_kernel(const double2 *__restrict__ RI, const double2 *__restrict__ RII,
+                                                       const double2 *__restrict__ tw3, int n1, int n3,
+                                                       double2 *__restrict__ F) {
+  const int j = blockIdx.x, p = blockIdx.y * blockDim.x + threadIdx.x;
+  if (p >= n3) return;
+  const double2 *R = (blockIdx.z ? RII : RI) + (int64_t)j * n3;
+  const double2 r0 = R[0];
+  double re = 0.5 * r0.x, im = 0.5 * r0.y;
+  int i = 0;
+#pragma unroll 4
+  for (int k = 1; k < n3; ++k) {
+    i += p;
+    i -= i >= n3 ? n3 : 0;
+    const double2 r = R[k], t = tw3[i];
+    re = fma(t.x, r.x, re);
+    im = fma(t.x, r.y, im);
+    re = fma(-t.y, r.y, re);
+    im = fma(t.y, r.x, im);
   }
-  SC[idx] = dtau * dtau * (sr + snr);
+  F[((int64_t)blockIdx.z * n1 + j) * n3 + p] = make_double2(re, im);
+}
+
+__global__ void __launch_bounds__(128) dft_cols_kernel(const double2 *__restrict__ F, const double2 *__restrict__ tw1,
+                                                       int n1, int n3, double dtau, double *__restrict__ SC) {
+  const int q = blockIdx.x, p = blockIdx.y * blockDim.x + threadIdx.x;
+  if (p >= n3) return;
+  const double2 *FI = F + p, *FII = F + (int64_t)n1 * n3 + p;
+  double s = 0.5 * (FI[0].y + FII[0].y), s2 = 0.0;
+  int i = 0;
+#pragma unroll 4
+  for (int j = 1; j < n1; ++j) {
+    i += q;
+    i -= i >= n1 ? n1 : 0;
+    const double2 a = FI[(int64_t)j * n3], b = FII[(int64_t)j * n3], t = tw1[i];
+    // Im[conj(t) a] + Im[t b]: the rephasing part enters at -Omega1
+    s = fma(t.x, a.y, s);
+    s = fma(t.x, b.y, s);
+    s2 = fma(t.y, b.x, s2);
+    s2 = fma(-t.y, a.x, s2);
+  }
+  SC[(int64_t)q * n3 + p] = dtau * dtau * (s + s2);
+}
+
+void dft2d_sc(const double2 *RI, const double2 *RII, int n1, int n3, double dtau, double *SC, double2 *work,
+              cudaStream_t st) {
+  double2 *F = work, *tw1 = work + 2 * (int64_t)n1 * n3, *tw3 = tw1 + n1;
+  const unsigned pb = (unsigned)((n3 + 127) / 128);
+  dft_twiddle_kernel<<<(unsigned)((n1 + n3 + 255) / 256), 256, 0, st>>>(tw1, n1, n3);
+  dft_rows_kernel<<<dim3((unsigned)n1, pb, 2), 128, 0, st>>>(RI, RII, tw3, n1, n3, F);
+  dft_cols_kernel<<<dim3((unsigned)n1, pb), 128, 0, st>>>(F, tw1, n1, n3, dtau, SC);
+  count_launch(3);
 }
 
 __global__ void dft1d_kernel(const double2 *__restrict__ R, int n, double dtau, double *__restrict__ I) {
