@@ -62,11 +62,13 @@ namespace heom {
 void stability_check(heom_hier *h, double dt) {
   if (!(dt > 0) || !std::isfinite(dt)) throw Fail{HEOM_EINVAL, "dt must be > 0"};
   const Model &M = h->M;
-  std::vector<double> A = M.H, w, Z;
-  jacobi_eigh(A, M.d, w, Z);
-  double spread = w.back() - w.front();
-  double maxdecay = 0;
-  for (double g : M.decay) maxdecay = std::max(maxdecay, g);
+  if (h->spread < 0) {   // of the model, not of dt: the d x d eigenvalues take 0.1 s at d = 216
+    std::vector<double> A = M.H, w, Z;
+    jacobi_eigh(A, M.d, w, Z);
+    for (double g : M.decay) h->max_decay = std::max(h->max_decay, g);
+    h->spread = w.back() - w.front();
+  }
+  const double spread = h->spread, maxdecay = h->max_decay;
   if (dt * spread > 2.78 || dt * maxdecay > 2.78)
     throw Fail{HEOM_EUNSTABLE, "dt outside the RK4 stability region (dt*spread(H) = " +
                                    std::to_string(dt * spread) + ", dt*max decay = " +

@@ -132,6 +132,7 @@ struct heom_hier {
   float *mu_vb32 = nullptr, *mup_vb32 = nullptr, *mum_vb32 = nullptr;
   double *mu_vb64 = nullptr;                     // mu in the coupling basis (traces)
   bool on_device = false;
+  double spread = -1.0, max_decay = 0.0;   // Bohr spread of H_S' (< 0: not computed yet), largest decay rate
   // copy of the model description (for the parameter gradient)
   heom_model desc{};
   std::vector<heom_mode> desc_modes;
