@@ -75,11 +75,12 @@ void stability_check(heom_hier *h, double dt) {
                                    std::to_string(dt * maxdecay) + ")"};
 }
 
-// Launch-shape autotuner for the grid-stride stage kernels.  The first launch of
-// a kernel kind at a given size times every candidate (block of 64, 128 or 256
-// threads; 4, 16 or 64 blocks per SM, capped at one element per thread) on the
-// real operands -- three timed launches each after one untimed -- and keeps the
-// fastest for this hierarchy; a size whose default launch already takes over
+// Launch-shape autotuner of the stage kernels.  The first launch of a kernel kind
+// at a given size times every candidate (grid_shapes: blocks of 64, 128 or 256
+// threads, 4, 16 or 64 blocks per SM, capped at one element per thread, for the
+// grid-stride kernels; three block sizes of the FP64 engine, whose grid follows from the
+// size) on the real operands -- three timed launches each after one untimed --
+// and keeps the fastest for this hierarchy; a size whose default launch already takes over
 // 50 ms keeps the default.  Candidate launches repeat the caller's first
 // stage, whose output is scratch that the step overwrites next, so tuning
 // changes no result.  Inside a stream capture, or when timing fails, the
@@ -87,8 +88,9 @@ void stability_check(heom_hier *h, double dt) {
 enum TuneKind { kTuneStage64 = 0, kTuneStageVb = 1 };
 
 static std::pair<int, int> tuned_shape(heom_hier *h, int kind, int64_t total, cudaStream_t st,
+                                       const std::pair<int, int> &dflt,
+                                       const std::vector<std::pair<int, int>> &candidates,
                                        const std::function<void(int, int)> &launch) {
-  const std::pair<int, int> dflt(256, grid_for(total));
   auto it = h->tuned.find({kind, total});
   if (it != h->tuned.end()) return it->second;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -118,30 +120,115 @@ static std::pair<int, int> tuned_shape(heom_hier *h, int kind, int64_t total, cu
       return dflt;
     }
   }
-  for (int block : {64, 128, 256})
-    for (int per_sm : {4, 16, 64}) {
-      const int64_t need = (total + block - 1) / block;
-      const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(need, 152LL * per_sm * 256 / block));
-      launch(block, grid);
-      cudaEventRecord(e0, st);
-      for (int r = 0; r < 3; ++r) launch(block, grid);
-      cudaEventRecord(e1, st);
-      float ms = 0.f;
-      if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
-        ok = false;
-        break;
-      }
-      if (ms < best_ms) {
-        best_ms = ms;
-        best = {block, grid};
-      }
+  for (const auto &c : candidates) {
+    launch(c.first, c.second);
+    cudaEventRecord(e0, st);
+    for (int r = 0; r < 3; ++r) launch(c.first, c.second);
+    cudaEventRecord(e1, st);
+    float ms = 0.f;
+    if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
+      ok = false;
+      break;
     }
+    if (ms < best_ms) {
+      best_ms = ms;
+      best = c;
+    }
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   LAUNCH_CHECK();
   if (!ok) return dflt;
   h->tuned[{kind, total}] = best;
   return best;
+}
+
+static std::vector<std::pair<int, int>> grid_shapes(int64_t total) {
+  std::vector<std::pair<int, int>> v;
+  for (int block : {64, 128, 256})
+    for (int per_sm : {4, 16, 64}) {
+      const int64_t need = (total + block - 1) / block;
+      v.emplace_back(block, (int)std::max<int64_t>(1, std::min<int64_t>(need, 152LL * per_sm * 256 / block)));
+    }
+  return v;
+}
+
+void work_in(heom_hier *h, const double2 *x, double2 *out, double2 *tmp, int branches, cudaStream_t st) {
+  const int64_t items = (int64_t)branches * h->M.n_ado, elems = items * h->M.d * h->M.d;
+  if (!h->f64.ready) {
+    if (x != out) CUDA_TRY(cudaMemcpyAsync(out, x, elems * 16, cudaMemcpyDeviceToDevice, st));
+  } else if (h->rot.ready) {
+    rotate<double2, double2>(h->rot, true, x, out, tmp, items, st);
+  } else {
+    sim_left_kernel<double2><<<grid_for(elems), 256, 0, st>>>(x, tmp, h->U64, h->M.d, elems);
+    sim_right_kernel<double2><<<grid_for(elems), 256, 0, st>>>(tmp, out, h->U64, h->M.d, elems);
+    count_launch(2);
+  }
+  LAUNCH_CHECK();
+}
+
+void work_out(heom_hier *h, const double2 *x, double2 *out, double2 *tmp, int branches, cudaStream_t st) {
+  const int64_t items = (int64_t)branches * h->M.n_ado, elems = items * h->M.d * h->M.d;
+  if (!h->f64.ready) {
+    if (x != out) CUDA_TRY(cudaMemcpyAsync(out, x, elems * 16, cudaMemcpyDeviceToDevice, st));
+  } else if (h->rot.ready) {
+    rotate<double2, double2>(h->rot, false, x, out, tmp, items, st);
+  } else {
+    sim_left_kernel<double2><<<grid_for(elems), 256, 0, st>>>(x, tmp, h->UT64, h->M.d, elems);
+    sim_right_kernel<double2><<<grid_for(elems), 256, 0, st>>>(tmp, out, h->UT64, h->M.d, elems);
+    count_launch(2);
+  }
+  LAUNCH_CHECK();
+}
+
+void rk4_work64(heom_hier *h, double2 *y, double2 *wa, double2 *wb, int branches, double dt, int64_t nsteps,
+                cudaStream_t st) {
+  const int64_t total = (int64_t)branches * h->M.n_ado * h->M.d * h->M.d;
+  if (total == 0 || nsteps <= 0) return;
+  if (h->f64.ready) {
+    // the commutator part of a stage goes to its output, in the last stage (out = y)
+    // to the free scratch
+    const F64Buf b[4] = {{&h->f64, y, y, wa, wa, branches},
+                         {&h->f64, wa, y, wb, wb, branches},
+                         {&h->f64, wb, y, wa, wa, branches},
+                         {&h->f64, wa, y, y, wb, branches}};
+    const double al[4] = {dt / 4, dt / 3, dt / 2, dt};
+    const auto shapes = f64_shapes(b[0]);
+    const auto sh = tuned_shape(h, kTuneStage64, total, st, shapes[0], shapes,
+                                [&](int block, int) { f64_stage(b[0], al[0], block, st); });
+    for (int64_t s = 0; s < nsteps; ++s)
+      for (int q = 0; q < 4; ++q) f64_stage(b[q], al[q], sh.first, st);
+    LAUNCH_CHECK();
+    return;
+  }
+  const DevModel<double> &dm = h->dm64;
+  const auto sh = tuned_shape(h, kTuneStage64, total, st, {256, grid_for(total)}, grid_shapes(total),
+                              [&](int block, int grid) {
+                                stage_kernel<double><<<grid, block, 0, st>>>(y, y, wa, dt / 4, dm, total);
+                                count_launch(1);
+                              });
+  const int grid = sh.second, block = sh.first;
+  for (int64_t s = 0; s < nsteps; ++s) {
+    stage_kernel<double><<<grid, block, 0, st>>>(y, y, wa, dt / 4, dm, total);
+    stage_kernel<double><<<grid, block, 0, st>>>(wa, y, wb, dt / 3, dm, total);
+    stage_kernel<double><<<grid, block, 0, st>>>(wb, y, wa, dt / 2, dm, total);
+    stage_kernel<double><<<grid, block, 0, st>>>(wa, y, y, dt, dm, total);
+    count_launch(4);
+  }
+  LAUNCH_CHECK();
+}
+
+void rhs_work64(heom_hier *h, const double2 *w, double2 *out, int branches, cudaStream_t st) {
+  if (h->f64.ready) {
+    const F64Buf b{&h->f64, w, nullptr, out, out, branches};
+    f64_stage(b, 1.0, f64_shapes(b)[0].first, st);
+  } else {
+    const int64_t n = (int64_t)branches * h->M.n_ado * h->M.d * h->M.d;
+    CUDA_TRY(cudaMemsetAsync(out, 0, (size_t)n * 16, st));
+    stage_kernel<double><<<grid_for(n), 256, 0, st>>>(w, out, out, 1.0, h->dm64, n);
+    count_launch(1);
+  }
+  LAUNCH_CHECK();
 }
 
 // One RK4 step on branches [y] with scratch wa, wb, Horner form:
@@ -172,7 +259,8 @@ void rk4_steps(heom_hier *h, typename CxT<R>::type *y, typename CxT<R>::type *wa
         count_launch(4);
       }
     } else {
-      const auto sh = tuned_shape(h, kTuneStageVb, total, st, [&](int block, int grid) {
+      const auto sh = tuned_shape(h, kTuneStageVb, total, st, {256, grid_for(total)}, grid_shapes(total),
+                                  [&](int block, int grid) {
         stage_kernel_vb<<<grid, block, 0, st>>>(fy, fy, fa, (float)(dt / 4), h->vb, total);
         count_launch(1);
       });
@@ -188,36 +276,26 @@ void rk4_steps(heom_hier *h, typename CxT<R>::type *y, typename CxT<R>::type *wa
     LAUNCH_CHECK();
     return;
   }
-  const auto sh = tuned_shape(h, kTuneStage64, total, st, [&](int block, int grid) {
-    stage_kernel<R><<<grid, block, 0, st>>>(y, y, wa, (R)(dt / 4), dm, total);
-    count_launch(1);
-  });
-  const int grid = sh.second, block = sh.first;
-  for (int64_t s = 0; s < nsteps; ++s) {
-    stage_kernel<R><<<grid, block, 0, st>>>(y, y, wa, (R)(dt / 4), dm, total);
-    stage_kernel<R><<<grid, block, 0, st>>>(wa, y, wb, (R)(dt / 3), dm, total);
-    stage_kernel<R><<<grid, block, 0, st>>>(wb, y, wa, (R)(dt / 2), dm, total);
-    stage_kernel<R><<<grid, block, 0, st>>>(wa, y, y, (R)dt, dm, total);
-    count_launch(4);
-  }
-  LAUNCH_CHECK();
+  double2 *dy = (double2 *)y, *da = (double2 *)wa, *db = (double2 *)wb;
+  if (h->f64.ready) work_in(h, dy, dy, da, branches, st);
+  rk4_work64(h, dy, da, db, branches, dt, nsteps, st);
+  if (h->f64.ready) work_out(h, dy, dy, da, branches, st);
 }
 
 template <typename R>
 void kick_into(heom_hier *h, const typename CxT<R>::type *in, typename CxT<R>::type *out,
-                      int branches, int which, cudaStream_t st) {
+                      int branches, const R *K, cudaStream_t st) {
   const Model &M = h->M;
   const int64_t total = (int64_t)branches * M.n_ado * M.d * M.d;
-  kick_kernel<R><<<grid_for(total), 256, 0, st>>>(in, out, mu_of<R>(h, which), M.d, total);
+  kick_kernel<R><<<grid_for(total), 256, 0, st>>>(in, out, K, M.d, total);
   count_launch(1);
   LAUNCH_CHECK();
 }
 
 template <typename R>
-void trace_into(heom_hier *h, const typename CxT<R>::type *w, int branches, int order,
-                       double2 *out, int64_t ostride, cudaStream_t st) {
+void trace_into(heom_hier *h, const typename CxT<R>::type *w, int branches, const double *mu, int order,
+                double2 *out, int64_t ostride, cudaStream_t st) {
   const Model &M = h->M;
-  const double *mu = sizeof(R) == 8 ? h->mu_trace : h->mu_vb64;
   trace_kernel<R><<<branches, 256, 0, st>>>(w, mu, M.d, M.n_ado, order, out, ostride);
   count_launch(1);
   LAUNCH_CHECK();
@@ -231,18 +309,26 @@ void trace_into(heom_hier *h, const typename CxT<R>::type *w, int branches, int 
 // Original-basis complex128 ADOs -> coupling-basis complex64 (U^T x U), and back.
 void to_coupling_basis(heom_hier *h, const double2 *x, float2 *out, int64_t elems, cudaStream_t st) {
   DeviceBuffer tmp(elems * 16);
-  sim_left_kernel<double2><<<grid_for(elems), 256, 0, st>>>(x, (double2 *)tmp.p, h->U64, h->M.d, elems);
-  sim_right_kernel<float2><<<grid_for(elems), 256, 0, st>>>((const double2 *)tmp.p, out, h->U64, h->M.d, elems);
-  count_launch(2);
+  if (h->rot.ready) {
+    rotate<double2, float2>(h->rot, true, x, out, (double2 *)tmp.p, elems / ((int64_t)h->M.d * h->M.d), st);
+  } else {
+    sim_left_kernel<double2><<<grid_for(elems), 256, 0, st>>>(x, (double2 *)tmp.p, h->U64, h->M.d, elems);
+    sim_right_kernel<float2><<<grid_for(elems), 256, 0, st>>>((const double2 *)tmp.p, out, h->U64, h->M.d, elems);
+    count_launch(2);
+  }
   LAUNCH_CHECK();
   CUDA_TRY(cudaStreamSynchronize(st));
 }
 
 static void from_coupling_basis(heom_hier *h, const float2 *x, double2 *out, int64_t elems, cudaStream_t st) {
   DeviceBuffer tmp(elems * 16);
-  sim_left_kernel<float2><<<grid_for(elems), 256, 0, st>>>(x, (double2 *)tmp.p, h->UT64, h->M.d, elems);
-  sim_right_kernel<double2><<<grid_for(elems), 256, 0, st>>>((const double2 *)tmp.p, out, h->UT64, h->M.d, elems);
-  count_launch(2);
+  if (h->rot.ready) {
+    rotate<float2, double2>(h->rot, false, x, out, (double2 *)tmp.p, elems / ((int64_t)h->M.d * h->M.d), st);
+  } else {
+    sim_left_kernel<float2><<<grid_for(elems), 256, 0, st>>>(x, (double2 *)tmp.p, h->UT64, h->M.d, elems);
+    sim_right_kernel<double2><<<grid_for(elems), 256, 0, st>>>((const double2 *)tmp.p, out, h->UT64, h->M.d, elems);
+    count_launch(2);
+  }
   LAUNCH_CHECK();
   CUDA_TRY(cudaStreamSynchronize(st));
 }
@@ -282,10 +368,16 @@ void response_2d_rows_impl(heom_hier *h, const heom_state *eq, const heom_grid *
   // single-branch buffers: equilibrium (precision R), trunk and its scratch
   DeviceBuffer eqR(per_branch * cb), T(per_branch * cb), ta(per_branch * cb), tb(per_branch * cb);
   if (sizeof(R) == 8) {
-    CUDA_TRY(cudaMemcpyAsync(eqR.p, eq->buf.p, per_branch * cb, cudaMemcpyDeviceToDevice, st));
+    work_in(h, (const double2 *)eq->buf.p, (double2 *)eqR.p, (double2 *)ta.p, 1, st);
   } else {
     to_coupling_basis(h, (const double2 *)eq->buf.p, (float2 *)eqR.p, per_branch, st);
   }
+  auto steps = [&](C *y, C *a, C *b, int br, int64_t n, int prec) {
+    if constexpr (sizeof(R) == 8)
+      rk4_work64(h, y, a, b, br, dt, n, st);
+    else
+      rk4_steps<R>(h, y, a, b, br, dt, n, st, prec);
+  };
   // branch chunk size: both pathways of jc t1 samples, 3 or 4 state sets
   const int nsets = nt2 > 1 ? 4 : 3;
   size_t free_b = 0, total_b = 0;
@@ -306,13 +398,13 @@ void response_2d_rows_impl(heom_hier *h, const heom_state *eq, const heom_grid *
     // branch is a small share of the scan's work.
     const int trunk_prec = M.precision == HEOM_TC ? HEOM_FP32 : M.precision;
     PhaseRange phase("heom: t1 trunk");
-    kick_into<R>(h, (const C *)eqR.p, (C *)T.p, 1, 2, st);
-    rk4_steps<R>(h, (C *)T.p, (C *)ta.p, (C *)tb.p, 1, dt, (int64_t)(jr0 + j0) * m, st, trunk_prec);
+    kick_into<R>(h, (const C *)eqR.p, (C *)T.p, 1, mu_work<R>(h, 2), st);
+    steps((C *)T.p, (C *)ta.p, (C *)tb.p, 1, (int64_t)(jr0 + j0) * m, trunk_prec);
     for (int j = 0; j < nj; ++j) {
-      if (j > 0) rk4_steps<R>(h, (C *)T.p, (C *)ta.p, (C *)tb.p, 1, dt, m, st, trunk_prec);
+      if (j > 0) steps((C *)T.p, (C *)ta.p, (C *)tb.p, 1, m, trunk_prec);
       kick2_pair_kernel<R><<<grid_for(per_branch), 256, 0, st>>>(
           (const C *)T.p, BR + (int64_t)j * per_branch, BR + (int64_t)(nj + j) * per_branch,
-          mu_of<R>(h, 1), mu_of<R>(h, 2), M.d, per_branch);
+          mu_work<R>(h, 1), mu_work<R>(h, 2), M.d, per_branch);
       count_launch(1);
       LAUNCH_CHECK();
     }
@@ -322,9 +414,9 @@ void response_2d_rows_impl(heom_hier *h, const heom_state *eq, const heom_grid *
       const int it = order[oi];
       C *Y = (C *)P1.p, *WA = (C *)P2.p, *WB = (C *)(nsets == 4 ? P3.p : P0.p);
       phase.next("heom: t2 fork");
-      rk4_steps<R>(h, BR, Y, WA, B, dt, n2[it] - t_now, st, M.precision);
+      steps(BR, Y, WA, B, n2[it] - t_now, M.precision);
       t_now = n2[it];
-      kick_into<R>(h, BR, Y, B, 1, st);
+      kick_into<R>(h, BR, Y, B, mu_work<R>(h, 1), st);
       // the coupling kernel's shape is tuned (once per size) before the capture
       if (sizeof(R) == 4 && M.precision == HEOM_TC)
         tc_tune({TcRk4Set{&h->tc, (float2 *)Y, (float2 *)WA, (float2 *)WB, B}}, dt, st);
@@ -333,10 +425,10 @@ void response_2d_rows_impl(heom_hier *h, const heom_state *eq, const heom_grid *
       phase.next("heom: t3 scan");
       GraphCapture cap(st);
       for (int k = 0; k < n3; ++k) {
-        if (k > 0) rk4_steps<R>(h, Y, WA, WB, B, dt, m, st, M.precision);
+        if (k > 0) steps(Y, WA, WB, B, m, M.precision);
         for (int pw = 0; pw < 2; ++pw) {
           double2 *base = Rdev + (int64_t)it * 2 * n1 * n3 + (int64_t)pw * n1 * n3 + (int64_t)j0 * n3 + k;
-          trace_into<R>(h, Y + (int64_t)pw * nj * per_branch, nj, 3, base, n3, st);
+          trace_into<R>(h, Y + (int64_t)pw * nj * per_branch, nj, mu_trace_work<R>(h), 3, base, n3, st);
         }
       }
       cap.replay();
@@ -347,10 +439,10 @@ void response_2d_rows_impl(heom_hier *h, const heom_state *eq, const heom_grid *
 // Instantiations used by the other translation units (batched.cu, grad.cu, steady.cu).
 template void rk4_steps<double>(heom_hier *, double2 *, double2 *, double2 *, int, double, int64_t, cudaStream_t, int);
 template void rk4_steps<float>(heom_hier *, float2 *, float2 *, float2 *, int, double, int64_t, cudaStream_t, int);
-template void kick_into<double>(heom_hier *, const double2 *, double2 *, int, int, cudaStream_t);
-template void kick_into<float>(heom_hier *, const float2 *, float2 *, int, int, cudaStream_t);
-template void trace_into<double>(heom_hier *, const double2 *, int, int, double2 *, int64_t, cudaStream_t);
-template void trace_into<float>(heom_hier *, const float2 *, int, int, double2 *, int64_t, cudaStream_t);
+template void kick_into<double>(heom_hier *, const double2 *, double2 *, int, const double *, cudaStream_t);
+template void kick_into<float>(heom_hier *, const float2 *, float2 *, int, const float *, cudaStream_t);
+template void trace_into<double>(heom_hier *, const double2 *, int, const double *, int, double2 *, int64_t, cudaStream_t);
+template void trace_into<float>(heom_hier *, const float2 *, int, const double *, int, double2 *, int64_t, cudaStream_t);
 template void response_2d_rows_impl<double>(heom_hier *, const heom_state *, const heom_grid *, int, int, double2 *);
 template void response_2d_rows_impl<float>(heom_hier *, const heom_state *, const heom_grid *, int, int, double2 *);
 
@@ -416,6 +508,8 @@ void ensure_device(heom_hier *h) {
   h->U64 = h->up(M.vb_U);
   h->UT64 = h->up(UT);
   h->mu_vb64 = h->up(M.vb_mu);
+  h->mup_vb64 = h->up(M.vb_mu_plus);
+  h->mum_vb64 = h->up(mumv);
   h->mu_vb32 = h->up(cast_vec<float>(M.vb_mu));
   h->mup_vb32 = h->up(cast_vec<float>(M.vb_mu_plus));
   h->mum_vb32 = h->up(cast_vec<float>(mumv));
@@ -434,6 +528,8 @@ void ensure_device(heom_hier *h) {
   vb.nb_cA = d32.nb_cA;
   vb.nb_cB = d32.nb_cB;
   h->vb = vb;
+  if (rot_supported(M)) h->rot = rot_build(M, h->allocs);
+  if (f64_supported(M)) h->f64 = f64_build(M, M.nb_off, M.nb_idx, M.nb_cA, M.nb_cB, 1.0, h->allocs);
   if (M.precision == HEOM_TC) tc_build(h->tc, M, h->vb, h->allocs);
   // the table uploads above are complete before any launch on any stream
   CUDA_TRY(cudaDeviceSynchronize());
@@ -621,9 +717,9 @@ heom_status heom_kick(heom_hier *h, heom_state *rho, int which) {
     const size_t bytes = rho->elems() * rho->elem_bytes();
     DeviceBuffer tmp(bytes);
     if (rho->precision == HEOM_FP64)
-      kick_into<double>(h, (const double2 *)rho->buf.p, (double2 *)tmp.p, rho->branches, which, h->stream);
+      kick_into<double>(h, (const double2 *)rho->buf.p, (double2 *)tmp.p, rho->branches, mu_of<double>(h, which), h->stream);
     else
-      kick_into<float>(h, (const float2 *)rho->buf.p, (float2 *)tmp.p, rho->branches, which, h->stream);
+      kick_into<float>(h, (const float2 *)rho->buf.p, (float2 *)tmp.p, rho->branches, mu_of<float>(h, which), h->stream);
     CUDA_TRY(cudaMemcpyAsync(rho->buf.p, tmp.p, bytes, cudaMemcpyDeviceToDevice, h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     return HEOM_OK;
@@ -636,9 +732,9 @@ heom_status heom_trace(heom_hier *h, const heom_state *rho, int order, double *o
     ensure_device(h);
     DeviceBuffer o((size_t)rho->branches * 16);
     if (rho->precision == HEOM_FP64)
-      trace_into<double>(h, (const double2 *)rho->buf.p, rho->branches, order, (double2 *)o.p, 1, h->stream);
+      trace_into<double>(h, (const double2 *)rho->buf.p, rho->branches, h->mu_trace, order, (double2 *)o.p, 1, h->stream);
     else
-      trace_into<float>(h, (const float2 *)rho->buf.p, rho->branches, order, (double2 *)o.p, 1, h->stream);
+      trace_into<float>(h, (const float2 *)rho->buf.p, rho->branches, h->mu_vb64, order, (double2 *)o.p, 1, h->stream);
     CUDA_TRY(cudaMemcpyAsync(out, o.p, (size_t)rho->branches * 16, cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     return HEOM_OK;
@@ -669,39 +765,43 @@ heom_status heom_equilibrate(heom_hier *h, double dt_fs, double t_max_fs, double
     DeviceBuffer a(per * 16), b(per * 16);
     const int64_t nmax = (int64_t)std::llround(t_max_fs / dt_fs);
     s->eq_dt = dt_fs;
+    double2 *rho = (double2 *)s->buf.p;
     if (tol <= 0) {
-      rk4_steps<double>(h, (double2 *)s->buf.p, (double2 *)a.p, (double2 *)b.p, 1, dt_fs, nmax, h->stream, HEOM_FP64);
+      rk4_steps<double>(h, rho, (double2 *)a.p, (double2 *)b.p, 1, dt_fs, nmax, h->stream, HEOM_FP64);
       CUDA_TRY(cudaStreamSynchronize(h->stream));
       s->eq_steps = nmax;
       return HEOM_OK;
     }
-    DeviceBuffer norms((size_t)M.n_ado * 8), zero(per * 16);
-    CUDA_TRY(cudaMemsetAsync(zero.p, 0, per * 16, h->stream));
+    DeviceBuffer norms((size_t)M.n_ado * 8);
     std::vector<double> hn(M.n_ado);
     int64_t done = 0;
-    while (done < nmax) {
+    bool converged = false;
+    work_in(h, rho, rho, (double2 *)a.p, 1, h->stream);   // the residual's norms do not depend on the basis
+    while (done < nmax && !converged) {
       int64_t chunk = std::min<int64_t>(100, nmax - done);
-      rk4_steps<double>(h, (double2 *)s->buf.p, (double2 *)a.p, (double2 *)b.p, 1, dt_fs, chunk, h->stream, HEOM_FP64);
+      rk4_work64(h, rho, (double2 *)a.p, (double2 *)b.p, 1, dt_fs, chunk, h->stream);
       done += chunk;
       s->eq_steps = done;
-      // residual: a = 0 + 1 * L(rho)
-      stage_kernel<double><<<grid_for(per), 256, 0, h->stream>>>((const double2 *)s->buf.p, (const double2 *)zero.p,
-                                                                  (double2 *)a.p, 1.0, h->dm64, per);
+      // residual: a = L(rho)
+      rhs_work64(h, rho, (double2 *)a.p, 1, h->stream);
       ado_norms_kernel<double><<<M.n_ado, 256, 0, h->stream>>>((const double2 *)a.p, (int64_t)M.d * M.d, M.n_ado, (double *)norms.p);
-      count_launch(2);
+      count_launch(1);
       LAUNCH_CHECK();
       CUDA_TRY(cudaMemcpyAsync(hn.data(), norms.p, M.n_ado * 8, cudaMemcpyDeviceToHost, h->stream));
       CUDA_TRY(cudaStreamSynchronize(h->stream));
       double res = 0;
       for (double v : hn) res = std::max(res, v);
-      ado_norms_kernel<double><<<1, 256, 0, h->stream>>>((const double2 *)s->buf.p, (int64_t)M.d * M.d, 1, (double *)norms.p);
+      ado_norms_kernel<double><<<1, 256, 0, h->stream>>>(rho, (int64_t)M.d * M.d, 1, (double *)norms.p);
       count_launch(1);
       double n0 = 0;
       CUDA_TRY(cudaMemcpyAsync(&n0, norms.p, 8, cudaMemcpyDeviceToHost, h->stream));
       CUDA_TRY(cudaStreamSynchronize(h->stream));
       if (!std::isfinite(res) || !std::isfinite(n0)) throw Fail{HEOM_ENONFINITE, "equilibrium residual is not finite"};
-      if (std::sqrt(res) <= tol * std::sqrt(n0)) return HEOM_OK;
+      converged = std::sqrt(res) <= tol * std::sqrt(n0);
     }
+    work_out(h, rho, rho, (double2 *)a.p, 1, h->stream);
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    if (converged) return HEOM_OK;
     g_last_error = "equilibrium tolerance not reached by t_max";
     return HEOM_ENOTCONV;
   });
@@ -856,9 +956,9 @@ heom_status heom_kick_dev(heom_hier *h, const void *in, void *out, int branches,
     ensure_device(h);
     cudaStream_t st = (cudaStream_t)stream;
     if (precision == HEOM_FP64)
-      kick_into<double>(h, (const double2 *)in, (double2 *)out, branches, which, st);
+      kick_into<double>(h, (const double2 *)in, (double2 *)out, branches, mu_of<double>(h, which), st);
     else
-      kick_into<float>(h, (const float2 *)in, (float2 *)out, branches, which, st);
+      kick_into<float>(h, (const float2 *)in, (float2 *)out, branches, mu_of<float>(h, which), st);
     return HEOM_OK;
   });
 }
@@ -870,9 +970,9 @@ heom_status heom_trace_dev(heom_hier *h, const void *state, int branches, int pr
     ensure_device(h);
     cudaStream_t st = (cudaStream_t)stream;
     if (precision == HEOM_FP64)
-      trace_into<double>(h, (const double2 *)state, branches, order, (double2 *)out, 1, st);
+      trace_into<double>(h, (const double2 *)state, branches, h->mu_trace, order, (double2 *)out, 1, st);
     else
-      trace_into<float>(h, (const float2 *)state, branches, order, (double2 *)out, 1, st);
+      trace_into<float>(h, (const float2 *)state, branches, h->mu_vb64, order, (double2 *)out, 1, st);
     return HEOM_OK;
   });
 }
@@ -888,10 +988,11 @@ heom_status heom_response_1d(heom_hier *h, const heom_state *rho_eq, double dt_f
     const Model &M = h->M;
     const int64_t per = (int64_t)M.n_ado * M.d * M.d;
     DeviceBuffer y(per * 16), a(per * 16), b(per * 16), Rd((size_t)n * 16);
-    kick_into<double>(h, (const double2 *)rho_eq->buf.p, (double2 *)y.p, 1, 0, h->stream);
+    work_in(h, (const double2 *)rho_eq->buf.p, (double2 *)a.p, (double2 *)b.p, 1, h->stream);
+    kick_into<double>(h, (const double2 *)a.p, (double2 *)y.p, 1, mu_work<double>(h, 0), h->stream);
     for (int k = 0; k < n; ++k) {
-      if (k > 0) rk4_steps<double>(h, (double2 *)y.p, (double2 *)a.p, (double2 *)b.p, 1, dt_fs, m, h->stream, HEOM_FP64);
-      trace_into<double>(h, (const double2 *)y.p, 1, 1, (double2 *)Rd.p + k, 1, h->stream);
+      if (k > 0) rk4_work64(h, (double2 *)y.p, (double2 *)a.p, (double2 *)b.p, 1, dt_fs, m, h->stream);
+      trace_into<double>(h, (const double2 *)y.p, 1, mu_trace_work<double>(h), 1, (double2 *)Rd.p + k, 1, h->stream);
     }
     CUDA_TRY(cudaMemcpyAsync(R1, Rd.p, (size_t)n * 16, cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));

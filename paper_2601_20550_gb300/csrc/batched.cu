@@ -19,77 +19,48 @@ using namespace heom;
 namespace heom {
 
 // Several FP64 parameter sets (hierarchies of any basis size) on one grid, with
-// every RK4 stage of all sets in one launch of multi_stage_kernel.  The branch
-// schedule is that of response_2d_rows_impl (one t1 trunk per set, both
-// pathways from it, t2 forks in ascending order, the t3 scan captured once into
-// a CUDA graph); kicks and traces stay per set (they are cheap).  Rdev[k] gets
-// set k's R in the layout [n_t2][2][n1][n3].
+// every RK4 stage of all sets together (f64_stage_plan: one launch, or launch pair, per
+// kernel variant the sets need).  The branch schedule is that of
+// response_2d_rows_impl (one t1 trunk per set, both pathways from it, t2 forks in
+// ascending order, the t3 scan captured once into a CUDA graph); kicks and traces stay
+// per set (they are cheap).  Rdev[k] gets set k's R in the layout [n_t2][2][n1][n3].
 struct MultiSet {
   heom_hier *h;
   const heom_state *eq;
-  int64_t per;                                     // n_ado d^2
-  std::unique_ptr<DeviceBuffer> T, ta, tb, P[4];   // trunk and its scratch; branch sets
+  int64_t per;                                          // n_ado d^2
+  std::unique_ptr<DeviceBuffer> eqW, T, ta, tb, P[4];   // equilibrium, trunk and its scratch; branch sets
 };
 
-// Descriptor arrays (device) for the four Horner stages of one RK4 step on the
-// buffers (y, wa, wb) of every set.
+// Plans of the four Horner stages of one RK4 step on the buffers (y, wa, wb) of every set.
 struct MultiStep {
-  DeviceBuffer desc[4];
-  int64_t grand = 0;
+  F64Plan stage[4];
 };
 
 static void multi_step_setup(std::vector<MultiSet> &S, MultiStep &ms, int which_y, int which_a, int which_b,
                              int branches, cudaStream_t st) {
-  const int n = (int)S.size();
-  std::vector<SetStage<double>> d4[4];
-  int64_t begin = 0;
-  for (int k = 0; k < n; ++k) {
+  std::vector<F64Buf> b[4];
+  for (MultiSet &s : S) {
     auto buf = [&](int w) -> double2 * {
-      if (w == -1) return (double2 *)S[k].T->p;
-      if (w == -2) return (double2 *)S[k].ta->p;
-      if (w == -3) return (double2 *)S[k].tb->p;
-      return (double2 *)S[k].P[w]->p;
+      if (w == -1) return (double2 *)s.T->p;
+      if (w == -2) return (double2 *)s.ta->p;
+      if (w == -3) return (double2 *)s.tb->p;
+      return (double2 *)s.P[w]->p;
     };
     double2 *y = buf(which_y), *wa = buf(which_a), *wb = buf(which_b);
-    const int64_t tot = (int64_t)branches * S[k].per;
-    const double2 *ws[4] = {y, wa, wb, wa};
-    double2 *outs[4] = {wa, wb, wa, y};
-    for (int q = 0; q < 4; ++q) {
-      SetStage<double> x{};
-      x.M = S[k].h->dm64;
-      x.w = ws[q];
-      x.y = y;
-      x.out = outs[q];
-      x.begin = begin;
-      x.total = tot;
-      d4[q].push_back(x);
-    }
-    begin += tot;
+    b[0].push_back({&s.h->f64, y, y, wa, wa, branches});
+    b[1].push_back({&s.h->f64, wa, y, wb, wb, branches});
+    b[2].push_back({&s.h->f64, wb, y, wa, wa, branches});
+    b[3].push_back({&s.h->f64, wa, y, y, wb, branches});
   }
-  ms.grand = begin;
-  for (int q = 0; q < 4; ++q) {
-    ms.desc[q].alloc(sizeof(SetStage<double>) * n);
-    CUDA_TRY(cudaMemcpyAsync(ms.desc[q].p, d4[q].data(), sizeof(SetStage<double>) * n, cudaMemcpyHostToDevice, st));
-  }
-  CUDA_TRY(cudaStreamSynchronize(st));
+  for (int q = 0; q < 4; ++q) f64_plan(ms.stage[q], b[q], st);
 }
 
-static void multi_rk4(const MultiStep &ms, int n_sets, double dt, int64_t nsteps, cudaStream_t st) {
-  if (ms.grand == 0 || nsteps <= 0) return;
+static void multi_rk4(const MultiStep &ms, double dt, int64_t nsteps, cudaStream_t st) {
   const double al[4] = {dt / 4, dt / 3, dt / 2, dt};
-  const int grid = grid_for(ms.grand);
-  for (int64_t s = 0; s < nsteps; ++s) {
-    for (int q = 0; q < 4; ++q)
-      multi_stage_kernel<double><<<grid, 256, 0, st>>>((const SetStage<double> *)ms.desc[q].p, n_sets, al[q],
-                                                       ms.grand);
-    count_launch(4);
-  }
+  for (int64_t s = 0; s < nsteps; ++s)
+    for (int q = 0; q < 4; ++q) f64_stage_plan(ms.stage[q], al[q], st);
   LAUNCH_CHECK();
 }
-
-}  // namespace heom
-
-namespace heom {
 
 static void response_2d_multi(heom_hier *const *hs, const heom_state *const *eqs, int n_sets, const heom_grid *g,
                               const std::vector<double2 *> &Rdev) {
@@ -116,6 +87,8 @@ static void response_2d_multi(heom_hier *const *hs, const heom_state *const *eqs
     S[k].T.reset(new DeviceBuffer(S[k].per * 16));
     S[k].ta.reset(new DeviceBuffer(S[k].per * 16));
     S[k].tb.reset(new DeviceBuffer(S[k].per * 16));
+    S[k].eqW.reset(new DeviceBuffer(S[k].per * 16));
+    work_in(hs[k], (const double2 *)eqs[k]->buf.p, (double2 *)S[k].eqW->p, (double2 *)S[k].ta->p, 1, st);
   }
   // t1 rows per chunk: both pathways of J rows, 3 or 4 branch sets per parameter set
   const int nbuf = nt2 > 1 ? 4 : 3;
@@ -137,16 +110,16 @@ static void response_2d_multi(heom_hier *const *hs, const heom_state *const *eqs
     multi_step_setup(S, scan, 1, 2, nbuf == 4 ? 3 : 0, B, st);       // y = Y, scratch WA, WB
     PhaseRange phase("heom: t1 trunk (sets)");
     for (int k = 0; k < n_sets; ++k)
-      kick_into<double>(S[k].h, (const double2 *)S[k].eq->buf.p, (double2 *)S[k].T->p, 1, 2, st);
-    multi_rk4(trunk, n_sets, dt, (int64_t)j0 * m, st);
+      kick_into<double>(S[k].h, (const double2 *)S[k].eqW->p, (double2 *)S[k].T->p, 1, mu_work<double>(S[k].h, 2), st);
+    multi_rk4(trunk, dt, (int64_t)j0 * m, st);
     for (int j = 0; j < nj; ++j) {
-      if (j > 0) multi_rk4(trunk, n_sets, dt, m, st);
+      if (j > 0) multi_rk4(trunk, dt, m, st);
       for (int k = 0; k < n_sets; ++k) {
         const int64_t per = S[k].per;
         double2 *br = (double2 *)S[k].P[0]->p;
         kick2_pair_kernel<double><<<grid_for(per), 256, 0, st>>>((const double2 *)S[k].T->p, br + (int64_t)j * per,
-                                                                br + (int64_t)(nj + j) * per, S[k].h->mup64,
-                                                                S[k].h->mum64, S[k].h->M.d, per);
+                                                                br + (int64_t)(nj + j) * per, mu_work<double>(S[k].h, 1),
+                                                                mu_work<double>(S[k].h, 2), S[k].h->M.d, per);
         count_launch(1);
         LAUNCH_CHECK();
       }
@@ -155,18 +128,18 @@ static void response_2d_multi(heom_hier *const *hs, const heom_state *const *eqs
     for (int oi = 0; oi < nt2; ++oi) {
       const int it = order[oi];
       phase.next("heom: t2 fork (sets)");
-      multi_rk4(fork, n_sets, dt, n2[it] - t_now, st);
+      multi_rk4(fork, dt, n2[it] - t_now, st);
       t_now = n2[it];
       for (int k = 0; k < n_sets; ++k)
-        kick_into<double>(S[k].h, (const double2 *)S[k].P[0]->p, (double2 *)S[k].P[1]->p, B, 1, st);
+        kick_into<double>(S[k].h, (const double2 *)S[k].P[0]->p, (double2 *)S[k].P[1]->p, B, mu_work<double>(S[k].h, 1), st);
       phase.next("heom: t3 scan (sets)");
       GraphCapture cap(st);
       for (int kk = 0; kk < n3; ++kk) {
-        if (kk > 0) multi_rk4(scan, n_sets, dt, m, st);
+        if (kk > 0) multi_rk4(scan, dt, m, st);
         for (int k = 0; k < n_sets; ++k)
           for (int pw = 0; pw < 2; ++pw) {
             double2 *base = Rdev[k] + (int64_t)it * 2 * n1 * n3 + (int64_t)pw * n1 * n3 + (int64_t)j0 * n3 + kk;
-            trace_into<double>(S[k].h, (const double2 *)S[k].P[1]->p + (int64_t)pw * nj * S[k].per, nj, 3, base, n3, st);
+            trace_into<double>(S[k].h, (const double2 *)S[k].P[1]->p + (int64_t)pw * nj * S[k].per, nj, mu_trace_work<double>(S[k].h), 3, base, n3, st);
           }
       }
       cap.replay();
@@ -237,7 +210,7 @@ static void response_2d_multi_tc(heom_hier *const *hs, const heom_state *const *
       heom_hier *h = hs[k];
       const int64_t per = S[k].per;
       float2 *T = (float2 *)S[k].T->p;
-      kick_into<float>(h, (const float2 *)S[k].eqR->p, T, 1, 2, st);
+      kick_into<float>(h, (const float2 *)S[k].eqR->p, T, 1, mu_of<float>(h, 2), st);
       rk4_steps<float>(h, T, (float2 *)S[k].ta->p, (float2 *)S[k].tb->p, 1, dt, (int64_t)j0 * m, st, HEOM_FP32);
       float2 *br = (float2 *)S[k].P[0]->p;
       for (int j = 0; j < nj; ++j) {
@@ -255,7 +228,7 @@ static void response_2d_multi_tc(heom_hier *const *hs, const heom_state *const *
       tc_rk4_sets(fork, dt, n2[it] - t_now, st);
       t_now = n2[it];
       for (int k = 0; k < n_sets; ++k)
-        kick_into<float>(hs[k], (const float2 *)S[k].P[0]->p, (float2 *)S[k].P[1]->p, B, 1, st);
+        kick_into<float>(hs[k], (const float2 *)S[k].P[0]->p, (float2 *)S[k].P[1]->p, B, mu_of<float>(hs[k], 1), st);
       tc_tune(scan, dt, st);   // coupling-kernel shape, once per size, before the capture
       phase.next("heom: t3 scan (tensor-core sets)");
       GraphCapture cap(st);
@@ -264,7 +237,7 @@ static void response_2d_multi_tc(heom_hier *const *hs, const heom_state *const *
         for (int k = 0; k < n_sets; ++k)
           for (int pw = 0; pw < 2; ++pw) {
             double2 *base = Rdev[k] + (int64_t)it * 2 * n1 * n3 + (int64_t)pw * n1 * n3 + (int64_t)j0 * n3 + kk;
-            trace_into<float>(hs[k], (const float2 *)S[k].P[1]->p + (int64_t)pw * nj * S[k].per, nj, 3, base, n3, st);
+            trace_into<float>(hs[k], (const float2 *)S[k].P[1]->p + (int64_t)pw * nj * S[k].per, nj, hs[k]->mu_vb64, 3, base, n3, st);
           }
       }
       cap.replay();
@@ -286,7 +259,7 @@ heom_status heom_response_2d_batched(heom_hier *const *hs, const heom_state *con
   for (int i = 0; i < n_sets; ++i) {
     heom_status a = check_response_args(hs[i], eqs[i], g);
     if (a != HEOM_OK) return a;
-    all64 = all64 && hs[i]->M.precision == HEOM_FP64;
+    all64 = all64 && hs[i]->M.precision == HEOM_FP64 && f64_supported(hs[i]->M);
     alltc = alltc && hs[i]->M.precision == HEOM_TC;
     // a tensor-core hierarchy keeps per-item scale workspace for one set at a
     // time: a batch that names one twice runs set by set

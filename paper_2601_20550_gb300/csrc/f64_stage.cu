@@ -1,0 +1,973 @@
+// FP64 stage out = y + alpha L(w) in the coupling eigenbasis (declared in f64_stage.h).
+//
+// What bounds it.  GB300 issues 2 FP64 operations per clock and SM, 1/64 of its FP32
+// rate.  The commutator's 2 x 2 x d multiply-adds per element were nine tenths of the
+// stage on that pipe.  Here they run as exact integer products on the IMAD pipe (32
+// IMAD.WIDE per clock and SM): w (per item, or per column and row) and H' are scaled by
+// powers of two to 57 bits and cut into two signed limbs, 31 bits above 26, and
+//   sum_c h z = 2^52 sum h1 z1 + 2^26 sum (h1 z0 + h0 z1)   (+ h0 z0, dropped: below
+//   2^-60 of the largest value of the sum)
+// is accumulated without rounding in two 64-bit integers, three IMAD.WIDE per product;
+// only H''s structural non-zeros are multiplied (37 of 64 columns at four levels, 61 of
+// 125 at five).  The sums are rounded once when they turn back into FP64.  The
+// elementwise rest takes ~38 FP64 operations per element and stage and shares the SM
+// with the integer phase of other resident blocks.
+#include "f64_stage.h"
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <map>
+#include <stdexcept>
+#include <type_traits>
+
+#include "tc_stage.h"   // device_malloc, DeviceOom
+
+namespace heom {
+
+void count_launch(uint64_t n);
+
+namespace {
+
+constexpr int kPanel = 32;                 // columns (rows) of w per panel block: one per lane
+constexpr int kPanelThreads = 384;
+constexpr int kF64MaxExp = 16;             // build_hierarchy's limit
+constexpr int kRotPad = 33;
+constexpr size_t kMaxSmem = 227 * 1024;
+// Whole-item blocks up to two per SM; above, one panel of 32 columns (rows) per block.
+constexpr size_t kFusedSmem = 112 * 1024;
+
+struct F64Set {
+  F64Ops O;
+  const double2 *w, *y;
+  double2 *out, *tp;
+  int64_t begin;      // first block of the set
+  int64_t items;
+  int per_block;      // fused: items per block; panels: panels per item
+  int smem_t;         // fused: commutator part kept in shared memory
+};
+
+struct F64Args {
+  F64Set one;
+  const F64Set *many;
+  int n;
+  double alpha;
+};
+
+template <bool kMulti>
+__device__ __forceinline__ const F64Set &pick(const F64Args &P) {
+  if (!kMulti) return P.one;
+  int k = 0;
+  while (k + 1 < P.n && (int64_t)blockIdx.x >= P.many[k + 1].begin) ++k;
+  return P.many[k];
+}
+
+__device__ __forceinline__ int exp_field(double2 v) {
+  return max((__double2hiint(v.x) >> 20) & 0x7ff, (__double2hiint(v.y) >> 20) & 0x7ff);
+}
+
+// x (exponent field at most emax) as round(x 2^(1021 + bits - emax)), magnitude at most
+// 2^(bits - 1), in two signed limbs hi 2^low + lo.  Integer operations only: a conversion
+// instruction would take the FP64 pipe.
+__device__ __forceinline__ int2 to_limbs(double x, int emax, int bits, int low) {
+  const long long b = __double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ff);
+  const long long m = ((b & 0xfffffffffffffLL) | (e > 0 ? 1LL << 52 : 0LL)) << (bits - 54);
+  const int sh = min(emax - max(e, 1), 62);
+  long long v = (m + ((1LL << sh) >> 1)) >> sh;
+  v = b < 0 ? -v : v;
+  int2 r;
+  r.y = ((int)((unsigned)v << (32 - low))) >> (32 - low);
+  r.x = (int)((v - r.y) >> low);
+  return r;
+}
+
+// Factor alpha 2^k of a finished sum, k the exponent of its unit (see to_limbs, f64_build
+// and finish), formed by adding to alpha's exponent field.  Below the normal range the
+// sum takes 2^-64 of it (deep); NaN for a column that holds an infinity or a NaN.
+struct Unit {
+  double f;
+  bool deep;
+};
+
+__device__ __forceinline__ Unit unit(int emax, int hexp, double alpha) {
+  if (emax >= 0x7ff) return {__longlong_as_double(0x7ff8000000000000LL), false};
+  const long long a = __double_as_longlong(alpha);
+  const int k = emax + hexp - 1083, e = (int)((a >> 52) & 0x7ff) + k;
+  if ((a << 1) == 0) return {0.0, false};
+  if (e >= 0x7ff) return {alpha * __longlong_as_double(0x7ff0000000000000LL), false};
+  if (e > 0) return {__longlong_as_double(a + ((long long)k << 52)), false};
+  return {e > -64 ? __longlong_as_double(a + ((long long)(k + 64) << 52)) : 0.0, true};
+}
+
+__device__ __forceinline__ double sum_value(long long t, const Unit &u) {
+  const double v = __ll2double_rn(t);
+  return u.deep ? v * 5.421010862427522e-20 : v;   // 2^-64
+}
+
+template <int R>
+struct Acc {
+  long long h[R], x[R];
+};
+
+// Rows g R .. g R + R - 1 of H' times one real column of w (the real or imaginary parts
+// of a complex one) at zl, elements stride apart.  One component per lane: ten 64-bit
+// sums of five rows leave room for 1152 threads per SM.
+template <int R>
+__device__ __forceinline__ void group_product(const F64Ops &O, int g, const int2 *zl, int stride, Acc<R> &A) {
+  constexpr int RP = (R + 1) / 2;
+#pragma unroll
+  for (int r = 0; r < R; ++r) A.h[r] = A.x[r] = 0;
+  auto mac = [&](int r, int hx, int hy, const int2 &z) {
+    A.h[r] += (long long)hx * z.x;
+    A.x[r] += (long long)hx * z.y;
+    A.x[r] += (long long)hy * z.x;
+  };
+  const int f1 = O.foff[g + 1];
+  const int4 *fh = O.fh;
+#pragma unroll 2
+  for (int q = O.foff[g]; q < f1; ++q) {
+    int4 h[RP];
+#pragma unroll
+    for (int p = 0; p < RP; ++p) h[p] = fh[q * RP + p];
+    const int2 z = zl[(R % 2 ? h[RP - 1].z : O.fc[q]) * stride];
+#pragma unroll
+    for (int p = 0; p < RP; ++p) {
+      mac(2 * p, h[p].x, h[p].y, z);
+      if (2 * p + 1 < R) mac(2 * p + 1, h[p].z, h[p].w, z);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int s1 = O.soff[g * R + r + 1];
+#pragma unroll 2
+    for (int q = O.soff[g * R + r]; q < s1; ++q) {
+      const int4 h = O.sh[q];
+      mac(r, h.x, h.y, zl[h.z * stride]);
+    }
+  }
+}
+
+// A sum as a 62-bit integer, units of 2^(2 low - 1).
+template <int R>
+__device__ __forceinline__ long long finish(const Acc<R> &A, int r, int low) {
+  return (A.h[r] << 1) + ((A.x[r] + (1LL << (low - 2))) >> (low - 1));
+}
+
+// An ADO's coupling list in shared memory.
+struct List {
+  F64Entry e[2 * kF64MaxExp];
+  int off[kF64MaxModes + 1];
+};
+
+__device__ __forceinline__ void fill_list(const F64Ops &O, int n, List *L, int t, int nt) {
+  const int *off = O.noff + n * O.n_modes;
+  const int q0 = off[0], nq = off[O.n_modes] - q0;
+  for (int i = t; i <= O.n_modes; i += nt) L->off[i] = off[i] - q0;
+  for (int i = t; i < nq; i += nt) L->e[i] = O.nb[q0 + i];
+}
+
+// (alpha (lam_a - lam_b), alpha (lam_a + lam_b)) of every digit pair, mode after mode.
+__device__ __forceinline__ void fill_tab(const F64Ops &O, double alpha, double2 *tab) {
+  for (int i = threadIdx.x; i < O.tab; i += blockDim.x) {
+    const double2 t = O.fg[i];
+    tab[i] = make_double2(alpha * t.x, alpha * t.y);
+  }
+}
+
+// Elementwise rest of element (a, b) (offset el) of the ADO at wn on top of acc:
+//   acc - alpha gamma w + sum_s [ -i f_s A_s + g_s B_s ],  A_s = sum cA w_m, B_s = sum cB w_m,
+// the neighbours' loads issued four at a time.
+__device__ __forceinline__ double2 couple(const F64Ops &O, const double2 *tab, const List &L, const double2 *wb,
+                                          const double2 *wn, int64_t dd, int a, int b, int el, double2 acc,
+                                          double adec) {
+  const double2 w = wn[el];
+  acc.x = fma(-adec, w.x, acc.x);
+  acc.y = fma(-adec, w.y, acc.y);
+  for (int s = 0; s < O.n_modes; ++s) {
+    const int q0 = L.off[s], q1 = L.off[s + 1];
+    if (q0 == q1) continue;
+    double2 A = make_double2(0.0, 0.0), B = A;
+    bool both = false;
+    for (int q = q0; q < q1; q += 4) {
+      double2 x[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (q + j < q1) x[j] = wb[(int64_t)L.e[q + j].idx * dd + el];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (q + j < q1) {
+          const F64Entry &en = L.e[q + j];
+          const bool first = q + j == q0;
+          if (en.kind == 0) {
+            A = first ? x[j] : make_double2(A.x + x[j].x, A.y + x[j].y);
+          } else {
+            const double c = en.cA;
+            A = first ? make_double2(c * x[j].x, c * x[j].y) : make_double2(fma(c, x[j].x, A.x), fma(c, x[j].y, A.y));
+            if (en.kind == 2) {
+              const double e = en.cB;
+              B = both ? make_double2(fma(e, x[j].x, B.x), fma(e, x[j].y, B.y)) : make_double2(e * x[j].x, e * x[j].y);
+              both = true;
+            }
+          }
+        }
+    }
+    const double2 fg = tab[O.tab_off[s] + O.dig[s * O.d + a] * O.dims[s] + O.dig[s * O.d + b]];
+    acc.x = fma(fg.x, A.y, acc.x);
+    acc.y = fma(-fg.x, A.x, acc.y);
+    if (both) {
+      acc.x = fma(fg.y, B.x, acc.x);
+      acc.y = fma(fg.y, B.y, acc.y);
+    }
+  }
+  return acc;
+}
+
+// ---------------------------------------------------------------------------
+// Whole items per block: w's limbs (scaled per item) in shared memory with an odd row
+// stride, so that a warp reads 32 columns of a row or 32 rows of a column without bank
+// conflicts.  H' w with lanes along the columns, w H' (H' symmetric) with lanes along
+// the rows, then the elementwise rest.
+// ---------------------------------------------------------------------------
+template <int R, bool kMulti>
+__global__ void __launch_bounds__(256, 4) f64_item_kernel(const __grid_constant__ F64Args P) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const F64Set &S = pick<kMulti>(P);
+  const F64Ops &O = S.O;
+  const int d = O.d, ld = d | 1, m = S.per_block, dd = d * d, isz = d * ld;
+  const int64_t i0 = ((int64_t)blockIdx.x - S.begin) * m;
+  const int nm = (int)min((int64_t)m, S.items - i0);
+  double2 *tab = reinterpret_cast<double2 *>(smem);
+  int4 *zs = reinterpret_cast<int4 *>(tab + O.tab);
+  double2 *ts = reinterpret_cast<double2 *>(zs + m * isz);
+  List *lists = reinterpret_cast<List *>(ts + (S.smem_t ? m * isz : 0));
+  int *iexp = reinterpret_cast<int *>(lists + m);
+  const double alpha = P.alpha, ah = alpha * O.hsign;
+  for (int i = threadIdx.x; i < m; i += blockDim.x) iexp[i] = 1;
+  fill_tab(O, alpha, tab);
+  __syncthreads();
+  const double2 *w = S.w + i0 * dd;
+  {
+    int cur = -1, e = 0;
+    for (int k = threadIdx.x; k < nm * dd; k += blockDim.x) {
+      const int i = k / dd, el = k - i * dd, a = el / d;
+      const double2 v = w[k];
+      if (i != cur) {
+        if (cur >= 0) atomicMax(iexp + cur, e);
+        cur = i;
+        e = 0;
+      }
+      e = max(e, exp_field(v));
+      reinterpret_cast<double2 *>(zs)[i * isz + a * ld + el - a * d] = v;
+    }
+    if (cur >= 0) atomicMax(iexp + cur, e);
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < nm * dd; k += blockDim.x) {
+    const int i = k / dd, el = k - i * dd, a = el / d;
+    int4 *p = zs + i * isz + a * ld + el - a * d;
+    const double2 v = *reinterpret_cast<double2 *>(p);
+    const int2 re = to_limbs(v.x, iexp[i], O.bits, O.bits - 31), im = to_limbs(v.y, iexp[i], O.bits, O.bits - 31);
+    *p = make_int4(re.x, re.y, im.x, im.y);
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  for (int i = warp; i < nm; i += warps) fill_list(O, (int)((i0 + i) % O.n_ado), lists + i, lane, 32);
+  const int cols = 2 * nm * d, chunks = (cols + 31) / 32, tasks = O.groups * chunks;
+  // phase 0: t = H' w (lane = column); phase 1: t -= w H' (lane = row); still integers
+  for (int ph = 0; ph < 2; ++ph) {
+    for (int k = warp; k < tasks; k += warps) {
+      const int ch = k / O.groups, g = k - ch * O.groups;
+      const int q = min(ch * 32 + lane, cols - 1), col = q >> 1, comp = q & 1;
+      const int i = col / d, l = col - i * d;
+      Acc<R> A;
+      group_product<R>(O, g, reinterpret_cast<const int2 *>(zs + i * isz + (ph == 0 ? l : l * ld)) + comp,
+                       ph == 0 ? 2 * ld : 2, A);
+      if (ch * 32 + lane < cols) {
+        long long *t = reinterpret_cast<long long *>(S.smem_t ? ts + i * isz : S.tp + (i0 + i) * dd) + comp;
+        const int tld = S.smem_t ? ld : d;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int x = g * R + r;
+          if (x < d) {
+            const long long v = finish(A, r, O.bits - 31);
+            if (ph == 0)
+              t[2 * (x * tld + l)] = v;
+            else
+              t[2 * (l * tld + x)] -= v;
+          }
+        }
+      }
+    }
+    __syncthreads();
+  }
+  for (int k = threadIdx.x; k < nm * dd; k += blockDim.x) {
+    const int i = k / dd, el = k - i * dd, a = el / d, b = el - a * d;
+    const int64_t item = i0 + i;
+    const int n = (int)(item % O.n_ado);
+    const longlong2 c = *reinterpret_cast<const longlong2 *>(S.smem_t ? ts + i * isz + a * ld + b : S.tp + item * dd + el);
+    const Unit f = unit(iexp[i], O.hexp, ah);
+    const double2 y = S.y ? S.y[item * dd + el] : make_double2(0.0, 0.0);
+    const double2 t = make_double2(fma(f.f, sum_value(c.y, f), y.x), fma(-f.f, sum_value(c.x, f), y.y));
+    const double2 *wb = S.w + (item - n) * dd;
+    S.out[item * dd + el] = couple(O, tab, lists[i], wb, wb + n * dd, dd, a, b, el, t, alpha * O.decay[n]);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// One panel per block, for bases whose items do not fit: 32 columns of w in the left
+// kernel (tp = -i alpha H' w), 32 rows in the right one (tp += i alpha w H', then the
+// elementwise rest of those rows).  Limbs scaled per column (row).
+// ---------------------------------------------------------------------------
+template <int R, bool kRight, bool kMulti>
+__global__ void __launch_bounds__(kPanelThreads, 3) f64_panel_kernel(const __grid_constant__ F64Args P) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const F64Set &S = pick<kMulti>(P);
+  const F64Ops &O = S.O;
+  const int d = O.d;
+  const int64_t dd = (int64_t)d * d;
+  const int64_t lb = (int64_t)blockIdx.x - S.begin;
+  const int64_t item = lb / S.per_block;
+  const int p0 = (int)(lb - item * S.per_block) * kPanel, np = min(kPanel, d - p0);
+  constexpr int ld = kRight ? kPanel + 1 : kPanel;
+  double2 *tab = reinterpret_cast<double2 *>(smem);
+  int4 *zs = reinterpret_cast<int4 *>(tab + O.tab);      // [d][ld]
+  __shared__ int lexp[kPanel];
+  __shared__ List list;
+  const double alpha = P.alpha, ah = alpha * O.hsign;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  if (threadIdx.x < kPanel) lexp[threadIdx.x] = 1;
+  const int n = (int)(item % O.n_ado);
+  if (kRight) {
+    fill_tab(O, alpha, tab);
+    fill_list(O, n, &list, threadIdx.x, blockDim.x);
+  }
+  __syncthreads();
+  const double2 *w = S.w + item * dd;
+  const double2 zero = make_double2(0.0, 0.0);
+  if (!kRight) {
+    int e = 0;
+    for (int c = warp; c < d; c += warps) {
+      const double2 v = lane < np ? w[(int64_t)c * d + p0 + lane] : zero;
+      e = max(e, exp_field(v));
+      reinterpret_cast<double2 *>(zs)[c * ld + lane] = v;
+    }
+    atomicMax(lexp + lane, e);
+  } else {
+    for (int a = warp; a < kPanel; a += warps) {
+      int e = 0;
+      for (int c = lane; c < d; c += 32) {
+        const double2 v = a < np ? w[(int64_t)(p0 + a) * d + c] : zero;
+        e = max(e, exp_field(v));
+        reinterpret_cast<double2 *>(zs)[c * ld + a] = v;
+      }
+      e = __reduce_max_sync(0xffffffffu, e);
+      if (lane == 0) lexp[a] = max(e, 1);
+    }
+  }
+  __syncthreads();
+  const int emax = lexp[lane];
+  for (int c = warp; c < d; c += warps) {
+    int4 *p = zs + c * ld + lane;
+    const double2 v = *reinterpret_cast<double2 *>(p);
+    const int2 re = to_limbs(v.x, emax, O.bits, O.bits - 31), im = to_limbs(v.y, emax, O.bits, O.bits - 31);
+    *p = make_int4(re.x, re.y, im.x, im.y);
+  }
+  __syncthreads();
+  // one task: a row group and 16 complex columns, lane = (column, component)
+  const int comp = lane & 1;
+  for (int k = warp; k < 2 * O.groups; k += warps) {
+    const int g = k >> 1, col = (k & 1) * 16 + (lane >> 1);
+    Acc<R> A;
+    group_product<R>(O, g, reinterpret_cast<const int2 *>(zs + col) + comp, 2 * ld, A);
+    if (col < np) {
+      // -i alpha (x + i y) = alpha (y - i x): the real sum goes to the imaginary part
+      const Unit f = unit(lexp[col], O.hexp, comp == (kRight ? 1 : 0) ? -ah : ah);
+      double *t = reinterpret_cast<double *>(S.tp + item * dd) + (comp ^ 1);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int x = g * R + r;
+        if (x < d) {
+          const double v = sum_value(finish(A, r, O.bits - 31), f);
+          if (!kRight) {
+            t[2 * ((int64_t)x * d + p0 + col)] = f.f * v;
+          } else {
+            double *o = t + 2 * ((int64_t)(p0 + col) * d + x);
+            *o = fma(f.f, v, *o);
+          }
+        }
+      }
+    }
+  }
+  if (kRight) {
+    __syncthreads();
+    const double2 *t = S.tp + item * dd;
+    const double2 *wb = S.w + (item - n) * dd;
+    const double2 *y = S.y ? S.y + item * dd : nullptr;
+    const double adec = alpha * O.decay[n];
+    for (int k = threadIdx.x; k < np * d; k += blockDim.x) {
+      const int ar = k / d, el = p0 * d + k;
+      double2 acc = t[el];
+      if (y) {
+        const double2 yv = y[el];
+        acc = make_double2(acc.x + yv.x, acc.y + yv.y);
+      }
+      S.out[item * dd + el] = couple(O, tab, list, wb, wb + n * dd, dd, p0 + ar, k - ar * d, el, acc, adec);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Basis change along one index of every ADO, mode by mode, a panel of 32 columns
+// (left: the row index) or rows (right) in shared memory; each thread transforms one
+// fibre of n_s values in registers: 6 n_s products per element and side instead of the
+// 2 d of a dense product.  In fixed point, 59 bits below the column's 2-norm (which the
+// orthogonal factors keep, so nothing overflows) with 59-bit coefficients in 30-bit
+// limbs: a state goes in and out of this basis in every call, and the roundings of the
+// same products in FP64 (3.6e-16 of the norm for a round trip at four levels) would
+// exceed a step's own; here the results' conversion to FP64 is what remains.
+// ---------------------------------------------------------------------------
+constexpr int kRotMaxN = 8;
+
+__device__ __forceinline__ long long to_fixed59(double x, int emax) {
+  const int2 l = to_limbs(x, emax, 60, 30);
+  return ((long long)l.x << 30) + l.y;
+}
+
+// t 2^(e - 1081), in two factors where one would leave the exponent range; NaN if not finite.
+template <typename T>
+__device__ __forceinline__ T from_fixed59(const longlong2 &t, int e, bool finite) {
+  const double f = __longlong_as_double(finite ? (long long)(e > 58 ? e - 58 : e + 964) << 52 : 0x7ff8000000000000LL);
+  double re = __ll2double_rn(t.x) * f, im = __ll2double_rn(t.y) * f;
+  if (e <= 58) {
+    re *= __longlong_as_double(1LL << 52);
+    im *= __longlong_as_double(1LL << 52);
+  }
+  T o;
+  o.x = re;
+  o.y = im;
+  return o;
+}
+
+// One fibre of N values, str apart.
+template <int N>
+__device__ __forceinline__ void rotate_fibre(longlong2 *p, const int2 *__restrict__ u, int str) {
+  {
+    int4 in[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const longlong2 t = p[k * str];
+      const int re = ((int)((unsigned)t.x << 2)) >> 2, im = ((int)((unsigned)t.y << 2)) >> 2;
+      in[k] = make_int4((int)((t.x - re) >> 30), re, (int)((t.y - im) >> 30), im);
+    }
+    for (int i = 0; i < N; ++i) {
+      long long hr = 0, xr = 0, hi = 0, xi = 0;
+#pragma unroll
+      for (int k = 0; k < N; ++k) {
+        const int2 c = u[k * N + i];
+        hr += (long long)c.x * in[k].x;
+        xr += (long long)c.x * in[k].y;
+        xr += (long long)c.y * in[k].x;
+        hi += (long long)c.x * in[k].z;
+        xi += (long long)c.x * in[k].w;
+        xi += (long long)c.y * in[k].z;
+      }
+      p[i * str] = make_longlong2((hr << 1) + ((xr + (1LL << 28)) >> 29), (hi << 1) + ((xi + (1LL << 28)) >> 29));
+    }
+  }
+}
+
+// Fibres f = warp, warp + warps, ... of one lane's column.
+template <int N>
+__device__ __forceinline__ void rotate_fibres(longlong2 *v, const int2 *__restrict__ u, int str, int d, int warp,
+                                              int warps) {
+  for (int f = warp; f < d / N; f += warps)
+    rotate_fibre<N>(v + ((f / str) * str * N + f % str) * kRotPad, u, str * kRotPad);
+}
+
+template <typename Tin, typename Tout, bool kRight>
+__global__ void __launch_bounds__(256) rotate_kernel(const Tin *x, Tout *out, const int2 *__restrict__ u, const __grid_constant__ RotOps r,
+                                                     int panels) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  longlong2 *v = reinterpret_cast<longlong2 *>(smem);   // [d][33], second index along the panel
+  __shared__ int lexp[32];
+  __shared__ unsigned lsum[32];
+  const int d = r.d;
+  const int64_t item = blockIdx.x / panels;
+  const int p0 = (int)(blockIdx.x - item * panels) * 32, np = min(32, d - p0);
+  const Tin *xi = x + item * d * d;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  if (threadIdx.x < 32) {
+    lexp[lane] = 1;
+    lsum[lane] = 0;
+  }
+  if (!kRight) {
+    if (lane < np)
+      for (int c = warp; c < d; c += warps) {
+        const Tin t = xi[(int64_t)c * d + p0 + lane];
+        reinterpret_cast<double2 *>(v)[c * kRotPad + lane] = make_double2((double)t.x, (double)t.y);
+      }
+  } else {
+    for (int k = threadIdx.x; k < np * d; k += blockDim.x) {
+      const Tin t = xi[(int64_t)p0 * d + k];
+      const int a = k / d;
+      reinterpret_cast<double2 *>(v)[(k - a * d) * kRotPad + a] = make_double2((double)t.x, (double)t.y);
+    }
+  }
+  __syncthreads();
+  // exponent of the column's largest component, then of (an upper bound of) its 2-norm,
+  // from an integer sum of squares (the same whatever the order)
+  if (lane < np) {
+    int e = 0;
+    for (int c = warp; c < d; c += warps) e = max(e, exp_field(reinterpret_cast<double2 *>(v)[c * kRotPad + lane]));
+    atomicMax(lexp + lane, e);
+  }
+  __syncthreads();
+  const int e1 = lexp[lane];
+  if (lane < np) {
+    unsigned q = 0;
+    for (int c = warp; c < d; c += warps) {
+      const double2 t = reinterpret_cast<double2 *>(v)[c * kRotPad + lane];
+      const int2 re = to_limbs(t.x, e1, 60, 30), im = to_limbs(t.y, e1, 60, 30);
+      // |component| / 2^29 < 1 up to the low limb's share
+      const float a = (float)(abs(re.x) + 1) * (1.f / (1 << 29)), b = (float)(abs(im.x) + 1) * (1.f / (1 << 29));
+      q += (unsigned)((a * a + b * b) * 262144.f) + 2u;
+    }
+    atomicAdd(lsum + lane, q);
+  }
+  __syncthreads();
+  // norm <= 2^(e1 - 1022 + k), 4^k >= lsum / 2^18
+  const int lg = 32 - __clz(lsum[lane]);
+  const int en = e1 + (lg > 18 ? (lg - 17) / 2 : 0);
+  if (lane < np)
+    for (int c = warp; c < d; c += warps) {
+      longlong2 *p = v + c * kRotPad + lane;
+      const double2 t = *reinterpret_cast<double2 *>(p);
+      *p = make_longlong2(to_fixed59(t.x, en), to_fixed59(t.y, en));
+    }
+  for (int s = 0; s < r.n_modes; ++s) {
+    __syncthreads();
+    const int n = r.dims[s], str = r.stride[s];
+    const int2 *us = u + r.off[s];
+    if (lane < np) {
+      longlong2 *vl = v + lane;
+      switch (n) {   // fibre lengths unrolled: the fibre stays in registers
+        case 2: rotate_fibres<2>(vl, us, str, d, warp, warps); break;
+        case 3: rotate_fibres<3>(vl, us, str, d, warp, warps); break;
+        case 4: rotate_fibres<4>(vl, us, str, d, warp, warps); break;
+        case 5: rotate_fibres<5>(vl, us, str, d, warp, warps); break;
+        case 6: rotate_fibres<6>(vl, us, str, d, warp, warps); break;
+        case 7: rotate_fibres<7>(vl, us, str, d, warp, warps); break;
+        case 8: rotate_fibres<8>(vl, us, str, d, warp, warps); break;
+        default: break;   // one level: the identity
+      }
+    }
+  }
+  __syncthreads();
+  Tout *oi = out + item * d * d;
+  auto store = [&](int64_t at, const longlong2 &t, int e, bool finite) { oi[at] = from_fixed59<Tout>(t, e, finite); };
+  if (!kRight) {
+    if (lane < np)
+      for (int c = warp; c < d; c += warps) store((int64_t)c * d + p0 + lane, v[c * kRotPad + lane], en, e1 < 0x7ff);
+  } else {
+    if (threadIdx.x < 32) lsum[lane] = (unsigned)en;
+    __syncthreads();
+    for (int k = threadIdx.x; k < np * d; k += blockDim.x) {
+      const int a = k / d;
+      store((int64_t)p0 * d + k, v[(k - a * d) * kRotPad + a], (int)lsum[a], lexp[a] < 0x7ff);
+    }
+  }
+}
+
+template <typename T>
+const T *up(const std::vector<T> &v, std::vector<void *> &allocs) {
+  void *p = nullptr;
+  const size_t bytes = std::max<size_t>(16, v.size() * sizeof(T));
+  if (device_malloc(&p, bytes) != cudaSuccess) {
+    (void)cudaGetLastError();
+    throw DeviceOom();
+  }
+  allocs.push_back(p);
+  if (!v.empty()) cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
+  return (const T *)p;
+}
+
+int digits_differ(const Model &M, int a, int c) {
+  int k = 0;
+  for (int s = 0; s < M.n_modes; ++s) k += (a / M.stride[s]) % M.dims[s] != (c / M.stride[s]) % M.dims[s];
+  return k;
+}
+
+// Structural non-zeros in a row of H'.
+int row_products(const Model &M) {
+  int nz = 0;
+  for (int c = 0; c < M.d; ++c) nz += digits_differ(M, 0, c) <= 2;
+  return nz;
+}
+
+// Unevaluated sum of two doubles (about 32 digits), enough operations for the basis
+// change of H.
+struct DD {
+  double h = 0.0, l = 0.0;
+  void add_product(DD a, DD b) {
+    const double p = a.h * b.h;
+    const double e = std::fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h);
+    const double s = h + p, v = s - h;
+    const double r = ((h - (s - v)) + (p - v)) + l + e;
+    h = s + r;
+    l = r - (h - s);
+  }
+};
+
+// H' = U^T H U, mode by mode, to about 32 digits.
+std::vector<DD> coupling_h(const Model &M) {
+  const int d = M.d;
+  std::vector<DD> A((size_t)d * d), v;
+  for (size_t i = 0; i < A.size(); ++i) A[i].h = M.H[i];
+  for (int side = 0; side < 2; ++side)
+    for (int s = 0; s < M.n_modes; ++s) {
+      const int n = M.dims[s], str = M.stride[s];
+      v.resize(n);
+      for (int f = 0; f < d / n; ++f) {
+        const int base = (f / str) * str * n + f % str;
+        for (int o = 0; o < d; ++o) {
+          auto at = [&](int k) -> DD & {
+            return side == 0 ? A[(size_t)(base + k * str) * d + o] : A[(size_t)o * d + base + k * str];
+          };
+          for (int k = 0; k < n; ++k) v[k] = at(k);
+          for (int i = 0; i < n; ++i) {
+            DD acc;
+            for (int k = 0; k < n; ++k)
+              acc.add_product(DD{M.vb_Us[s][(size_t)k * n + i], M.vb_Us_lo[s][(size_t)k * n + i]}, v[k]);
+            at(i) = acc;
+          }
+        }
+      }
+    }
+  return A;
+}
+
+int table_size(const Model &M) {
+  int t = 0;
+  for (int s = 0; s < M.n_modes; ++s) t += M.dims[s] * M.dims[s];
+  return t;
+}
+
+size_t panel_smem(int d, int tab) { return (size_t)tab * 16 + (size_t)d * (kPanel + 1) * 16; }
+
+size_t fused_smem(int d, int tab, int m, bool t) {
+  return (size_t)tab * 16 + (size_t)m * d * (d | 1) * 16 * (t ? 2 : 1) + (size_t)m * (sizeof(List) + 4) + 64;
+}
+
+int row_group(const Model &M) {
+  const int n = M.dims.back();
+  return n % 5 == 0 ? 5 : n % 3 == 0 ? 6 : 4;
+}
+
+bool is_fused(int d, int tab) { return fused_smem(d, tab, 1, false) <= kFusedSmem; }
+
+// Items per block of the whole-item kernel: enough columns for two to four warps of
+// lanes, as long as the launch still has a few blocks per SM.
+int items_per_block(int d, int tab, int64_t items) {
+  int m = std::max(1, 128 / d);
+  m = (int)std::min<int64_t>(m, std::max<int64_t>(1, items / (152 * 4)));
+  while (m > 1 && fused_smem(d, tab, m, true) > 56 * 1024) --m;
+  return m;
+}
+
+F64Set make_set(const F64Buf &b, int64_t begin, bool *fused, size_t *smem, int64_t *blocks) {
+  const F64Ops &O = *b.ops;
+  F64Set s{};
+  s.O = O;
+  s.w = b.w;
+  s.y = b.y;
+  s.out = b.out;
+  s.tp = b.tp;
+  s.begin = begin;
+  s.items = (int64_t)b.branches * O.n_ado;
+  *fused = is_fused(O.d, O.tab);
+  if (*fused) {
+    s.per_block = items_per_block(O.d, O.tab, s.items);
+    s.smem_t = fused_smem(O.d, O.tab, s.per_block, true) <= 56 * 1024;
+    *smem = fused_smem(O.d, O.tab, s.per_block, s.smem_t);
+    *blocks = (s.items + s.per_block - 1) / s.per_block;
+  } else {
+    s.per_block = (O.d + kPanel - 1) / kPanel;
+    *smem = panel_smem(O.d, O.tab);
+    *blocks = s.items * s.per_block;
+  }
+  return s;
+}
+
+template <typename K>
+void allow_smem(K kernel, size_t smem) {
+  if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
+template <int R, bool kMulti>
+void launch_r(const F64Args &a, bool fused, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
+  if (fused) {
+    allow_smem(f64_item_kernel<R, kMulti>, smem);
+    f64_item_kernel<R, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
+    count_launch(1);
+  } else {
+    allow_smem(f64_panel_kernel<R, false, kMulti>, smem);
+    allow_smem(f64_panel_kernel<R, true, kMulti>, smem);
+    f64_panel_kernel<R, false, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
+    f64_panel_kernel<R, true, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
+    count_launch(2);
+  }
+}
+
+void launch(const F64Args &a, int R, bool fused, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
+  if (blocks == 0) return;
+  if (blocks > 0x7fffffffLL) throw std::invalid_argument("too many work items for one stage launch");
+  auto with = [&](auto multi) {
+    constexpr bool m = decltype(multi)::value;
+    if (R == 4)
+      launch_r<4, m>(a, fused, blocks, smem, threads, st);
+    else if (R == 5)
+      launch_r<5, m>(a, fused, blocks, smem, threads, st);
+    else
+      launch_r<6, m>(a, fused, blocks, smem, threads, st);
+  };
+  if (a.n > 0)
+    with(std::true_type());
+  else
+    with(std::false_type());
+}
+
+}  // namespace
+
+bool f64_supported(const Model &M) {
+  const int tab = table_size(M);
+  if (M.n_exp > kF64MaxExp || M.n_modes > kF64MaxModes || tab > kF64MaxTab || panel_smem(M.d, tab) + sizeof(List) + 256 > kMaxSmem) return false;
+  if (row_products(M) > 500) return false;   // the 64-bit sums stay exact
+  for (double h : M.vb_H)
+    if (!std::isfinite(h)) return false;
+  return true;
+}
+
+F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::vector<int32_t> &nb_idx,
+                 const std::vector<double> &nb_cA, const std::vector<double> &nb_cB, double hsign,
+                 std::vector<void *> &allocs) {
+  F64Ops O;
+  const int d = M.d, R = row_group(M);
+  O.d = d;
+  O.n_ado = M.n_ado;
+  O.n_modes = M.n_modes;
+  O.R = R;
+  O.groups = (d + R - 1) / R;
+  O.tab = table_size(M);
+  O.hsign = hsign;
+  // H' shifted by the middle of its diagonal (the commutator does not change; smaller
+  // entries, smaller rounding of the limbs) and scaled by a power of two so that the
+  // absolute sum of a row stays below 1: with |w| < 1 the integer sums cannot overflow.
+  std::vector<DD> Hc = coupling_h(M);
+  double lo = Hc[0].h, hi = lo;
+  for (int a = 0; a < d; ++a) {
+    lo = std::min(lo, Hc[(size_t)a * d + a].h);
+    hi = std::max(hi, Hc[(size_t)a * d + a].h);
+  }
+  for (int a = 0; a < d; ++a) Hc[(size_t)a * d + a].add_product(DD{-0.5 * (lo + hi), 0.0}, DD{1.0, 0.0});
+  auto h_at = [&](int a, int c) {
+    if (digits_differ(M, a, c) > 2) return DD();
+    return Hc[(size_t)std::min(a, c) * d + std::max(a, c)];
+  };
+  double norm = 0.0;
+  for (int a = 0; a < d; ++a) {
+    double s = 0.0;
+    for (int c = 0; c < d; ++c) s += std::fabs(h_at(a, c).h);
+    norm = std::max(norm, s);
+  }
+  std::frexp(norm > 0 ? norm * (1 + 1e-12) : 1.0, &O.hexp);
+  // |h1|, |z1| <= 2^30 and |h0|, |z0| <= 2^(low - 1): the cross sum stays below
+  // (products + 1) 2^(29 + low) < 2^63
+  const int bits = row_products(M) <= 250 ? 57 : 56, low = bits - 31;
+  O.bits = bits;
+  auto limbs = [&](int a, int c) {
+    const DD h = h_at(a, c);
+    const double x = std::ldexp(h.h, bits - 1 - O.hexp);
+    const long long v0 = std::llrint(x), v = v0 + std::llrint(x - (double)v0 + std::ldexp(h.l, bits - 1 - O.hexp));
+    int2 r;
+    r.y = (int)((unsigned)(unsigned long long)v << (32 - low)) >> (32 - low);
+    r.x = (int)((v - r.y) >> low);
+    return r;
+  };
+  std::vector<int> foff(1, 0), fc, soff(1, 0);
+  std::vector<int4> fh, sh;
+  for (int g = 0; g < O.groups; ++g) {
+    const int a0 = g * R, a1 = std::min(d, a0 + R);
+    std::vector<std::vector<int>> single(R);
+    for (int c = 0; c < d; ++c) {
+      int nz = 0;
+      for (int a = a0; a < a1; ++a) nz += digits_differ(M, a, c) <= 2;
+      // all rows together (one read of w, R products) or row by row
+      if (2 * nz > R) {
+        fc.push_back(c);
+        for (int p = 0; p < (R + 1) / 2; ++p) {
+          const int2 u = a0 + 2 * p < a1 ? limbs(a0 + 2 * p, c) : make_int2(0, 0);
+          const int2 v = 2 * p + 1 >= R ? make_int2(c, 0) : a0 + 2 * p + 1 < a1 ? limbs(a0 + 2 * p + 1, c) : make_int2(0, 0);
+          fh.push_back(make_int4(u.x, u.y, v.x, v.y));
+        }
+      } else {
+        for (int a = a0; a < a1; ++a)
+          if (digits_differ(M, a, c) <= 2) single[a - a0].push_back(c);
+      }
+    }
+    foff.push_back((int)fc.size());
+    for (int r = 0; r < R; ++r) {
+      for (int c : single[r]) {
+        const int2 v = limbs(a0 + r, c);
+        sh.push_back(make_int4(v.x, v.y, c, 0));
+      }
+      soff.push_back((int)sh.size());
+    }
+  }
+  std::vector<F64Entry> nb(nb_idx.size());
+  for (size_t q = 0; q < nb.size(); ++q)
+    nb[q] = F64Entry{nb_idx[q], nb_cB[q] != 0.0 ? 2 : nb_cA[q] != 1.0 ? 1 : 0, nb_cA[q], nb_cB[q]};
+  std::vector<double2> fg;
+  std::vector<uint16_t> dig((size_t)M.n_modes * d);
+  for (int s = 0; s < M.n_modes; ++s) {
+    O.dims[s] = M.dims[s];
+    O.tab_off[s] = (int)fg.size();
+    for (int a = 0; a < M.dims[s]; ++a)
+      for (int b = 0; b < M.dims[s]; ++b)   // lam_a -+ lam_b, rounded once
+        fg.push_back(make_double2((M.vb_lam[s][a] - M.vb_lam[s][b]) + (M.vb_lam_lo[s][a] - M.vb_lam_lo[s][b]),
+                                  (M.vb_lam[s][a] + M.vb_lam[s][b]) + (M.vb_lam_lo[s][a] + M.vb_lam_lo[s][b])));
+    for (int a = 0; a < d; ++a) dig[(size_t)s * d + a] = (uint16_t)((a / M.stride[s]) % M.dims[s]);
+  }
+  O.foff = up(foff, allocs);
+  O.fc = up(fc, allocs);
+  O.fh = up(fh, allocs);
+  O.soff = up(soff, allocs);
+  O.sh = up(sh, allocs);
+  O.noff = up(std::vector<int>(nb_off.begin(), nb_off.end()), allocs);
+  O.nb = up(nb, allocs);
+  O.decay = up(M.decay, allocs);
+  O.fg = up(fg, allocs);
+  O.dig = up(dig, allocs);
+  O.ready = true;
+  return O;
+}
+
+std::vector<std::pair<int, int>> f64_shapes(const F64Buf &b) {
+  bool fused = false;
+  size_t smem = 0;
+  int64_t blocks = 0;
+  make_set(b, 0, &fused, &smem, &blocks);
+  const int n = (int)std::min<int64_t>(blocks, 0x7fffffff);
+  if (fused) return {{256, n}, {128, n}, {64, n}};
+  return {{kPanelThreads, n}, {256, n}, {192, n}};
+}
+
+void f64_stage(const F64Buf &b, double alpha, int threads, cudaStream_t st) {
+  bool fused = false;
+  size_t smem = 0;
+  int64_t blocks = 0;
+  F64Args a{};
+  a.one = make_set(b, 0, &fused, &smem, &blocks);
+  a.alpha = alpha;
+  launch(a, b.ops->R, fused, blocks, smem, threads, st);
+}
+
+F64Plan::~F64Plan() {
+  for (Class &c : classes)
+    if (c.desc) cudaFree(c.desc);
+}
+
+void f64_plan(F64Plan &p, const std::vector<F64Buf> &sets, cudaStream_t st) {
+  std::map<std::pair<int, bool>, std::vector<F64Set>> by;
+  std::map<std::pair<int, bool>, std::pair<int64_t, size_t>> size;
+  for (const F64Buf &b : sets) {
+    bool fused = false;
+    size_t smem = 0;
+    int64_t blocks = 0;
+    F64Set s = make_set(b, 0, &fused, &smem, &blocks);
+    auto key = std::make_pair(b.ops->R, fused);
+    s.begin = size[key].first;
+    size[key].first += blocks;
+    size[key].second = std::max(size[key].second, smem);
+    by[key].push_back(s);
+  }
+  for (auto &kv : by) {
+    F64Plan::Class c{kv.first.first, kv.first.second, size[kv.first].first, size[kv.first].second,
+                     (int)kv.second.size(), nullptr};
+    if (device_malloc(&c.desc, kv.second.size() * sizeof(F64Set)) != cudaSuccess) {
+      (void)cudaGetLastError();
+      throw DeviceOom();
+    }
+    p.classes.push_back(c);
+    cudaMemcpyAsync(c.desc, kv.second.data(), kv.second.size() * sizeof(F64Set), cudaMemcpyHostToDevice, st);
+  }
+  cudaStreamSynchronize(st);
+}
+
+void f64_stage_plan(const F64Plan &p, double alpha, cudaStream_t st) {
+  for (const F64Plan::Class &c : p.classes) {
+    F64Args a{};
+    a.many = (const F64Set *)c.desc;
+    a.n = c.n;
+    a.alpha = alpha;
+    launch(a, c.R, c.fused, c.blocks, c.smem, c.fused ? 256 : kPanelThreads, st);
+  }
+}
+
+bool rot_supported(const Model &M) {
+  if (M.n_modes > kF64MaxModes || (size_t)M.d * kRotPad * 16 + 512 > kMaxSmem) return false;
+  for (int n : M.dims)
+    if (n > kRotMaxN) return false;
+  return true;
+}
+
+RotOps rot_build(const Model &M, std::vector<void *> &allocs) {
+  RotOps r;
+  r.d = M.d;
+  r.n_modes = M.n_modes;
+  std::vector<int2> f, b;
+  for (int s = 0; s < M.n_modes; ++s) {
+    const int n = M.dims[s];
+    auto limbs = [&](int k, int i) {
+      const double h = std::ldexp(M.vb_Us[s][(size_t)k * n + i], 59), l = std::ldexp(M.vb_Us_lo[s][(size_t)k * n + i], 59);
+      const long long v0 = std::llrint(h), v = v0 + std::llrint(h - (double)v0 + l);
+      int2 c;
+      c.y = (int)((unsigned)(unsigned long long)v << 2) >> 2;
+      c.x = (int)((v - c.y) >> 30);
+      return c;
+    };
+    r.dims[s] = n;
+    r.stride[s] = M.stride[s];
+    r.off[s] = (int)f.size();
+    for (int k = 0; k < n; ++k)
+      for (int i = 0; i < n; ++i) {
+        f.push_back(limbs(k, i));
+        b.push_back(limbs(i, k));
+      }
+  }
+  r.fwd = up(f, allocs);
+  r.bwd = up(b, allocs);
+  r.ready = true;
+  return r;
+}
+
+template <typename Tin, typename Tout>
+void rotate(const RotOps &r, bool forward, const Tin *x, Tout *out, double2 *tmp, int64_t items, cudaStream_t st) {
+  if (items <= 0) return;
+  const int panels = (r.d + 31) / 32;
+  const int64_t blocks = items * panels;
+  if (blocks > 0x7fffffffLL) throw std::invalid_argument("too many work items for one launch");
+  const int2 *u = forward ? r.fwd : r.bwd;
+  const size_t smem = (size_t)r.d * kRotPad * 16;
+  allow_smem(rotate_kernel<Tin, double2, false>, smem);
+  allow_smem(rotate_kernel<double2, Tout, true>, smem);
+  rotate_kernel<Tin, double2, false><<<(unsigned)blocks, 256, smem, st>>>(x, tmp, u, r, panels);
+  rotate_kernel<double2, Tout, true><<<(unsigned)blocks, 256, smem, st>>>(tmp, out, u, r, panels);
+  count_launch(2);
+}
+
+template void rotate<double2, double2>(const RotOps &, bool, const double2 *, double2 *, double2 *, int64_t, cudaStream_t);
+template void rotate<double2, float2>(const RotOps &, bool, const double2 *, float2 *, double2 *, int64_t, cudaStream_t);
+template void rotate<float2, double2>(const RotOps &, bool, const float2 *, double2 *, double2 *, int64_t, cudaStream_t);
+
+}  // namespace heom

@@ -386,7 +386,7 @@ extern "C" heom_status heom_response_2d_grad(heom_hier *h, const heom_state *rho
     DeviceBuffer Tst((size_t)n1 * sz1), Tbar((size_t)n1 * sz1);
     CUDA_TRY(cudaMemsetAsync(Tbar.p, 0, Tbar.bytes, st));
     double2 *T = (double2 *)Tst.p, *Tb = (double2 *)Tbar.p;
-    kick_into<double>(h, (const double2 *)rho_eq->buf.p, T, 1, 2, st);
+    kick_into<double>(h, (const double2 *)rho_eq->buf.p, T, 1, mu_of<double>(h, 2), st);
     for (int j = 1; j < n1; ++j) {
       CUDA_TRY(cudaMemcpyAsync(T + (int64_t)j * per, T + (int64_t)(j - 1) * per, sz1, cudaMemcpyDeviceToDevice, st));
       rk4_steps<double>(h, T + (int64_t)j * per, c.W4, c.W3, 1, dt, m, st, HEOM_FP64);
@@ -409,7 +409,7 @@ extern "C" heom_status heom_response_2d_grad(heom_hier *h, const heom_state *rho
         }
         CUDA_TRY(cudaMemcpyAsync(t1, br, (size_t)B * sz1, cudaMemcpyDeviceToDevice, st));   // F = G^{n2} BR
         rk4_steps<double>(h, t1, c.W4, c.W3, B, dt, n2[it], st, HEOM_FP64);
-        kick_into<double>(h, t1, y0, B, 1, st);                                              // Y0 = mu+^x F
+        kick_into<double>(h, t1, y0, B, mu_of<double>(h, 1), st);                                              // Y0 = mu+^x F
         // t3: traces at t = k m; lam starts with the source of the last sample
         CUDA_TRY(cudaMemsetAsync(lm, 0, (size_t)B * sz1, st));
         auto trace_src = [&](int64_t t, const double2 *y, double2 *l) {
@@ -434,19 +434,19 @@ extern "C" heom_status heom_response_2d_grad(heom_hier *h, const heom_state *rho
         backprop_span(c, y0, N3, B, dt, Mck, lm, trace_src);
         // third kick: Fbar = mu-^x Y0bar; d/d mu+
         comm_grad(c, lm, t1, (int64_t)B * M.n_ado, 1.0, 0.0, 1.0, c.G + c.L.mup);
-        kick_into<double>(h, lm, t2b, B, 2, st);
+        kick_into<double>(h, lm, t2b, B, mu_of<double>(h, 2), st);
         // t2
         backprop_span(c, br, n2[it], B, dt, Mck, t2b, nullptr);
         // second kicks: I_j = mu+^x T_j, II_j = mu-^x (-T_j^dagger)
         double2 *Tj = T + (int64_t)j0 * per, *Tbj = Tb + (int64_t)j0 * per;
         const int64_t nI = (int64_t)nj * per;
         comm_grad(c, t2b, Tj, (int64_t)nj * M.n_ado, 1.0, 0.0, 1.0, c.G + c.L.mup);
-        kick_into<double>(h, t2b, t1, nj, 2, st);
+        kick_into<double>(h, t2b, t1, nj, mu_of<double>(h, 2), st);
         axpy64(c, Tbj, t1, 1.0, nI);
         neg_dagger_kernel<<<grid_for(nI), 256, 0, st>>>(Tj, t1, d, nI);                     // U = -T^dagger
         count_launch(1);
         comm_grad(c, t2b + nI, t1, (int64_t)nj * M.n_ado, 1.0, 0.0, 1.0, c.G + c.L.mum);
-        kick_into<double>(h, t2b + nI, t1, nj, 1, st);                                      // Ubar = mu+^x IIbar
+        kick_into<double>(h, t2b + nI, t1, nj, mu_of<double>(h, 1), st);                                      // Ubar = mu+^x IIbar
         neg_dagger_kernel<<<grid_for(nI), 256, 0, st>>>(t1, y0, d, nI);
         count_launch(1);
         LAUNCH_CHECK();
@@ -464,7 +464,7 @@ extern "C" heom_status heom_response_2d_grad(heom_hier *h, const heom_state *rho
     backprop_span(c, T, N1, 1, dt, Mck, lm, trunk_src);
     comm_grad(c, lm, (const double2 *)rho_eq->buf.p, M.n_ado, 1.0, 0.0, 1.0, c.G + c.L.mum);
     double2 *eqbar = (double2 *)tmp.p;
-    kick_into<double>(h, lm, eqbar, 1, 1, st);                                             // (mu-^x)^H = mu+^x
+    kick_into<double>(h, lm, eqbar, 1, mu_of<double>(h, 1), st);                                             // (mu-^x)^H = mu+^x
     DeviceBuffer rho0(sz1);
     CUDA_TRY(cudaMemsetAsync(rho0.p, 0, sz1, st));
     const double one[2] = {1.0, 0.0};

@@ -26,6 +26,7 @@
 #endif
 
 #include "heom2dvs.h"
+#include "f64_stage.h"
 #include "kernels.cuh"
 #include "model.h"
 #include "tc_stage.h"
@@ -130,7 +131,10 @@ struct heom_hier {
   VbModel vb{};                 // coupling-eigenbasis model (FP32 paths)
   double *U64 = nullptr, *UT64 = nullptr;        // coupling eigenbasis U and U^T
   float *mu_vb32 = nullptr, *mup_vb32 = nullptr, *mum_vb32 = nullptr;
-  double *mu_vb64 = nullptr;                     // mu in the coupling basis (traces)
+  double *mu_vb64 = nullptr, *mup_vb64 = nullptr, *mum_vb64 = nullptr;   // mu, mu+, mu- there
+  // FP64 propagation in the coupling basis (f64.ready), and the basis change mode by mode
+  F64Ops f64{}, f64_adj{};
+  RotOps rot{};
   bool on_device = false;
   double spread = -1.0, max_decay = 0.0;   // Bohr spread of H_S' (< 0: not computed yet), largest decay rate
   // copy of the model description (for the parameter gradient)
@@ -206,21 +210,49 @@ inline const float *mu_of<float>(heom_hier *h, int which) {
   return which == 0 ? h->mu_vb32 : which == 1 ? h->mup_vb32 : h->mum_vb32;
 }
 
+// The working basis of FP64 propagations inside a call: the coupling eigenbasis when
+// the model fits the engine of f64_stage.h, else the product basis.  mu_work and
+// mu_trace_work give mu, mu+, mu- (which 0, 1, 2) and the trace's mu there; complex64
+// states are always in the coupling basis.
+template <typename R>
+const R *mu_work(heom_hier *h, int which);
+template <>
+inline const double *mu_work<double>(heom_hier *h, int which) {
+  if (!h->f64.ready) return mu_of<double>(h, which);
+  return which == 0 ? h->mu_vb64 : which == 1 ? h->mup_vb64 : h->mum_vb64;
+}
+template <>
+inline const float *mu_work<float>(heom_hier *h, int which) { return mu_of<float>(h, which); }
+template <typename R>
+const double *mu_trace_work(heom_hier *h) {
+  return sizeof(R) == 8 && !h->f64.ready ? h->mu_trace : h->mu_vb64;
+}
+// Product basis -> working basis and back (tmp: scratch of the same size; out may
+// equal x).
+void work_in(heom_hier *h, const double2 *x, double2 *out, double2 *tmp, int branches, cudaStream_t st);
+void work_out(heom_hier *h, const double2 *x, double2 *out, double2 *tmp, int branches, cudaStream_t st);
+// RK4 steps of FP64 branches in the working basis, and one right-hand side out = L w
+// (out not w).
+void rk4_work64(heom_hier *h, double2 *y, double2 *wa, double2 *wb, int branches, double dt, int64_t nsteps,
+                cudaStream_t st);
+void rhs_work64(heom_hier *h, const double2 *w, double2 *out, int branches, cudaStream_t st);
+
 // Necessary condition for RK4 stability (Bohr spread and decay rates x dt inside
 // the RK4 region); throws HEOM_EUNSTABLE.
 void stability_check(heom_hier *h, double dt);
 
-// nsteps RK4 steps (Horner form) of every branch in y, scratch wa and wb.
+// nsteps RK4 steps (Horner form) of every branch in y, scratch wa and wb; FP64 states
+// in the product basis.
 template <typename R>
 void rk4_steps(heom_hier *h, typename CxT<R>::type *y, typename CxT<R>::type *wa, typename CxT<R>::type *wb,
                int branches, double dt, int64_t nsteps, cudaStream_t st, int precision);
-// out = K^x in for K = mu (which 0), mu+ (1), mu- (2).
+// out = K^x in (K of mu_of or mu_work).
 template <typename R>
-void kick_into(heom_hier *h, const typename CxT<R>::type *in, typename CxT<R>::type *out, int branches, int which,
+void kick_into(heom_hier *h, const typename CxT<R>::type *in, typename CxT<R>::type *out, int branches, const R *K,
                cudaStream_t st);
 // i^order tr{mu rho_0} of each branch into out[branch * ostride].
 template <typename R>
-void trace_into(heom_hier *h, const typename CxT<R>::type *w, int branches, int order, double2 *out,
+void trace_into(heom_hier *h, const typename CxT<R>::type *w, int branches, const double *mu, int order, double2 *out,
                 int64_t ostride, cudaStream_t st);
 
 // Stream capture of a launch sequence into a CUDA graph, replayed once by

@@ -115,29 +115,6 @@ __global__ void __launch_bounds__(256) stage_kernel(const typename CxT<R>::type 
     stage_element<R>(w, y, out, alpha, M, e);
 }
 
-// The same stage for several hierarchies (parameter sets, any basis size) in one
-// launch: set k owns elements [begin_k, begin_k + total_k) of the flattened
-// index space and has its own model and state pointers.
-template <typename R>
-struct SetStage {
-  DevModel<R> M;
-  const typename CxT<R>::type *w, *y;
-  typename CxT<R>::type *out;
-  int64_t begin, total;
-};
-
-template <typename R>
-__global__ void __launch_bounds__(256) multi_stage_kernel(const SetStage<R> *__restrict__ sets, int n_sets,
-                                                          R alpha, int64_t grand_total) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < grand_total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    int k = 0;
-    while (k + 1 < n_sets && e >= sets[k + 1].begin) ++k;
-    const SetStage<R> &S = sets[k];
-    stage_element<R>(S.w, S.y, S.out, alpha, S.M, e - S.begin);
-  }
-}
-
 // out = K w - w K for every ADO of every branch (dipole kick K^x).  K real d x d.
 template <typename R>
 __global__ void __launch_bounds__(256) kick_kernel(const typename CxT<R>::type *__restrict__ w,

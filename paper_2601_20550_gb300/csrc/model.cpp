@@ -24,38 +24,39 @@ static const double kBoltzmannCm = 0.6950348005;
 // destroyed; on return w holds ascending eigenvalues and the columns of Z the
 // eigenvectors.
 // ---------------------------------------------------------------------------
-void jacobi_eigh(std::vector<double> &A, int n, std::vector<double> &w, std::vector<double> &Z) {
+template <typename T>
+static void jacobi(std::vector<T> &A, int n, std::vector<T> &w, std::vector<T> &Z, T rel) {
   Z.assign((size_t)n * n, 0.0);
   for (int i = 0; i < n; ++i) Z[(size_t)i * n + i] = 1.0;
-  auto a = [&](int i, int j) -> double & { return A[(size_t)i * n + j]; };
+  auto a = [&](int i, int j) -> T & { return A[(size_t)i * n + j]; };
   for (int sweep = 0; sweep < 100; ++sweep) {
-    double off = 0.0, diag = 0.0;
+    T off = 0.0, diag = 0.0;
     for (int i = 0; i < n; ++i) {
       diag += a(i, i) * a(i, i);
       for (int j = i + 1; j < n; ++j) off += a(i, j) * a(i, j);
     }
-    if (off <= 1e-30 * diag || off == 0.0) break;
+    if (off <= rel * diag || off == 0.0) break;
     for (int p = 0; p < n - 1; ++p) {
       for (int q = p + 1; q < n; ++q) {
-        double apq = a(p, q);
+        T apq = a(p, q);
         if (std::fabs(apq) < 1e-300) continue;
-        double app = a(p, p), aqq = a(q, q);
-        double theta = (aqq - app) / (2.0 * apq);
-        double t = (theta >= 0 ? 1.0 : -1.0) / (std::fabs(theta) + std::sqrt(theta * theta + 1.0));
-        double c = 1.0 / std::sqrt(t * t + 1.0), s = t * c;
+        T app = a(p, p), aqq = a(q, q);
+        T theta = (aqq - app) / (2 * apq);
+        T t = (theta >= 0 ? T(1) : T(-1)) / (std::fabs(theta) + std::sqrt(theta * theta + T(1)));
+        T c = T(1) / std::sqrt(t * t + T(1)), s = t * c;
         // rotate rows/columns p and q
         for (int k = 0; k < n; ++k) {
-          double akp = a(k, p), akq = a(k, q);
+          T akp = a(k, p), akq = a(k, q);
           a(k, p) = c * akp - s * akq;
           a(k, q) = s * akp + c * akq;
         }
         for (int k = 0; k < n; ++k) {
-          double apk = a(p, k), aqk = a(q, k);
+          T apk = a(p, k), aqk = a(q, k);
           a(p, k) = c * apk - s * aqk;
           a(q, k) = s * apk + c * aqk;
         }
         for (int k = 0; k < n; ++k) {
-          double zkp = Z[(size_t)k * n + p], zkq = Z[(size_t)k * n + q];
+          T zkp = Z[(size_t)k * n + p], zkq = Z[(size_t)k * n + q];
           Z[(size_t)k * n + p] = c * zkp - s * zkq;
           Z[(size_t)k * n + q] = s * zkp + c * zkq;
         }
@@ -66,12 +67,16 @@ void jacobi_eigh(std::vector<double> &A, int n, std::vector<double> &w, std::vec
   for (int i = 0; i < n; ++i) order[i] = i;
   std::sort(order.begin(), order.end(), [&](int x, int y) { return a(x, x) < a(y, y); });
   w.resize(n);
-  std::vector<double> Zs((size_t)n * n);
+  std::vector<T> Zs((size_t)n * n);
   for (int c = 0; c < n; ++c) {
     w[c] = a(order[c], order[c]);
     for (int r = 0; r < n; ++r) Zs[(size_t)r * n + c] = Z[(size_t)r * n + order[c]];
   }
   Z.swap(Zs);
+}
+
+void jacobi_eigh(std::vector<double> &A, int n, std::vector<double> &w, std::vector<double> &Z) {
+  jacobi<double>(A, n, w, Z, 1e-30);
 }
 
 // C = A^T B A restricted: out (k x k) = U^T M U with U (n x k) column-major in a
@@ -402,13 +407,30 @@ void build_coupling_basis(Model &M) {
   const int d = M.d;
   std::vector<std::vector<double>> Us;
   M.vb_lam.clear();
+  M.vb_Us_lo.clear();
+  M.vb_lam_lo.clear();
   for (int s = 0; s < M.n_modes; ++s) {
     const int n = M.dims[s];
-    std::vector<double> A = M.Vloc[s], w, Z;
-    jacobi_eigh(A, n, w, Z);
+    // in extended precision for the usual small n_s: FP64 states are rotated into this
+    // basis and back, so the vectors are kept to twice a double's digits (hi + lo)
+    std::vector<double> w, Z, lo((size_t)n * n, 0.0), wlo(n, 0.0);
+    if (n <= 32) {
+      std::vector<long double> A(M.Vloc[s].begin(), M.Vloc[s].end()), wl, Zl;
+      jacobi<long double>(A, n, wl, Zl, 1e-36L);
+      w.assign(wl.begin(), wl.end());
+      Z.assign(Zl.begin(), Zl.end());
+      for (int i = 0; i < n; ++i) wlo[i] = (double)(wl[i] - (long double)w[i]);
+      for (size_t i = 0; i < lo.size(); ++i) lo[i] = (double)(Zl[i] - (long double)Z[i]);
+    } else {
+      std::vector<double> A = M.Vloc[s];
+      jacobi_eigh(A, n, w, Z);
+    }
     M.vb_lam.push_back(w);
     Us.push_back(Z);
+    M.vb_Us_lo.push_back(lo);
+    M.vb_lam_lo.push_back(wlo);
   }
+  M.vb_Us = Us;
   M.vb_U.assign((size_t)d * d, 0.0);
   for (int a = 0; a < d; ++a)
     for (int b = 0; b < d; ++b) {

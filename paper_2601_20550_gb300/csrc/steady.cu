@@ -48,14 +48,6 @@ static void multi_axpy(double2 *w, const double2 *V, int64_t n, const std::vecto
   CUDA_TRY(cudaStreamSynchronize(st));
 }
 
-// out = L x (one branch, FP64 product basis)
-static void apply_L(heom_hier *h, const double2 *x, double2 *out, int64_t n, cudaStream_t st) {
-  CUDA_TRY(cudaMemsetAsync(out, 0, (size_t)n * 16, st));
-  stage_kernel<double><<<grid_for(n), 256, 0, st>>>(x, out, out, 1.0, h->dm64, n);
-  count_launch(1);
-  LAUNCH_CHECK();
-}
-
 }  // namespace heom
 
 extern "C" heom_status heom_steady_state(heom_hier *h, double tol, int restart, int max_iter, double dt_fs,
@@ -94,24 +86,34 @@ extern "C" heom_status heom_steady_state(heom_hier *h, double tol, int restart, 
     if (steps_per_matvec > 0) stability_check(h, dt_fs);
     auto apply_A = [&](const double2 *in, double2 *out) {
       if (steps_per_matvec == 0) {
-        apply_L(h, in, out, n, st);
+        rhs_work64(h, in, out, 1, st);
         return;
       }
       CUDA_TRY(cudaMemcpyAsync(out, in, (size_t)n * 16, cudaMemcpyDeviceToDevice, st));
-      rk4_steps<double>(h, out, (double2 *)sa.p, (double2 *)sb.p, 1, dt_fs, steps_per_matvec, st, HEOM_FP64);
+      rk4_work64(h, out, (double2 *)sa.p, (double2 *)sb.p, 1, dt_fs, steps_per_matvec, st);
       axpy_kernel<<<grid_for(n), 256, 0, st>>>(out, in, -1.0, n);
       count_launch(1);
       LAUNCH_CHECK();
     };
     // the reference scale: ||x_0||_F of the starting state (= 1)
     const double scale = 1.0;
+    // the solve runs in the working basis (an orthogonal change: norms and inner
+    // products stay), x goes back to the product basis at the end
+    work_in(h, x, x, wp, 1, st);
+    auto back = [&]() {
+      work_out(h, x, x, wp, 1, st);
+      CUDA_TRY(cudaStreamSynchronize(st));
+    };
     while (its < max_iter) {
       // r = -L x; every vector of range(L) has tr(.)_0 = 0 (tr rho_0 is conserved),
       // so the corrections keep tr x_0 = 1
-      apply_L(h, x, vec(0), n, st);
+      rhs_work64(h, x, vec(0), 1, st);
       const double resL = std::sqrt(multi_dot(vec(0), n, 1, vec(0), partial, st)[0].real());
       if (!std::isfinite(resL)) throw Fail{HEOM_ENONFINITE, "steady-state residual is not finite"};
-      if (resL <= tol * scale) return HEOM_OK;
+      if (resL <= tol * scale) {
+        back();
+        return HEOM_OK;
+      }
       if (steps_per_matvec > 0) apply_A(x, vec(0));
       const double beta = std::sqrt(multi_dot(vec(0), n, 1, vec(0), partial, st)[0].real());
       zscal_kernel<<<grid_for(n), 256, 0, st>>>(vec(0), n, -1.0 / beta, 0.0);
@@ -172,8 +174,9 @@ extern "C" heom_status heom_steady_state(heom_hier *h, double tol, int restart, 
       }
       multi_axpy(x, Vp, n, y, coef, st);
     }
-    apply_L(h, x, wp, n, st);
+    rhs_work64(h, x, wp, 1, st);
     const double res = std::sqrt(multi_dot(wp, n, 1, wp, partial, st)[0].real());
+    back();
     if (res <= tol * scale) return HEOM_OK;
     g_last_error = "steady-state tolerance not reached within max_iter";
     return HEOM_ENOTCONV;
