@@ -186,6 +186,11 @@ void rk4_work64(heom_hier *h, double2 *y, double2 *wa, double2 *wb, int branches
   const int64_t total = (int64_t)branches * h->M.n_ado * h->M.d * h->M.d;
   if (total == 0 || nsteps <= 0) return;
   if (h->f64.ready) {
+    std::pair<int, int> one(0, 0);
+    if (f64_small_steps(h->f64, y, wa, wb, branches, dt, nsteps, st, &one)) {
+      h->tuned[{kTuneStage64, total}] = one;
+      return;
+    }
     // the commutator part of a stage goes to its output, in the last stage (out = y)
     // to the free scratch
     const F64Buf b[4] = {{&h->f64, y, y, wa, wa, branches},

@@ -31,14 +31,17 @@ struct MultiSet {
   std::unique_ptr<DeviceBuffer> eqW, T, ta, tb, P[4];   // equilibrium, trunk and its scratch; branch sets
 };
 
-// Plans of the four Horner stages of one RK4 step on the buffers (y, wa, wb) of every set.
+// Plans of RK4 steps on the buffers (y, wa, wb) of every set: all steps in one launch if
+// every set is small enough, else the four Horner stages.
 struct MultiStep {
+  F64SmallPlan small;
   F64Plan stage[4];
 };
 
 static void multi_step_setup(std::vector<MultiSet> &S, MultiStep &ms, int which_y, int which_a, int which_b,
                              int branches, cudaStream_t st) {
   std::vector<F64Buf> b[4];
+  std::vector<F64SmallBuf> all;
   for (MultiSet &s : S) {
     auto buf = [&](int w) -> double2 * {
       if (w == -1) return (double2 *)s.T->p;
@@ -47,15 +50,18 @@ static void multi_step_setup(std::vector<MultiSet> &S, MultiStep &ms, int which_
       return (double2 *)s.P[w]->p;
     };
     double2 *y = buf(which_y), *wa = buf(which_a), *wb = buf(which_b);
+    all.push_back({&s.h->f64, y, wa, wb, branches});
     b[0].push_back({&s.h->f64, y, y, wa, wa, branches});
     b[1].push_back({&s.h->f64, wa, y, wb, wb, branches});
     b[2].push_back({&s.h->f64, wb, y, wa, wa, branches});
     b[3].push_back({&s.h->f64, wa, y, y, wb, branches});
   }
+  f64_small_plan(ms.small, all, st);
   for (int q = 0; q < 4; ++q) f64_plan(ms.stage[q], b[q], st);
 }
 
 static void multi_rk4(const MultiStep &ms, double dt, int64_t nsteps, cudaStream_t st) {
+  if (nsteps <= 0 || f64_small_steps_plan(ms.small, dt, nsteps, st)) return;
   const double al[4] = {dt / 4, dt / 3, dt / 2, dt};
   for (int64_t s = 0; s < nsteps; ++s)
     for (int q = 0; q < 4; ++q) f64_stage_plan(ms.stage[q], al[q], st);

@@ -21,7 +21,11 @@
 #include <stdexcept>
 #include <type_traits>
 
+#include <cooperative_groups.h>
+
 #include "tc_stage.h"   // device_malloc, DeviceOom
+
+namespace cg = cooperative_groups;
 
 namespace heom {
 
@@ -33,6 +37,7 @@ constexpr int kPanel = 32;                 // columns (rows) of w per panel bloc
 constexpr int kPanelThreads = 384;
 constexpr int kF64MaxExp = 16;             // build_hierarchy's limit
 constexpr int kRotPad = 33;
+constexpr int kSmallD = 32;                // largest basis of f64_small_kernel
 constexpr size_t kMaxSmem = 227 * 1024;
 // Whole-item blocks up to two per SM; above, one panel of 32 columns (rows) per block.
 constexpr size_t kFusedSmem = 112 * 1024;
@@ -418,6 +423,243 @@ __global__ void __launch_bounds__(kPanelThreads, 3) f64_panel_kernel(const __gri
 }
 
 // ---------------------------------------------------------------------------
+// Many RK4 steps of a small hierarchy in one launch.  A stage of such a hierarchy takes
+// 1-3 us of the FP64 pipe of the SMs it spreads over, but 12-19 us as a launch of its
+// own, which starts with a chain of dependent table loads; here the tables stay in
+// shared memory and the blocks meet at a barrier after each stage.  Work is split into
+// units (item, row range); kSync 0: one block per branch, 1: one cluster per branch, 2:
+// the whole (cooperative) grid shares all branches' units.  The states are the caller's
+// buffers, exchanged through L2.
+// ---------------------------------------------------------------------------
+struct F64SmallSet {
+  F64Ops O;
+  double2 *y, *wa, *wb;
+  int branches;
+  int parts;          // row ranges per item
+  int units;          // units per block
+  int bpb;            // blocks per branch (kSync 0, 1), or blocks of the grid (2)
+  int begin;          // first block of the set
+};
+
+struct F64SmallArgs {
+  F64SmallSet one;
+  const F64SmallSet *many;   // kMulti: the sets' blocks follow one another (kSync 0, 1)
+  int n;
+  double alpha[4];           // dt / 4, dt / 3, dt / 2, dt
+  int64_t steps;
+};
+
+constexpr int kSmallPre = 8;   // neighbours whose loads are issued ahead
+
+// What a block of f64_small_kernel keeps in shared memory: everything the steps need
+// besides the states, with the index arithmetic done once.
+struct SmallItem {
+  int64_t base, branch;   // element offsets of the item and of its branch
+  double decay;
+  int n_nb, off[kF64MaxModes + 1];
+  F64Entry e[2 * kF64MaxExp];   // idx: element offset within the branch
+};
+
+// One thread per component of an element: the commutator's sum takes 6 IMAD.WIDE per
+// column, the rest about ten FP64 operations, which have 67 cycles of latency each and
+// so need the parallelism more than the shared loads.
+template <int kSync, bool kMulti>
+__global__ void __launch_bounds__(512) f64_small_kernel(const __grid_constant__ F64SmallArgs G) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  int ks = 0;
+  while (kMulti && ks + 1 < G.n && (int)blockIdx.x >= G.many[ks + 1].begin) ++ks;
+  const F64SmallSet &P = kMulti ? G.many[ks] : G.one;
+  const F64Ops &O = P.O;
+  const int d = O.d, ld = d | 1, dd = d * d, isz = d * ld, low = O.bits - 31, nm = O.n_modes;
+  // this block's units: consecutive in (item, part) order of its branch (kSync 2: of all)
+  const int blk = (int)blockIdx.x - P.begin;
+  const int n_units = (kSync == 2 ? P.branches : 1) * O.n_ado * P.parts;
+  const int u0 = min(n_units, (blk % P.bpb) * P.units);
+  const int nu = min(P.units, n_units - u0);
+  const int first = kSync == 2 ? 0 : (blk / P.bpb) * O.n_ado;   // first item of the branch
+  const int i0 = first + u0 / P.parts;
+  const int ni = nu > 0 ? (first + (u0 + nu - 1) / P.parts - i0) + 1 : 0;      // items touched
+  const int max_items = (P.units + P.parts - 1) / P.parts + (P.parts > 1 ? 1 : 0);
+  double2 *tab = reinterpret_cast<double2 *>(smem);
+  int4 *zs = reinterpret_cast<int4 *>(tab + O.tab);
+  SmallItem *items = reinterpret_cast<SmallItem *>(zs + max_items * isz);
+  int2 *hs = reinterpret_cast<int2 *>(items + max_items);       // H' limbs, dense
+  int *iexp = reinterpret_cast<int *>(hs + dd);                 // [2][max_items], by stage parity
+  int *dig = iexp + 2 * max_items;                              // [n_modes][2][d] table offsets of row and column
+  int *elem = dig + 2 * nm * d;                                 // this block's elements: item, row, column
+  int *place = elem + P.units * ((d + P.parts - 1) / P.parts) * d;   // its items' elements: item, offset in zs
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const int rows = (d + P.parts - 1) / P.parts;   // rows per part
+  for (int i = warp; i < ni; i += warps) {
+    SmallItem &I = items[i];
+    const int item = i0 + i, n = item % O.n_ado;
+    const int *off = O.noff + n * nm;
+    const int q0 = off[0], nq = off[nm] - q0;
+    if (lane == 0) {
+      I.base = (int64_t)item * dd;
+      I.branch = (int64_t)(item - n) * dd;
+      I.decay = O.decay[n];
+      I.n_nb = nq;
+    }
+    for (int m = lane; m <= nm; m += 32) I.off[m] = off[m] - q0;
+    for (int q = lane; q < nq; q += 32) {
+      I.e[q] = O.nb[q0 + q];
+      I.e[q].idx *= dd;
+    }
+  }
+  for (int i = threadIdx.x; i < dd; i += blockDim.x) hs[i] = O.hd[i];
+  for (int i = threadIdx.x; i < O.tab; i += blockDim.x) tab[i] = O.fg[i];
+  for (int i = threadIdx.x; i < 2 * ni; i += blockDim.x) iexp[i] = 1;
+  for (int i = threadIdx.x; i < nm * d; i += blockDim.x) {
+    const int s = i / d, a = i - s * d;
+    dig[2 * s * d + a] = O.tab_off[s] + O.dig[i] * O.dims[s];
+    dig[(2 * s + 1) * d + a] = O.dig[i];
+  }
+  for (int k = threadIdx.x; k < nu * rows * d; k += blockDim.x) {
+    const int u = k / (rows * d), r = k - u * rows * d, ug = u0 + u;
+    const int a = (ug % P.parts) * rows + r / d, b = r % d;
+    elem[k] = (first + ug / P.parts - i0) << 12 | a << 6 | b;   // a may pass d in the last part: skipped
+  }
+  for (int k = threadIdx.x; k < ni * dd; k += blockDim.x) {
+    const int i = k / dd, el = k - i * dd;
+    place[k] = i << 20 | (i * isz + el / d * ld + el % d);
+  }
+  __syncthreads();
+  const int work = 2 * nu * rows * d, nz = ni * dd;
+  const int64_t z0 = (int64_t)i0 * dd;
+  int parity = 0;
+  for (int64_t s = 0; s < G.steps; ++s)
+    for (int q = 0; q < 4; ++q, parity ^= 1) {
+      const double2 *w = q == 0 ? P.y : q == 2 ? P.wb : P.wa;
+      double2 *out = q == 3 ? P.y : q == 1 ? P.wb : P.wa;
+      const double alpha = G.alpha[q];
+      int *ie = iexp + parity * ni;
+      // component k of this block: all its loads (y, w, the first neighbours) at once
+      int el = 0, a = 0, b = 0;
+      const SmallItem *I = items;
+      double yv = 0.0, wv = 0.0;
+      double2 x[kSmallPre];
+      const int comp = threadIdx.x & 1;
+      bool live = false;
+      auto fetch = [&](int k) {
+        live = false;
+        if (k >= work) return;
+        const int e = elem[k >> 1];
+        a = (e >> 6) & 63;
+        b = e & 63;
+        if (a >= d) return;
+        live = true;
+        I = items + (e >> 12);
+        el = a * d + b;
+        yv = __ldcg(reinterpret_cast<const double *>(P.y + I->base + el) + comp);
+        wv = __ldcg(reinterpret_cast<const double *>(w + I->base + el) + comp);
+        const double2 *wb = w + I->branch + el;
+        const int nq = I->n_nb;
+#pragma unroll
+        for (int j = 0; j < kSmallPre; ++j)
+          if (j < nq) x[j] = __ldcg(wb + I->e[j].idx);
+      };
+      fetch(threadIdx.x);
+      // limbs of the items' w
+      for (int k = threadIdx.x; k < ((nz + 31) & ~31); k += blockDim.x) {
+        int it = ni - 1, e = 0;
+        if (k < nz) {
+          const int p = place[k];
+          const double2 v = __ldcg(w + z0 + k);
+          it = p >> 20;
+          e = exp_field(v);
+          reinterpret_cast<double2 *>(zs)[p & 0xfffff] = v;
+        }
+        const int il = __shfl_sync(0xffffffffu, it, 0), ih = __shfl_sync(0xffffffffu, it, 31);
+        if (il == ih) {
+          e = __reduce_max_sync(0xffffffffu, e);
+          if (lane == 0) atomicMax(ie + it, e);
+        } else {
+          atomicMax(ie + it, e);
+        }
+      }
+      __syncthreads();
+      for (int k = threadIdx.x; k < nz; k += blockDim.x) {
+        const int p = place[k], e = ie[p >> 20];
+        int4 *z = zs + (p & 0xfffff);
+        const double2 v = *reinterpret_cast<double2 *>(z);
+        const int2 re = to_limbs(v.x, e, O.bits, low), im = to_limbs(v.y, e, O.bits, low);
+        *z = make_int4(re.x, re.y, im.x, im.y);
+      }
+      for (int k = threadIdx.x; k < ni; k += blockDim.x) iexp[(parity ^ 1) * ni + k] = 1;
+      __syncthreads();
+      for (int k = threadIdx.x; k < work; k += blockDim.x) {
+        if (live) {
+          // -i C: the real component takes the commutator's imaginary part, and back
+          const int it = (int)(I - items);
+          const int2 *zb = reinterpret_cast<const int2 *>(zs + it * isz + b) + (comp ^ 1);
+          const int2 *za = reinterpret_cast<const int2 *>(zs + it * isz + a * ld) + (comp ^ 1);
+          const int2 *ha = hs + a * d, *hb = hs + b * d;   // H' is symmetric
+          long long h1 = 0, x1 = 0, h2 = 0, x2 = 0;
+#pragma unroll 4
+          for (int c = 0; c < d; ++c) {
+            const int2 h = ha[c], g = hb[c], z = *zb, t = za[2 * c];
+            zb += 2 * ld;
+            h1 += (long long)h.x * z.x;
+            x1 += (long long)h.x * z.y;
+            x1 += (long long)h.y * z.x;
+            h2 += (long long)g.x * t.x;
+            x2 += (long long)g.x * t.y;
+            x2 += (long long)g.y * t.x;
+          }
+          const Unit f = unit(ie[it], O.hexp, comp ? -O.hsign : O.hsign);
+          const double cm = sum_value(((h1 - h2) << 1) + ((x1 - x2 + (1LL << (low - 2))) >> (low - 1)), f);
+          // acc = -gamma w + sum_s [ +- f_s A_s(other component) + g_s B_s ] +- f C
+          double acc = -I->decay * wv, A = 0.0, B = 0.0;
+          int m = 0;
+          bool any = false, both = false;
+          auto close = [&]() {
+            if (!any) return;
+            const double2 fg = tab[dig[2 * m * d + a] + dig[(2 * m + 1) * d + b]];
+            acc = fma(comp ? -fg.x : fg.x, A, acc);
+            if (both) acc = fma(fg.y, B, acc);
+            any = both = false;
+          };
+          auto entry = [&](int j, const double2 &v) {
+            while (j >= I->off[m + 1]) {
+              close();
+              ++m;
+            }
+            const F64Entry &en = I->e[j];
+            const double o = comp ? v.x : v.y;
+            if (en.kind == 0) {
+              A = any ? A + o : o;
+            } else {
+              A = any ? fma(en.cA, o, A) : en.cA * o;
+              if (en.kind == 2) {
+                const double t = comp ? v.y : v.x;
+                B = both ? fma(en.cB, t, B) : en.cB * t;
+                both = true;
+              }
+            }
+            any = true;
+          };
+          const int nq = I->n_nb;
+#pragma unroll
+          for (int j = 0; j < kSmallPre; ++j)
+            if (j < nq) entry(j, x[j]);
+          for (int j = kSmallPre; j < nq; ++j) entry(j, __ldcg(w + I->branch + I->e[j].idx + el));
+          close();
+          acc = fma(f.f, cm, acc);
+          __stcg(reinterpret_cast<double *>(out + I->base + el) + comp, fma(alpha, acc, yv));
+        }
+        fetch(k + blockDim.x);
+      }
+      if (kSync == 0)
+        __syncthreads();
+      else if (kSync == 1)
+        cg::this_cluster().sync();
+      else
+        cg::this_grid().sync();
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Basis change along one index of every ADO, mode by mode, a panel of 32 columns
 // (left: the row index) or rows (right) in shared memory; each thread transforms one
 // fibre of n_s values in registers: 6 n_s products per element and side instead of the
@@ -577,6 +819,77 @@ __global__ void __launch_bounds__(256) rotate_kernel(const Tin *x, Tout *out, co
       store((int64_t)p0 * d + k, v[(k - a * d) * kRotPad + a], (int)lsum[a], lexp[a] < 0x7ff);
     }
   }
+}
+
+// Both sides at once for small bases: one item per block in shared memory, one scale
+// for it (its Frobenius norm).  Two launches of the panel kernels are ~17 us however
+// small the state is.
+template <typename Tin, typename Tout>
+__global__ void __launch_bounds__(256) rotate_item_kernel(const Tin *x, Tout *out, const int2 *__restrict__ u,
+                                                          const __grid_constant__ RotOps r) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  longlong2 *v = reinterpret_cast<longlong2 *>(smem);   // [d][d | 1]
+  __shared__ int s_exp;
+  __shared__ unsigned s_sum;
+  const int d = r.d, ld = d | 1, dd = d * d;
+  const Tin *xi = x + (int64_t)blockIdx.x * dd;
+  if (threadIdx.x == 0) {
+    s_exp = 1;
+    s_sum = 0;
+  }
+  __syncthreads();
+  int e = 0;
+  for (int k = threadIdx.x; k < dd; k += blockDim.x) {
+    const Tin t = xi[k];
+    const double2 z = make_double2((double)t.x, (double)t.y);
+    e = max(e, exp_field(z));
+    reinterpret_cast<double2 *>(v)[(k / d) * ld + k % d] = z;
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((threadIdx.x & 31) == 0) atomicMax(&s_exp, e);
+  __syncthreads();
+  const int e1 = s_exp;
+  unsigned q = 0;
+  for (int k = threadIdx.x; k < dd; k += blockDim.x) {
+    const double2 t = reinterpret_cast<double2 *>(v)[(k / d) * ld + k % d];
+    const int2 re = to_limbs(t.x, e1, 60, 30), im = to_limbs(t.y, e1, 60, 30);
+    const float a = (float)(abs(re.x) + 1) * (1.f / (1 << 29)), b = (float)(abs(im.x) + 1) * (1.f / (1 << 29));
+    q += (unsigned)((a * a + b * b) * 262144.f) + 2u;   // up to 1024 elements: below 2^30
+  }
+  atomicAdd(&s_sum, q);
+  __syncthreads();
+  const int lg = 32 - __clz(s_sum);
+  const int en = e1 + (lg > 18 ? (lg - 17) / 2 : 0);
+  for (int k = threadIdx.x; k < dd; k += blockDim.x) {
+    longlong2 *p = v + (k / d) * ld + k % d;
+    const double2 t = *reinterpret_cast<double2 *>(p);
+    *p = make_longlong2(to_fixed59(t.x, en), to_fixed59(t.y, en));
+  }
+  for (int side = 0; side < 2; ++side)
+    for (int s = 0; s < r.n_modes; ++s) {
+      __syncthreads();
+      const int n = r.dims[s], str = r.stride[s];
+      const int2 *us = u + r.off[s];
+      for (int k = threadIdx.x; k < dd / n; k += blockDim.x) {
+        const int f = side == 0 ? k / d : k % (d / n), o = side == 0 ? k % d : k / (d / n);
+        const int base = (f / str) * str * n + f % str;
+        longlong2 *p = side == 0 ? v + base * ld + o : v + o * ld + base;
+        const int ps = side == 0 ? str * ld : str;
+        switch (n) {
+          case 2: rotate_fibre<2>(p, us, ps); break;
+          case 3: rotate_fibre<3>(p, us, ps); break;
+          case 4: rotate_fibre<4>(p, us, ps); break;
+          case 5: rotate_fibre<5>(p, us, ps); break;
+          case 6: rotate_fibre<6>(p, us, ps); break;
+          case 7: rotate_fibre<7>(p, us, ps); break;
+          case 8: rotate_fibre<8>(p, us, ps); break;
+          default: break;
+        }
+      }
+    }
+  __syncthreads();
+  for (int k = threadIdx.x; k < dd; k += blockDim.x)
+    out[(int64_t)blockIdx.x * dd + k] = from_fixed59<Tout>(v[(k / d) * ld + k % d], en, e1 < 0x7ff);
 }
 
 template <typename T>
@@ -838,6 +1151,12 @@ F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::
                                   (M.vb_lam[s][a] + M.vb_lam[s][b]) + (M.vb_lam_lo[s][a] + M.vb_lam_lo[s][b])));
     for (int a = 0; a < d; ++a) dig[(size_t)s * d + a] = (uint16_t)((a / M.stride[s]) % M.dims[s]);
   }
+  if (d <= kSmallD) {
+    std::vector<int2> hd((size_t)d * d);
+    for (int a = 0; a < d; ++a)
+      for (int c = 0; c < d; ++c) hd[(size_t)a * d + c] = digits_differ(M, a, c) <= 2 ? limbs(a, c) : make_int2(0, 0);
+    O.hd = up(hd, allocs);
+  }
   O.foff = up(foff, allocs);
   O.fc = up(fc, allocs);
   O.fh = up(fh, allocs);
@@ -870,6 +1189,181 @@ void f64_stage(const F64Buf &b, double alpha, int threads, cudaStream_t st) {
   a.one = make_set(b, 0, &fused, &smem, &blocks);
   a.alpha = alpha;
   launch(a, b.ops->R, fused, blocks, smem, threads, st);
+}
+
+namespace {
+
+struct SmallShape {
+  int sync = 0, blocks = 0, threads = 0, cluster = 1;
+  size_t smem = 0;
+};
+
+int sm_count() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
+// Elements per block up to which a launch for all steps wins: beyond it a stage's own
+// work (20-26 FP64 operations per element, two per clock and SM) exceeds what a launch
+// per stage costs, and the whole-item kernel, which multiplies only H''s non-zeros over
+// the whole GPU, takes over.
+constexpr int kSmallElems = 1536;
+
+bool small_fit(F64SmallSet &p, SmallShape &sh) {
+  const F64Ops &O = p.O;
+  const int dd = O.d * O.d;
+  const int64_t n_units = (sh.sync == 2 ? p.branches : 1) * (int64_t)O.n_ado * p.parts;
+  p.units = (int)std::min<int64_t>((n_units + p.bpb - 1) / p.bpb, 1 << 20);
+  if (sh.sync == 2) p.bpb = (int)((n_units + p.units - 1) / p.units);
+  const int64_t max_items = (p.units + p.parts - 1) / p.parts + (p.parts > 1 ? 1 : 0);
+  const int64_t work = (int64_t)p.units * dd / p.parts;
+  const int rows = (O.d + p.parts - 1) / p.parts;
+  const int64_t smem = O.tab * 16 + max_items * ((int64_t)O.d * (O.d | 1) * 16 + sizeof(SmallItem) + 8 + dd * 4) + dd * 8 +
+                       2 * O.n_modes * O.d * 4 + (int64_t)p.units * rows * O.d * 4;
+  if (work > kSmallElems || smem > (int64_t)kMaxSmem - 1024 || n_units * dd > (1 << 30)) return false;
+  sh.smem = std::max(sh.smem, (size_t)smem);
+  sh.threads = std::max(sh.threads, work <= 32 ? 64 : work <= 64 ? 128 : work <= 256 ? 256 : 512);
+  sh.blocks += sh.sync == 2 ? p.bpb : p.branches * p.bpb;
+  return true;
+}
+
+// How the steps of one hierarchy's branches run as one launch; false: they do not.
+bool small_shape(F64SmallSet &p, SmallShape &sh) {
+  if (!p.O.hd || p.branches < 1) return false;
+  const int sms = sm_count(), B = p.branches;
+  const int64_t elems = (int64_t)p.O.n_ado * p.O.d * p.O.d;
+  p.parts = 1;
+  int c = 1;
+  while (c < 16 && 2 * c * (int64_t)B <= sms && c < p.O.n_ado) c *= 2;
+  p.bpb = sh.cluster = c;
+  sh.sync = c > 1 ? 1 : 0;
+  // a cluster reaches 16 SMs; a few larger branches spread over the whole grid instead
+  if (B * (int64_t)c * 3 < 2 * sms && elems / c > 256) {
+    sh.sync = 2;
+    const int64_t items = (int64_t)B * p.O.n_ado;
+    p.parts = (int)std::max<int64_t>(1, std::min<int64_t>(4, sms / items));
+    p.bpb = (int)std::min<int64_t>(sms, items * p.parts);
+  }
+  return small_fit(p, sh);
+}
+
+template <bool kMulti>
+bool launch_small(const F64SmallArgs &a, const SmallShape &sh, cudaStream_t st) {
+  auto kernel = sh.sync == 0 ? f64_small_kernel<0, kMulti> : f64_small_kernel<1, kMulti>;
+  if constexpr (!kMulti)
+    if (sh.sync == 2) kernel = f64_small_kernel<2, false>;
+  allow_smem(kernel, sh.smem);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)sh.blocks);
+  cfg.blockDim = dim3((unsigned)sh.threads);
+  cfg.dynamicSmemBytes = sh.smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  cfg.attrs = &at;
+  if (sh.sync == 1) {
+    if (sh.cluster > 8) cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)sh.cluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
+      (void)cudaGetLastError();
+      return false;
+    }
+  } else if (sh.sync == 2) {
+    at.id = cudaLaunchAttributeCooperative;
+    at.val.cooperative = 1;
+    cfg.numAttrs = 1;
+  }
+  if (cudaLaunchKernelEx(&cfg, kernel, a) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  count_launch(1);
+  return true;
+}
+
+}  // namespace
+
+bool f64_small_steps(const F64Ops &O, double2 *y, double2 *wa, double2 *wb, int branches, double dt, int64_t steps,
+                     cudaStream_t st, std::pair<int, int> *shape) {
+  F64SmallArgs a{};
+  SmallShape sh;
+  a.one.O = O;
+  a.one.y = y;
+  a.one.wa = wa;
+  a.one.wb = wb;
+  a.one.branches = branches;
+  for (int q = 0; q < 4; ++q) a.alpha[q] = dt / (4 - q);
+  a.steps = steps;
+  if (!small_shape(a.one, sh) || !launch_small<false>(a, sh, st)) return false;
+  if (shape) *shape = {sh.threads, sh.blocks};
+  return true;
+}
+
+F64SmallPlan::~F64SmallPlan() {
+  if (desc) cudaFree(desc);
+}
+
+void f64_small_plan(F64SmallPlan &p, const std::vector<F64SmallBuf> &sets, cudaStream_t st) {
+  std::vector<F64SmallSet> v;
+  SmallShape sh;
+  const int sms = sm_count();
+  int64_t total = 0;
+  int least = 1 << 30;
+  for (const F64SmallBuf &b : sets) {
+    if (!b.ops->hd) return;
+    total += b.branches;
+    least = std::min(least, b.ops->n_ado);
+  }
+  // one cluster size for all sets; no row ranges and no grid-wide barrier here
+  while (sh.cluster < 16 && 2 * sh.cluster * total <= sms && sh.cluster < least) sh.cluster *= 2;
+  sh.sync = sh.cluster > 1 ? 1 : 0;
+  for (const F64SmallBuf &b : sets) {
+    F64SmallSet s{};
+    s.O = *b.ops;
+    s.y = b.y;
+    s.wa = b.wa;
+    s.wb = b.wb;
+    s.branches = b.branches;
+    s.parts = 1;
+    s.bpb = sh.cluster;
+    s.begin = sh.blocks;
+    if (!small_fit(s, sh)) return;
+    v.push_back(s);
+  }
+  if (device_malloc(&p.desc, v.size() * sizeof(F64SmallSet)) != cudaSuccess) {
+    p.desc = nullptr;
+    (void)cudaGetLastError();
+    throw DeviceOom();
+  }
+  cudaMemcpyAsync(p.desc, v.data(), v.size() * sizeof(F64SmallSet), cudaMemcpyHostToDevice, st);
+  cudaStreamSynchronize(st);
+  p.n = (int)v.size();
+  p.sync = sh.sync;
+  p.blocks = sh.blocks;
+  p.threads = sh.threads;
+  p.cluster = sh.cluster;
+  p.smem = sh.smem;
+}
+
+bool f64_small_steps_plan(const F64SmallPlan &p, double dt, int64_t steps, cudaStream_t st) {
+  if (!p.desc) return false;
+  F64SmallArgs a{};
+  a.many = (const F64SmallSet *)p.desc;
+  a.n = p.n;
+  for (int q = 0; q < 4; ++q) a.alpha[q] = dt / (4 - q);
+  a.steps = steps;
+  SmallShape sh;
+  sh.sync = p.sync;
+  sh.blocks = p.blocks;
+  sh.threads = p.threads;
+  sh.cluster = p.cluster;
+  sh.smem = p.smem;
+  return launch_small<true>(a, sh, st);
 }
 
 F64Plan::~F64Plan() {
@@ -958,6 +1452,13 @@ void rotate(const RotOps &r, bool forward, const Tin *x, Tout *out, double2 *tmp
   const int64_t blocks = items * panels;
   if (blocks > 0x7fffffffLL) throw std::invalid_argument("too many work items for one launch");
   const int2 *u = forward ? r.fwd : r.bwd;
+  if (r.d <= kSmallD) {
+    const int dd = r.d * r.d;
+    rotate_item_kernel<Tin, Tout><<<(unsigned)items, dd <= 64 ? 64 : dd <= 128 ? 128 : 256, r.d * (r.d | 1) * 16, st>>>(
+        x, out, u, r);
+    count_launch(1);
+    return;
+  }
   const size_t smem = (size_t)r.d * kRotPad * 16;
   allow_smem(rotate_kernel<Tin, double2, false>, smem);
   allow_smem(rotate_kernel<double2, Tout, true>, smem);

@@ -47,6 +47,7 @@ struct F64Ops {
   const F64Entry *nb = nullptr;
   const double *decay = nullptr;  // [n_ado]
   const double2 *fg = nullptr;    // (lam_a - lam_b, lam_a + lam_b) per digit pair, mode after mode
+  const int2 *hd = nullptr;       // limbs of H', dense (small bases)
   const uint16_t *dig = nullptr;  // [n_modes][d] digit of mode s
 };
 
@@ -72,6 +73,31 @@ F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::
 // first, and the stage with one of them (the result does not depend on it).
 std::vector<std::pair<int, int>> f64_shapes(const F64Buf &b);
 void f64_stage(const F64Buf &b, double alpha, int threads, cudaStream_t st);
+
+// steps RK4 steps (Horner form) of branches in one launch, for hierarchies small enough
+// that a launch per stage would cost more than the stage; false if this one is not, or
+// the launch is not possible (nothing has run then).  shape receives the launch's
+// threads per block and blocks.
+bool f64_small_steps(const F64Ops &O, double2 *y, double2 *wa, double2 *wb, int branches, double dt, int64_t steps,
+                     cudaStream_t st, std::pair<int, int> *shape);
+
+// The same for several hierarchies (empty desc: they do not all fit).
+struct F64SmallBuf {
+  const F64Ops *ops;
+  double2 *y, *wa, *wb;
+  int branches;
+};
+struct F64SmallPlan {
+  void *desc = nullptr;
+  int n = 0, sync = 0, blocks = 0, threads = 0, cluster = 1;
+  size_t smem = 0;
+  F64SmallPlan() = default;
+  ~F64SmallPlan();
+  F64SmallPlan(const F64SmallPlan &) = delete;
+  F64SmallPlan &operator=(const F64SmallPlan &) = delete;
+};
+void f64_small_plan(F64SmallPlan &p, const std::vector<F64SmallBuf> &sets, cudaStream_t st);
+bool f64_small_steps_plan(const F64SmallPlan &p, double dt, int64_t steps, cudaStream_t st);
 
 // One stage of several hierarchies: a plan (device descriptors) per set of buffers.
 struct F64Plan {
