@@ -158,7 +158,7 @@ void work_in(heom_hier *h, const double2 *x, double2 *out, double2 *tmp, int bra
   if (!h->f64.ready) {
     if (x != out) CUDA_TRY(cudaMemcpyAsync(out, x, elems * 16, cudaMemcpyDeviceToDevice, st));
   } else if (h->rot.ready) {
-    rotate<double2, double2>(h->rot, true, x, out, tmp, items, st);
+    rotate(h->rot, true, x, out, tmp, items, st);
   } else {
     sim_left_kernel<double2><<<grid_for(elems), 256, 0, st>>>(x, tmp, h->U64, h->M.d, elems);
     sim_right_kernel<double2><<<grid_for(elems), 256, 0, st>>>(tmp, out, h->U64, h->M.d, elems);
@@ -172,7 +172,7 @@ void work_out(heom_hier *h, const double2 *x, double2 *out, double2 *tmp, int br
   if (!h->f64.ready) {
     if (x != out) CUDA_TRY(cudaMemcpyAsync(out, x, elems * 16, cudaMemcpyDeviceToDevice, st));
   } else if (h->rot.ready) {
-    rotate<double2, double2>(h->rot, false, x, out, tmp, items, st);
+    rotate(h->rot, false, x, out, tmp, items, st);
   } else {
     sim_left_kernel<double2><<<grid_for(elems), 256, 0, st>>>(x, tmp, h->UT64, h->M.d, elems);
     sim_right_kernel<double2><<<grid_for(elems), 256, 0, st>>>(tmp, out, h->UT64, h->M.d, elems);
@@ -311,29 +311,22 @@ void trace_into(heom_hier *h, const typename CxT<R>::type *w, int branches, cons
 // ---------------------------------------------------------------------------
 
 
-// Original-basis complex128 ADOs -> coupling-basis complex64 (U^T x U), and back.
+// Original-basis complex128 ADOs -> coupling-basis complex64 (U^T x U), and back; the
+// dense FP64 product, so that complex64 states keep their bits.
 void to_coupling_basis(heom_hier *h, const double2 *x, float2 *out, int64_t elems, cudaStream_t st) {
   DeviceBuffer tmp(elems * 16);
-  if (h->rot.ready) {
-    rotate<double2, float2>(h->rot, true, x, out, (double2 *)tmp.p, elems / ((int64_t)h->M.d * h->M.d), st);
-  } else {
-    sim_left_kernel<double2><<<grid_for(elems), 256, 0, st>>>(x, (double2 *)tmp.p, h->U64, h->M.d, elems);
-    sim_right_kernel<float2><<<grid_for(elems), 256, 0, st>>>((const double2 *)tmp.p, out, h->U64, h->M.d, elems);
-    count_launch(2);
-  }
+  sim_left_kernel<double2><<<grid_for(elems), 256, 0, st>>>(x, (double2 *)tmp.p, h->U64, h->M.d, elems);
+  sim_right_kernel<float2><<<grid_for(elems), 256, 0, st>>>((const double2 *)tmp.p, out, h->U64, h->M.d, elems);
+  count_launch(2);
   LAUNCH_CHECK();
   CUDA_TRY(cudaStreamSynchronize(st));
 }
 
 static void from_coupling_basis(heom_hier *h, const float2 *x, double2 *out, int64_t elems, cudaStream_t st) {
   DeviceBuffer tmp(elems * 16);
-  if (h->rot.ready) {
-    rotate<float2, double2>(h->rot, false, x, out, (double2 *)tmp.p, elems / ((int64_t)h->M.d * h->M.d), st);
-  } else {
-    sim_left_kernel<float2><<<grid_for(elems), 256, 0, st>>>(x, (double2 *)tmp.p, h->UT64, h->M.d, elems);
-    sim_right_kernel<double2><<<grid_for(elems), 256, 0, st>>>((const double2 *)tmp.p, out, h->UT64, h->M.d, elems);
-    count_launch(2);
-  }
+  sim_left_kernel<float2><<<grid_for(elems), 256, 0, st>>>(x, (double2 *)tmp.p, h->UT64, h->M.d, elems);
+  sim_right_kernel<double2><<<grid_for(elems), 256, 0, st>>>((const double2 *)tmp.p, out, h->UT64, h->M.d, elems);
+  count_launch(2);
   LAUNCH_CHECK();
   CUDA_TRY(cudaStreamSynchronize(st));
 }
@@ -513,8 +506,6 @@ void ensure_device(heom_hier *h) {
   h->U64 = h->up(M.vb_U);
   h->UT64 = h->up(UT);
   h->mu_vb64 = h->up(M.vb_mu);
-  h->mup_vb64 = h->up(M.vb_mu_plus);
-  h->mum_vb64 = h->up(mumv);
   h->mu_vb32 = h->up(cast_vec<float>(M.vb_mu));
   h->mup_vb32 = h->up(cast_vec<float>(M.vb_mu_plus));
   h->mum_vb32 = h->up(cast_vec<float>(mumv));
@@ -534,7 +525,16 @@ void ensure_device(heom_hier *h) {
   vb.nb_cB = d32.nb_cB;
   h->vb = vb;
   if (rot_supported(M)) h->rot = rot_build(M, h->allocs);
-  if (f64_supported(M)) h->f64 = f64_build(M, M.nb_off, M.nb_idx, M.nb_cA, M.nb_cB, 1.0, h->allocs);
+  if (f64_supported(M)) {
+    h->f64 = f64_build(M, M.nb_off, M.nb_idx, M.nb_cA, M.nb_cB, 1.0, h->allocs);
+    const std::vector<double> mp = f64_matrix(M, M.mu_plus);
+    std::vector<double> mm(mp.size());
+    for (int a = 0; a < M.d; ++a)
+      for (int b = 0; b < M.d; ++b) mm[(size_t)a * M.d + b] = mp[(size_t)b * M.d + a];
+    h->mu_w64 = h->up(f64_matrix(M, M.mu));
+    h->mup_w64 = h->up(mp);
+    h->mum_w64 = h->up(mm);
+  }
   if (M.precision == HEOM_TC) tc_build(h->tc, M, h->vb, h->allocs);
   // the table uploads above are complete before any launch on any stream
   CUDA_TRY(cudaDeviceSynchronize());

@@ -677,18 +677,14 @@ __device__ __forceinline__ long long to_fixed59(double x, int emax) {
 }
 
 // t 2^(e - 1081), in two factors where one would leave the exponent range; NaN if not finite.
-template <typename T>
-__device__ __forceinline__ T from_fixed59(const longlong2 &t, int e, bool finite) {
+__device__ __forceinline__ double2 from_fixed59(const longlong2 &t, int e, bool finite) {
   const double f = __longlong_as_double(finite ? (long long)(e > 58 ? e - 58 : e + 964) << 52 : 0x7ff8000000000000LL);
   double re = __ll2double_rn(t.x) * f, im = __ll2double_rn(t.y) * f;
   if (e <= 58) {
     re *= __longlong_as_double(1LL << 52);
     im *= __longlong_as_double(1LL << 52);
   }
-  T o;
-  o.x = re;
-  o.y = im;
-  return o;
+  return make_double2(re, im);
 }
 
 // One fibre of N values, str apart.
@@ -727,8 +723,8 @@ __device__ __forceinline__ void rotate_fibres(longlong2 *v, const int2 *__restri
     rotate_fibre<N>(v + ((f / str) * str * N + f % str) * kRotPad, u, str * kRotPad);
 }
 
-template <typename Tin, typename Tout, bool kRight>
-__global__ void __launch_bounds__(256) rotate_kernel(const Tin *x, Tout *out, const int2 *__restrict__ u, const __grid_constant__ RotOps r,
+template <bool kRight>
+__global__ void __launch_bounds__(256) rotate_kernel(const double2 *x, double2 *out, const int2 *__restrict__ u, const __grid_constant__ RotOps r,
                                                      int panels) {
   extern __shared__ __align__(16) uint8_t smem[];
   longlong2 *v = reinterpret_cast<longlong2 *>(smem);   // [d][33], second index along the panel
@@ -737,7 +733,7 @@ __global__ void __launch_bounds__(256) rotate_kernel(const Tin *x, Tout *out, co
   const int d = r.d;
   const int64_t item = blockIdx.x / panels;
   const int p0 = (int)(blockIdx.x - item * panels) * 32, np = min(32, d - p0);
-  const Tin *xi = x + item * d * d;
+  const double2 *xi = x + item * d * d;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   if (threadIdx.x < 32) {
     lexp[lane] = 1;
@@ -745,15 +741,12 @@ __global__ void __launch_bounds__(256) rotate_kernel(const Tin *x, Tout *out, co
   }
   if (!kRight) {
     if (lane < np)
-      for (int c = warp; c < d; c += warps) {
-        const Tin t = xi[(int64_t)c * d + p0 + lane];
-        reinterpret_cast<double2 *>(v)[c * kRotPad + lane] = make_double2((double)t.x, (double)t.y);
-      }
+      for (int c = warp; c < d; c += warps)
+        reinterpret_cast<double2 *>(v)[c * kRotPad + lane] = xi[(int64_t)c * d + p0 + lane];
   } else {
     for (int k = threadIdx.x; k < np * d; k += blockDim.x) {
-      const Tin t = xi[(int64_t)p0 * d + k];
       const int a = k / d;
-      reinterpret_cast<double2 *>(v)[(k - a * d) * kRotPad + a] = make_double2((double)t.x, (double)t.y);
+      reinterpret_cast<double2 *>(v)[(k - a * d) * kRotPad + a] = xi[(int64_t)p0 * d + k];
     }
   }
   __syncthreads();
@@ -806,8 +799,8 @@ __global__ void __launch_bounds__(256) rotate_kernel(const Tin *x, Tout *out, co
     }
   }
   __syncthreads();
-  Tout *oi = out + item * d * d;
-  auto store = [&](int64_t at, const longlong2 &t, int e, bool finite) { oi[at] = from_fixed59<Tout>(t, e, finite); };
+  double2 *oi = out + item * d * d;
+  auto store = [&](int64_t at, const longlong2 &t, int e, bool finite) { oi[at] = from_fixed59(t, e, finite); };
   if (!kRight) {
     if (lane < np)
       for (int c = warp; c < d; c += warps) store((int64_t)c * d + p0 + lane, v[c * kRotPad + lane], en, e1 < 0x7ff);
@@ -824,15 +817,14 @@ __global__ void __launch_bounds__(256) rotate_kernel(const Tin *x, Tout *out, co
 // Both sides at once for small bases: one item per block in shared memory, one scale
 // for it (its Frobenius norm).  Two launches of the panel kernels are ~17 us however
 // small the state is.
-template <typename Tin, typename Tout>
-__global__ void __launch_bounds__(256) rotate_item_kernel(const Tin *x, Tout *out, const int2 *__restrict__ u,
+__global__ void __launch_bounds__(256) rotate_item_kernel(const double2 *x, double2 *out, const int2 *__restrict__ u,
                                                           const __grid_constant__ RotOps r) {
   extern __shared__ __align__(16) uint8_t smem[];
   longlong2 *v = reinterpret_cast<longlong2 *>(smem);   // [d][d | 1]
   __shared__ int s_exp;
   __shared__ unsigned s_sum;
   const int d = r.d, ld = d | 1, dd = d * d;
-  const Tin *xi = x + (int64_t)blockIdx.x * dd;
+  const double2 *xi = x + (int64_t)blockIdx.x * dd;
   if (threadIdx.x == 0) {
     s_exp = 1;
     s_sum = 0;
@@ -840,8 +832,7 @@ __global__ void __launch_bounds__(256) rotate_item_kernel(const Tin *x, Tout *ou
   __syncthreads();
   int e = 0;
   for (int k = threadIdx.x; k < dd; k += blockDim.x) {
-    const Tin t = xi[k];
-    const double2 z = make_double2((double)t.x, (double)t.y);
+    const double2 z = xi[k];
     e = max(e, exp_field(z));
     reinterpret_cast<double2 *>(v)[(k / d) * ld + k % d] = z;
   }
@@ -889,7 +880,7 @@ __global__ void __launch_bounds__(256) rotate_item_kernel(const Tin *x, Tout *ou
     }
   __syncthreads();
   for (int k = threadIdx.x; k < dd; k += blockDim.x)
-    out[(int64_t)blockIdx.x * dd + k] = from_fixed59<Tout>(v[(k / d) * ld + k % d], en, e1 < 0x7ff);
+    out[(int64_t)blockIdx.x * dd + k] = from_fixed59(v[(k / d) * ld + k % d], en, e1 < 0x7ff);
 }
 
 template <typename T>
@@ -932,11 +923,11 @@ struct DD {
   }
 };
 
-// H' = U^T H U, mode by mode, to about 32 digits.
-std::vector<DD> coupling_h(const Model &M) {
+// X' = U^T X U, mode by mode, to about 32 digits.
+std::vector<DD> coupling_matrix(const Model &M, const std::vector<double> &X) {
   const int d = M.d;
   std::vector<DD> A((size_t)d * d), v;
-  for (size_t i = 0; i < A.size(); ++i) A[i].h = M.H[i];
+  for (size_t i = 0; i < A.size(); ++i) A[i].h = X[i];
   for (int side = 0; side < 2; ++side)
     for (int s = 0; s < M.n_modes; ++s) {
       const int n = M.dims[s], str = M.stride[s];
@@ -951,7 +942,7 @@ std::vector<DD> coupling_h(const Model &M) {
           for (int i = 0; i < n; ++i) {
             DD acc;
             for (int k = 0; k < n; ++k)
-              acc.add_product(DD{M.vb_Us[s][(size_t)k * n + i], M.vb_Us_lo[s][(size_t)k * n + i]}, v[k]);
+              acc.add_product(DD{M.cb_U[s][(size_t)k * n + i], M.cb_U_lo[s][(size_t)k * n + i]}, v[k]);
             at(i) = acc;
           }
         }
@@ -1061,6 +1052,13 @@ bool f64_supported(const Model &M) {
   return true;
 }
 
+std::vector<double> f64_matrix(const Model &M, const std::vector<double> &X) {
+  const std::vector<DD> A = coupling_matrix(M, X);
+  std::vector<double> r(A.size());
+  for (size_t i = 0; i < r.size(); ++i) r[i] = A[i].h;
+  return r;
+}
+
 F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::vector<int32_t> &nb_idx,
                  const std::vector<double> &nb_cA, const std::vector<double> &nb_cB, double hsign,
                  std::vector<void *> &allocs) {
@@ -1076,7 +1074,7 @@ F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::
   // H' shifted by the middle of its diagonal (the commutator does not change; smaller
   // entries, smaller rounding of the limbs) and scaled by a power of two so that the
   // absolute sum of a row stays below 1: with |w| < 1 the integer sums cannot overflow.
-  std::vector<DD> Hc = coupling_h(M);
+  std::vector<DD> Hc = coupling_matrix(M, M.H);
   double lo = Hc[0].h, hi = lo;
   for (int a = 0; a < d; ++a) {
     lo = std::min(lo, Hc[(size_t)a * d + a].h);
@@ -1147,8 +1145,8 @@ F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::
     O.tab_off[s] = (int)fg.size();
     for (int a = 0; a < M.dims[s]; ++a)
       for (int b = 0; b < M.dims[s]; ++b)   // lam_a -+ lam_b, rounded once
-        fg.push_back(make_double2((M.vb_lam[s][a] - M.vb_lam[s][b]) + (M.vb_lam_lo[s][a] - M.vb_lam_lo[s][b]),
-                                  (M.vb_lam[s][a] + M.vb_lam[s][b]) + (M.vb_lam_lo[s][a] + M.vb_lam_lo[s][b])));
+        fg.push_back(make_double2((M.cb_lam[s][a] - M.cb_lam[s][b]) + (M.cb_lam_lo[s][a] - M.cb_lam_lo[s][b]),
+                                  (M.cb_lam[s][a] + M.cb_lam[s][b]) + (M.cb_lam_lo[s][a] + M.cb_lam_lo[s][b])));
     for (int a = 0; a < d; ++a) dig[(size_t)s * d + a] = (uint16_t)((a / M.stride[s]) % M.dims[s]);
   }
   if (d <= kSmallD) {
@@ -1423,7 +1421,7 @@ RotOps rot_build(const Model &M, std::vector<void *> &allocs) {
   for (int s = 0; s < M.n_modes; ++s) {
     const int n = M.dims[s];
     auto limbs = [&](int k, int i) {
-      const double h = std::ldexp(M.vb_Us[s][(size_t)k * n + i], 59), l = std::ldexp(M.vb_Us_lo[s][(size_t)k * n + i], 59);
+      const double h = std::ldexp(M.cb_U[s][(size_t)k * n + i], 59), l = std::ldexp(M.cb_U_lo[s][(size_t)k * n + i], 59);
       const long long v0 = std::llrint(h), v = v0 + std::llrint(h - (double)v0 + l);
       int2 c;
       c.y = (int)((unsigned)(unsigned long long)v << 2) >> 2;
@@ -1445,8 +1443,7 @@ RotOps rot_build(const Model &M, std::vector<void *> &allocs) {
   return r;
 }
 
-template <typename Tin, typename Tout>
-void rotate(const RotOps &r, bool forward, const Tin *x, Tout *out, double2 *tmp, int64_t items, cudaStream_t st) {
+void rotate(const RotOps &r, bool forward, const double2 *x, double2 *out, double2 *tmp, int64_t items, cudaStream_t st) {
   if (items <= 0) return;
   const int panels = (r.d + 31) / 32;
   const int64_t blocks = items * panels;
@@ -1454,21 +1451,18 @@ void rotate(const RotOps &r, bool forward, const Tin *x, Tout *out, double2 *tmp
   const int2 *u = forward ? r.fwd : r.bwd;
   if (r.d <= kSmallD) {
     const int dd = r.d * r.d;
-    rotate_item_kernel<Tin, Tout><<<(unsigned)items, dd <= 64 ? 64 : dd <= 128 ? 128 : 256, r.d * (r.d | 1) * 16, st>>>(
+    rotate_item_kernel<<<(unsigned)items, dd <= 64 ? 64 : dd <= 128 ? 128 : 256, r.d * (r.d | 1) * 16, st>>>(
         x, out, u, r);
     count_launch(1);
     return;
   }
   const size_t smem = (size_t)r.d * kRotPad * 16;
-  allow_smem(rotate_kernel<Tin, double2, false>, smem);
-  allow_smem(rotate_kernel<double2, Tout, true>, smem);
-  rotate_kernel<Tin, double2, false><<<(unsigned)blocks, 256, smem, st>>>(x, tmp, u, r, panels);
-  rotate_kernel<double2, Tout, true><<<(unsigned)blocks, 256, smem, st>>>(tmp, out, u, r, panels);
+  allow_smem(rotate_kernel<false>, smem);
+  allow_smem(rotate_kernel<true>, smem);
+  rotate_kernel<false><<<(unsigned)blocks, 256, smem, st>>>(x, tmp, u, r, panels);
+  rotate_kernel<true><<<(unsigned)blocks, 256, smem, st>>>(tmp, out, u, r, panels);
   count_launch(2);
 }
 
-template void rotate<double2, double2>(const RotOps &, bool, const double2 *, double2 *, double2 *, int64_t, cudaStream_t);
-template void rotate<double2, float2>(const RotOps &, bool, const double2 *, float2 *, double2 *, int64_t, cudaStream_t);
-template void rotate<float2, double2>(const RotOps &, bool, const float2 *, double2 *, double2 *, int64_t, cudaStream_t);
 
 }  // namespace heom

@@ -129,9 +129,9 @@ struct RotOps {
 };
 bool rot_supported(const Model &M);
 RotOps rot_build(const Model &M, std::vector<void *> &allocs);
-// tmp: scratch of the same element count (complex128); may equal x if x is complex128
-// and may be overwritten.  out may equal x.
-template <typename Tin, typename Tout>
-void rotate(const RotOps &r, bool forward, const Tin *x, Tout *out, double2 *tmp, int64_t items, cudaStream_t st);
+// tmp: scratch of the same element count; out may equal x.
+void rotate(const RotOps &r, bool forward, const double2 *x, double2 *out, double2 *tmp, int64_t items, cudaStream_t st);
+// U^T X U of a d x d matrix of the model, rounded once.
+std::vector<double> f64_matrix(const Model &M, const std::vector<double> &X);
 
 }  // namespace heom

@@ -131,7 +131,8 @@ struct heom_hier {
   VbModel vb{};                 // coupling-eigenbasis model (FP32 paths)
   double *U64 = nullptr, *UT64 = nullptr;        // coupling eigenbasis U and U^T
   float *mu_vb32 = nullptr, *mup_vb32 = nullptr, *mum_vb32 = nullptr;
-  double *mu_vb64 = nullptr, *mup_vb64 = nullptr, *mum_vb64 = nullptr;   // mu, mu+, mu- there
+  double *mu_vb64 = nullptr;                     // mu in the coupling basis (traces of complex64 states)
+  double *mu_w64 = nullptr, *mup_w64 = nullptr, *mum_w64 = nullptr;   // mu, mu+, mu- there (FP64 path)
   // FP64 propagation in the coupling basis (f64.ready), and the basis change mode by mode
   F64Ops f64{}, f64_adj{};
   RotOps rot{};
@@ -219,13 +220,13 @@ const R *mu_work(heom_hier *h, int which);
 template <>
 inline const double *mu_work<double>(heom_hier *h, int which) {
   if (!h->f64.ready) return mu_of<double>(h, which);
-  return which == 0 ? h->mu_vb64 : which == 1 ? h->mup_vb64 : h->mum_vb64;
+  return which == 0 ? h->mu_w64 : which == 1 ? h->mup_w64 : h->mum_w64;
 }
 template <>
 inline const float *mu_work<float>(heom_hier *h, int which) { return mu_of<float>(h, which); }
 template <typename R>
 const double *mu_trace_work(heom_hier *h) {
-  return sizeof(R) == 8 && !h->f64.ready ? h->mu_trace : h->mu_vb64;
+  return sizeof(R) == 4 ? h->mu_vb64 : h->f64.ready ? h->mu_w64 : h->mu_trace;
 }
 // Product basis -> working basis and back (tmp: scratch of the same size; out may
 // equal x).

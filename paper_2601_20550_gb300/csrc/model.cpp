@@ -407,30 +407,27 @@ void build_coupling_basis(Model &M) {
   const int d = M.d;
   std::vector<std::vector<double>> Us;
   M.vb_lam.clear();
-  M.vb_Us_lo.clear();
-  M.vb_lam_lo.clear();
+  for (auto *v : {&M.cb_lam, &M.cb_lam_lo, &M.cb_U, &M.cb_U_lo}) v->clear();
   for (int s = 0; s < M.n_modes; ++s) {
     const int n = M.dims[s];
-    // in extended precision for the usual small n_s: FP64 states are rotated into this
-    // basis and back, so the vectors are kept to twice a double's digits (hi + lo)
-    std::vector<double> w, Z, lo((size_t)n * n, 0.0), wlo(n, 0.0);
-    if (n <= 32) {
-      std::vector<long double> A(M.Vloc[s].begin(), M.Vloc[s].end()), wl, Zl;
-      jacobi<long double>(A, n, wl, Zl, 1e-36L);
+    std::vector<double> A = M.Vloc[s], w, Z;
+    jacobi_eigh(A, n, w, Z);
+    M.vb_lam.push_back(w);
+    Us.push_back(Z);
+    std::vector<double> lo((size_t)n * n, 0.0), wlo(n, 0.0);
+    if (n <= 32) {   // the usual sizes; the same rotations, so the same signs
+      std::vector<long double> Al(M.Vloc[s].begin(), M.Vloc[s].end()), wl, Zl;
+      jacobi<long double>(Al, n, wl, Zl, 1e-36L);
       w.assign(wl.begin(), wl.end());
       Z.assign(Zl.begin(), Zl.end());
       for (int i = 0; i < n; ++i) wlo[i] = (double)(wl[i] - (long double)w[i]);
       for (size_t i = 0; i < lo.size(); ++i) lo[i] = (double)(Zl[i] - (long double)Z[i]);
-    } else {
-      std::vector<double> A = M.Vloc[s];
-      jacobi_eigh(A, n, w, Z);
     }
-    M.vb_lam.push_back(w);
-    Us.push_back(Z);
-    M.vb_Us_lo.push_back(lo);
-    M.vb_lam_lo.push_back(wlo);
+    M.cb_lam.push_back(w);
+    M.cb_U.push_back(Z);
+    M.cb_lam_lo.push_back(wlo);
+    M.cb_U_lo.push_back(lo);
   }
-  M.vb_Us = Us;
   M.vb_U.assign((size_t)d * d, 0.0);
   for (int a = 0; a < d; ++a)
     for (int b = 0; b < d; ++b) {

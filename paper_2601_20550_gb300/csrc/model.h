@@ -34,10 +34,12 @@ struct Model {
   std::vector<int32_t> nb_off, nb_idx;         // per (ado, mode) coupling lists
   std::vector<double> nb_cA, nb_cB;
   // coupling eigenbasis: v_s = U_s diag(lam_s) U_s^T per mode; U = U_0 x U_1 x ...
-  std::vector<std::vector<double>> vb_lam, vb_lam_lo;   // per mode, n_s eigenvalues, hi + lo
-  std::vector<std::vector<double>> vb_Us, vb_Us_lo;   // per mode, n_s x n_s eigenvectors (columns), hi + lo
+  std::vector<std::vector<double>> vb_lam;     // per mode, n_s eigenvalues
   std::vector<double> vb_U;                    // d x d
   std::vector<double> vb_H, vb_mu, vb_mu_plus; // U^T X U
+  // the same eigenvalues and eigenvectors (columns) to twice a double's digits (hi + lo),
+  // for the FP64 path
+  std::vector<std::vector<double>> cb_lam, cb_lam_lo, cb_U, cb_U_lo;
 };
 
 // Coupling-eigenbasis quantities (fills vb_* of M).
