@@ -33,8 +33,9 @@ void count_launch(uint64_t n);
 
 namespace {
 
-constexpr int kPanel = 32;                 // columns (rows) of w per panel block: one per lane
-constexpr int kPanelThreads = 384;
+// Threads of a panel block: three blocks' registers fit an SM without spills, and the
+// row groups of the usual sizes (2 x 25 at five levels, 36 at six) divide evenly.
+__host__ __device__ constexpr int panel_threads(int R) { return R == 5 ? 320 : 384; }
 constexpr int kF64MaxExp = 16;             // build_hierarchy's limit
 constexpr int kRotPad = 33;
 constexpr int kSmallD = 32;                // largest basis of f64_small_kernel
@@ -142,6 +143,16 @@ __device__ __forceinline__ void group_product(const F64Ops &O, int g, const int2
       if (2 * p + 1 < R) mac(2 * p + 1, h[p].z, h[p].w, z);
     }
   }
+  // columns between states that differ in the two leading modes: the last digit stays,
+  // so row r meets column c + r, all with one factor
+  const int d1 = O.doff[g + 1];
+  for (int q = O.doff[g]; q < d1; ++q) {
+    const int4 h = O.dh[q];
+    const int2 *zc = zl + h.z * stride;
+#pragma unroll
+    for (int r = 0; r < R; ++r) mac(r, h.x, h.y, zc[r * stride]);
+  }
+  if (!O.soff) return;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int s1 = O.soff[g * R + r + 1];
@@ -320,12 +331,15 @@ __global__ void __launch_bounds__(256, 4) f64_item_kernel(const __grid_constant_
 }
 
 // ---------------------------------------------------------------------------
-// One panel per block, for bases whose items do not fit: 32 columns of w in the left
-// kernel (tp = -i alpha H' w), 32 rows in the right one (tp += i alpha w H', then the
-// elementwise rest of those rows).  Limbs scaled per column (row).
+// One panel per block, for bases whose items do not fit and for launches with few
+// items: kPanel columns of w in the left kernel (tp = -i alpha H' w), kPanel rows in the
+// right one, which adds i alpha w H' and the elementwise rest of those rows.  Limbs
+// scaled per column (row).  Half of the right kernel's blocks take the elementwise part
+// first: it lives on the FP64 pipe and the products on the IMAD pipe, and blocks that
+// start together would otherwise wait for the same pipe all the time.
 // ---------------------------------------------------------------------------
-template <int R, bool kRight, bool kMulti>
-__global__ void __launch_bounds__(kPanelThreads, 3) f64_panel_kernel(const __grid_constant__ F64Args P) {
+template <int R, int kPanel, bool kRight, bool kMulti>
+__global__ void __launch_bounds__(panel_threads(R), 3) f64_panel_kernel(const __grid_constant__ F64Args P) {
   extern __shared__ __align__(16) uint8_t smem[];
   const F64Set &S = pick<kMulti>(P);
   const F64Ops &O = S.O;
@@ -350,14 +364,15 @@ __global__ void __launch_bounds__(kPanelThreads, 3) f64_panel_kernel(const __gri
   __syncthreads();
   const double2 *w = S.w + item * dd;
   const double2 zero = make_double2(0.0, 0.0);
+  const int col_t = threadIdx.x & (kPanel - 1), row_t = threadIdx.x / kPanel, rows_t = blockDim.x / kPanel;
   if (!kRight) {
     int e = 0;
-    for (int c = warp; c < d; c += warps) {
-      const double2 v = lane < np ? w[(int64_t)c * d + p0 + lane] : zero;
+    for (int c = row_t; c < d; c += rows_t) {
+      const double2 v = col_t < np ? w[(int64_t)c * d + p0 + col_t] : zero;
       e = max(e, exp_field(v));
-      reinterpret_cast<double2 *>(zs)[c * ld + lane] = v;
+      reinterpret_cast<double2 *>(zs)[c * ld + col_t] = v;
     }
-    atomicMax(lexp + lane, e);
+    atomicMax(lexp + col_t, e);
   } else {
     for (int a = warp; a < kPanel; a += warps) {
       int e = 0;
@@ -371,24 +386,42 @@ __global__ void __launch_bounds__(kPanelThreads, 3) f64_panel_kernel(const __gri
     }
   }
   __syncthreads();
-  const int emax = lexp[lane];
-  for (int c = warp; c < d; c += warps) {
-    int4 *p = zs + c * ld + lane;
+  const int emax = lexp[col_t];
+  for (int c = row_t; c < d; c += rows_t) {
+    int4 *p = zs + c * ld + col_t;
     const double2 v = *reinterpret_cast<double2 *>(p);
     const int2 re = to_limbs(v.x, emax, O.bits, O.bits - 31), im = to_limbs(v.y, emax, O.bits, O.bits - 31);
     *p = make_int4(re.x, re.y, im.x, im.y);
   }
+  // the elementwise rest of the panel's rows on top of from
+  auto elementwise = [&](const double2 *from) {
+    const double2 *wb = S.w + (item - n) * dd;
+    const double2 *y = S.y ? S.y + item * dd : nullptr;
+    const double adec = alpha * O.decay[n];
+    for (int k = threadIdx.x; k < np * d; k += blockDim.x) {
+      const int ar = k / d, el = p0 * d + k;
+      double2 acc = from[el];
+      if (y) {
+        const double2 yv = y[el];
+        acc = make_double2(acc.x + yv.x, acc.y + yv.y);
+      }
+      S.out[item * dd + el] = couple(O, tab, list, wb, w, dd, p0 + ar, k - ar * d, el, acc, adec);
+    }
+  };
+  const bool early = kRight && ((unsigned)lb * 2654435761u >> 31);
+  if (early) elementwise(S.tp + item * dd);
   __syncthreads();
   // one task: a row group and 16 complex columns, lane = (column, component)
+  constexpr int kHalves = kPanel / 16;
   const int comp = lane & 1;
-  for (int k = warp; k < 2 * O.groups; k += warps) {
-    const int g = k >> 1, col = (k & 1) * 16 + (lane >> 1);
+  for (int k = warp; k < kHalves * O.groups; k += warps) {
+    const int g = k / kHalves, col = (k % kHalves) * 16 + (lane >> 1);
     Acc<R> A;
     group_product<R>(O, g, reinterpret_cast<const int2 *>(zs + col) + comp, 2 * ld, A);
     if (col < np) {
       // -i alpha (x + i y) = alpha (y - i x): the real sum goes to the imaginary part
       const Unit f = unit(lexp[col], O.hexp, comp == (kRight ? 1 : 0) ? -ah : ah);
-      double *t = reinterpret_cast<double *>(S.tp + item * dd) + (comp ^ 1);
+      double *t = reinterpret_cast<double *>((early ? S.out : S.tp) + item * dd) + (comp ^ 1);
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const int x = g * R + r;
@@ -404,21 +437,9 @@ __global__ void __launch_bounds__(kPanelThreads, 3) f64_panel_kernel(const __gri
       }
     }
   }
-  if (kRight) {
+  if (kRight && !early) {
     __syncthreads();
-    const double2 *t = S.tp + item * dd;
-    const double2 *wb = S.w + (item - n) * dd;
-    const double2 *y = S.y ? S.y + item * dd : nullptr;
-    const double adec = alpha * O.decay[n];
-    for (int k = threadIdx.x; k < np * d; k += blockDim.x) {
-      const int ar = k / d, el = p0 * d + k;
-      double2 acc = t[el];
-      if (y) {
-        const double2 yv = y[el];
-        acc = make_double2(acc.x + yv.x, acc.y + yv.y);
-      }
-      S.out[item * dd + el] = couple(O, tab, list, wb, wb + n * dd, dd, p0 + ar, k - ar * d, el, acc, adec);
-    }
+    elementwise(S.tp + item * dd);
   }
 }
 
@@ -957,10 +978,17 @@ int table_size(const Model &M) {
   return t;
 }
 
-size_t panel_smem(int d, int tab) { return (size_t)tab * 16 + (size_t)d * (kPanel + 1) * 16; }
+size_t panel_smem(int d, int tab, int panel) { return (size_t)tab * 16 + (size_t)d * (panel + 1) * 16; }
 
 size_t fused_smem(int d, int tab, int m, bool t) {
   return (size_t)tab * 16 + (size_t)m * d * (d | 1) * 16 * (t ? 2 : 1) + (size_t)m * (sizeof(List) + 4) + 64;
+}
+
+int sm_count() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
 }
 
 int row_group(const Model &M) {
@@ -968,7 +996,16 @@ int row_group(const Model &M) {
   return n % 5 == 0 ? 5 : n % 3 == 0 ? 6 : 4;
 }
 
-bool is_fused(int d, int tab) { return fused_smem(d, tab, 1, false) <= kFusedSmem; }
+// Columns (rows) per block of the panel kernels, or 0 for whole items.  An item keeps one
+// SM busy for 70 us at d = 64 and 150 us at d = 80, so a launch with fewer than four
+// items per SM spreads each over panels; 16 columns where 32 would leave fewer than
+// three blocks on an SM or fewer blocks than two per SM.
+int panel_width(int d, int tab, int64_t items) {
+  const int sms = sm_count();
+  if (fused_smem(d, tab, 1, false) <= kFusedSmem && (d < 48 || items >= 4 * sms)) return 0;
+  if (3 * (panel_smem(d, tab, 32) + 2048) > kMaxSmem || items * ((d + 31) / 32) < 2 * sms) return 16;
+  return 32;
+}
 
 // Items per block of the whole-item kernel: enough columns for two to four warps of
 // lanes, as long as the launch still has a few blocks per SM.
@@ -979,7 +1016,7 @@ int items_per_block(int d, int tab, int64_t items) {
   return m;
 }
 
-F64Set make_set(const F64Buf &b, int64_t begin, bool *fused, size_t *smem, int64_t *blocks) {
+F64Set make_set(const F64Buf &b, int64_t begin, int *panel, size_t *smem, int64_t *blocks) {
   const F64Ops &O = *b.ops;
   F64Set s{};
   s.O = O;
@@ -989,15 +1026,15 @@ F64Set make_set(const F64Buf &b, int64_t begin, bool *fused, size_t *smem, int64
   s.tp = b.tp;
   s.begin = begin;
   s.items = (int64_t)b.branches * O.n_ado;
-  *fused = is_fused(O.d, O.tab);
-  if (*fused) {
+  *panel = panel_width(O.d, O.tab, s.items);
+  if (*panel == 0) {
     s.per_block = items_per_block(O.d, O.tab, s.items);
     s.smem_t = fused_smem(O.d, O.tab, s.per_block, true) <= 56 * 1024;
     *smem = fused_smem(O.d, O.tab, s.per_block, s.smem_t);
     *blocks = (s.items + s.per_block - 1) / s.per_block;
   } else {
-    s.per_block = (O.d + kPanel - 1) / kPanel;
-    *smem = panel_smem(O.d, O.tab);
+    s.per_block = (O.d + *panel - 1) / *panel;
+    *smem = panel_smem(O.d, O.tab, *panel);
     *blocks = s.items * s.per_block;
   }
   return s;
@@ -1008,32 +1045,35 @@ void allow_smem(K kernel, size_t smem) {
   if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
-template <int R, bool kMulti>
-void launch_r(const F64Args &a, bool fused, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
-  if (fused) {
-    allow_smem(f64_item_kernel<R, kMulti>, smem);
-    f64_item_kernel<R, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
-    count_launch(1);
-  } else {
-    allow_smem(f64_panel_kernel<R, false, kMulti>, smem);
-    allow_smem(f64_panel_kernel<R, true, kMulti>, smem);
-    f64_panel_kernel<R, false, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
-    f64_panel_kernel<R, true, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
-    count_launch(2);
-  }
+template <int R, int kPanel, bool kMulti>
+void launch_panels(const F64Args &a, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
+  allow_smem(f64_panel_kernel<R, kPanel, false, kMulti>, smem);
+  allow_smem(f64_panel_kernel<R, kPanel, true, kMulti>, smem);
+  f64_panel_kernel<R, kPanel, false, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
+  f64_panel_kernel<R, kPanel, true, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
+  count_launch(2);
 }
 
-void launch(const F64Args &a, int R, bool fused, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
+template <int R, bool kMulti>
+void launch_r(const F64Args &a, int panel, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
+  if (panel == 32) return launch_panels<R, 32, kMulti>(a, blocks, smem, threads, st);
+  if (panel == 16) return launch_panels<R, 16, kMulti>(a, blocks, smem, threads, st);
+  allow_smem(f64_item_kernel<R, kMulti>, smem);
+  f64_item_kernel<R, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
+  count_launch(1);
+}
+
+void launch(const F64Args &a, int R, int panel, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
   if (blocks == 0) return;
   if (blocks > 0x7fffffffLL) throw std::invalid_argument("too many work items for one stage launch");
   auto with = [&](auto multi) {
     constexpr bool m = decltype(multi)::value;
     if (R == 4)
-      launch_r<4, m>(a, fused, blocks, smem, threads, st);
+      launch_r<4, m>(a, panel, blocks, smem, threads, st);
     else if (R == 5)
-      launch_r<5, m>(a, fused, blocks, smem, threads, st);
+      launch_r<5, m>(a, panel, blocks, smem, threads, st);
     else
-      launch_r<6, m>(a, fused, blocks, smem, threads, st);
+      launch_r<6, m>(a, panel, blocks, smem, threads, st);
   };
   if (a.n > 0)
     with(std::true_type());
@@ -1045,7 +1085,7 @@ void launch(const F64Args &a, int R, bool fused, int64_t blocks, size_t smem, in
 
 bool f64_supported(const Model &M) {
   const int tab = table_size(M);
-  if (M.n_exp > kF64MaxExp || M.n_modes > kF64MaxModes || tab > kF64MaxTab || panel_smem(M.d, tab) + sizeof(List) + 256 > kMaxSmem) return false;
+  if (M.n_exp > kF64MaxExp || M.n_modes > kF64MaxModes || tab > kF64MaxTab || panel_smem(M.d, tab, 16) + sizeof(List) + 256 > kMaxSmem) return false;
   if (row_products(M) > 500) return false;   // the 64-bit sums stay exact
   for (double h : M.vb_H)
     if (!std::isfinite(h)) return false;
@@ -1105,8 +1145,10 @@ F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::
     r.x = (int)((v - r.y) >> low);
     return r;
   };
-  std::vector<int> foff(1, 0), fc, soff(1, 0);
-  std::vector<int4> fh, sh;
+  std::vector<int> foff(1, 0), fc, doff(1, 0), soff(1, 0);
+  std::vector<int4> fh, dh, sh;
+  const bool aligned = R == M.dims.back();   // a group is the last mode's digits
+  auto last_digit_kept = [&](int a, int c) { return a % R == c % R; };
   for (int g = 0; g < O.groups; ++g) {
     const int a0 = g * R, a1 = std::min(d, a0 + R);
     std::vector<std::vector<int>> single(R);
@@ -1127,6 +1169,16 @@ F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::
       }
     }
     foff.push_back((int)fc.size());
+    if (aligned) {
+      const std::vector<int> cand = single[0];
+      for (int c : cand)
+        if (last_digit_kept(a0, c)) {
+          const int2 v = limbs(a0, c);
+          dh.push_back(make_int4(v.x, v.y, c, 0));
+          for (int r = 0; r < R; ++r) single[r].erase(std::find(single[r].begin(), single[r].end(), c + r));
+        }
+    }
+    doff.push_back((int)dh.size());
     for (int r = 0; r < R; ++r) {
       for (int c : single[r]) {
         const int2 v = limbs(a0 + r, c);
@@ -1158,8 +1210,12 @@ F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::
   O.foff = up(foff, allocs);
   O.fc = up(fc, allocs);
   O.fh = up(fh, allocs);
-  O.soff = up(soff, allocs);
-  O.sh = up(sh, allocs);
+  O.doff = up(doff, allocs);
+  O.dh = up(dh, allocs);
+  if (!sh.empty()) {
+    O.soff = up(soff, allocs);
+    O.sh = up(sh, allocs);
+  }
   O.noff = up(std::vector<int>(nb_off.begin(), nb_off.end()), allocs);
   O.nb = up(nb, allocs);
   O.decay = up(M.decay, allocs);
@@ -1170,23 +1226,23 @@ F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::
 }
 
 std::vector<std::pair<int, int>> f64_shapes(const F64Buf &b) {
-  bool fused = false;
+  int panel = 0;
   size_t smem = 0;
   int64_t blocks = 0;
-  make_set(b, 0, &fused, &smem, &blocks);
+  make_set(b, 0, &panel, &smem, &blocks);
   const int n = (int)std::min<int64_t>(blocks, 0x7fffffff);
-  if (fused) return {{256, n}, {128, n}, {64, n}};
-  return {{kPanelThreads, n}, {256, n}, {192, n}};
+  if (panel == 0) return {{256, n}, {128, n}, {64, n}};
+  return {{panel_threads(b.ops->R), n}, {256, n}, {192, n}};
 }
 
 void f64_stage(const F64Buf &b, double alpha, int threads, cudaStream_t st) {
-  bool fused = false;
+  int panel = 0;
   size_t smem = 0;
   int64_t blocks = 0;
   F64Args a{};
-  a.one = make_set(b, 0, &fused, &smem, &blocks);
+  a.one = make_set(b, 0, &panel, &smem, &blocks);
   a.alpha = alpha;
-  launch(a, b.ops->R, fused, blocks, smem, threads, st);
+  launch(a, b.ops->R, panel, blocks, smem, threads, st);
 }
 
 namespace {
@@ -1195,13 +1251,6 @@ struct SmallShape {
   int sync = 0, blocks = 0, threads = 0, cluster = 1;
   size_t smem = 0;
 };
-
-int sm_count() {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms;
-}
 
 // Elements per block up to which a launch for all steps wins: beyond it a stage's own
 // work (20-26 FP64 operations per element, two per clock and SM) exceeds what a launch
@@ -1370,14 +1419,14 @@ F64Plan::~F64Plan() {
 }
 
 void f64_plan(F64Plan &p, const std::vector<F64Buf> &sets, cudaStream_t st) {
-  std::map<std::pair<int, bool>, std::vector<F64Set>> by;
-  std::map<std::pair<int, bool>, std::pair<int64_t, size_t>> size;
+  std::map<std::pair<int, int>, std::vector<F64Set>> by;
+  std::map<std::pair<int, int>, std::pair<int64_t, size_t>> size;
   for (const F64Buf &b : sets) {
-    bool fused = false;
+    int panel = 0;
     size_t smem = 0;
     int64_t blocks = 0;
-    F64Set s = make_set(b, 0, &fused, &smem, &blocks);
-    auto key = std::make_pair(b.ops->R, fused);
+    F64Set s = make_set(b, 0, &panel, &smem, &blocks);
+    auto key = std::make_pair(b.ops->R, panel);
     s.begin = size[key].first;
     size[key].first += blocks;
     size[key].second = std::max(size[key].second, smem);
@@ -1402,7 +1451,7 @@ void f64_stage_plan(const F64Plan &p, double alpha, cudaStream_t st) {
     a.many = (const F64Set *)c.desc;
     a.n = c.n;
     a.alpha = alpha;
-    launch(a, c.R, c.fused, c.blocks, c.smem, c.fused ? 256 : kPanelThreads, st);
+    launch(a, c.R, c.panel, c.blocks, c.smem, c.panel == 0 ? 256 : panel_threads(c.R), st);
   }
 }
 

@@ -39,10 +39,11 @@ struct F64Ops {
   int dims[kF64MaxModes] = {}, tab_off[kF64MaxModes] = {};
   // entries of H' as two signed limbs, h = (hi 2^(bits - 31) + lo) 2^(hexp + 1 - bits).  Per
   // group: columns where most rows are non-zero (all R rows' limbs, two per int4; for odd
-  // R the spare half of the last holds the column), then per row the remaining columns
-  // (limbs and column).
-  const int *foff = nullptr, *fc = nullptr, *soff = nullptr;
-  const int4 *fh = nullptr, *sh = nullptr;
+  // R the spare half of the last holds the column), the columns that all rows meet with
+  // one factor, shifted by the row (limbs and first column), then per row the remaining
+  // columns (limbs and column; soff null if there are none).
+  const int *foff = nullptr, *fc = nullptr, *doff = nullptr, *soff = nullptr;
+  const int4 *fh = nullptr, *dh = nullptr, *sh = nullptr;
   const int *noff = nullptr;      // [n_ado * n_modes + 1]
   const F64Entry *nb = nullptr;
   const double *decay = nullptr;  // [n_ado]
@@ -103,7 +104,7 @@ bool f64_small_steps_plan(const F64SmallPlan &p, double dt, int64_t steps, cudaS
 struct F64Plan {
   struct Class {   // sets of one kernel variant
     int R;
-    bool fused;
+    int panel;   // columns per block, 0: whole items
     int64_t blocks;
     size_t smem;
     int n;
