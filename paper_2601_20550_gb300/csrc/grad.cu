@@ -55,6 +55,8 @@ static void ensure_adjoint(heom_hier *h) {
   int nvl = 0;
   for (int s = 0; s < S; ++s) nvl += M.dims[s] * M.dims[s];
   if (nvl > kAdjMaxVl) throw Fail{HEOM_EINVAL, "mode bases too large for the gradient"};
+  bool work = h->f64.ready && (size_t)2 * M.d * kGradLd * 16 + 1024 <= 227 * 1024;
+  for (int n : M.dims) work = work && n <= kGradMaxN;
   std::vector<int> off((size_t)N * S + 1, 0), idx(M.nb_idx.size());
   std::vector<double> cA(M.nb_idx.size()), cB(M.nb_idx.size());
   for (int n = 0; n < N; ++n)
@@ -80,6 +82,8 @@ static void ensure_adjoint(heom_hier *h) {
   a.nb_cA = h->up(cA);
   a.nb_cB = h->up(cB);
   h->dm_adj = a;
+  if (work) h->f64_adj = f64_build(M, off, idx, cA, cB, -1.0, h->allocs);
+  h->adj_work = work;
   h->adj_ado = h->up(M.ado);
   h->adj_entry_exp = h->up(eexp);
   h->adj_ready = true;
@@ -119,15 +123,24 @@ struct AdjCtx {
 
 static void comm_grad(AdjCtx &c, const double2 *g, const double2 *w, int64_t items, double ph_re, double ph_im,
                       double alpha, double *G) {
-  const int d = c.h->M.d, tiles = (d + 15) / 16;
-  const int64_t chunks = std::max<int64_t>(1, std::min<int64_t>(items, std::max(1, 2432 / (tiles * tiles))));
   // Re(-i x) = Im x (Hamiltonian term); Re(1 x) = Re x (kicks)
-  if (ph_re == 0.0 && ph_im == -1.0)
-    comm_grad_kernel<true><<<(unsigned)(tiles * tiles * chunks), 256, 0, c.st>>>(g, w, items, d, alpha, G);
-  else if (ph_re == 1.0 && ph_im == 0.0)
-    comm_grad_kernel<false><<<(unsigned)(tiles * tiles * chunks), 256, 0, c.st>>>(g, w, items, d, alpha, G);
+  const bool imag = ph_re == 0.0 && ph_im == -1.0;
+  if (!imag && !(ph_re == 1.0 && ph_im == 0.0)) throw Fail{HEOM_EINVAL, "unsupported gradient phase"};
+  const int d = c.h->M.d, slices = (d + kCommSlice - 1) / kCommSlice;
+  auto launch = [&](auto kernel, int T) {
+    const int tiles = (d + 16 * T - 1) / (16 * T);
+    // two blocks per SM share the (item, slice) units
+    const int64_t chunks = std::max<int64_t>(1, std::min<int64_t>(items * slices, 304 / (tiles * tiles)));
+    CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, comm_smem(T)));
+    kernel<<<(unsigned)(tiles * tiles * chunks), 256, comm_smem(T), c.st>>>(g, w, items, d, alpha, G);
+  };
+  // 16 x 16 tiles where one covers G (d = 16, 224 items: 10 against 16 us), else 32 x 32
+  // (d = 24: 28 against 31 us, d = 64: 133 against 206 us; 64 x 64: 129 us there, but 614
+  // against 366 us at d = 80 and 6.8 against 5.5 ms at d = 216)
+  if (d <= 16)
+    imag ? launch(comm_grad_kernel<true, 1>, 1) : launch(comm_grad_kernel<false, 1>, 1);
   else
-    throw Fail{HEOM_EINVAL, "unsupported gradient phase"};
+    imag ? launch(comm_grad_kernel<true, 2>, 2) : launch(comm_grad_kernel<false, 2>, 2);
   count_launch(1);
   LAUNCH_CHECK();
 }
@@ -137,6 +150,23 @@ static void grad_pair(AdjCtx &c, const double2 *g, const double2 *w, int branche
   const Model &M = c.h->M;
   const int64_t items = (int64_t)branches * M.n_ado;
   comm_grad(c, g, w, items, 0.0, -1.0, alpha, c.G + c.L.H);
+  if (c.h->adj_work) {
+    // an item's panels in up to four waves of blocks (each block ends with its reduction)
+    const int64_t units = items * 2 * M.n_modes, panels = (M.d + kGradPanel - 1) / kGradPanel;
+    const int splits = (int)std::min<int64_t>(panels, (2432 + units - 1) / units);
+    const CouplingGradArgs a{g, w, c.h->f64, c.h->adj_ado, c.h->adj_entry_exp, M.n_exp,
+                             splits, alpha, c.G + c.L.v, c.G + c.L.re, c.G + c.L.im, c.G + c.L.nu};
+    const int64_t blocks = units * splits;
+    if (blocks > 0x7fffffffLL) throw Fail{HEOM_EINVAL, "too many work items for one launch"};
+    const int smem = 2 * M.d * kGradLd * 16;
+    const auto kernel = *std::max_element(M.dims.begin(), M.dims.end()) > 4 ? coupling_grad_vb_kernel<kGradMaxN>
+                                                                            : coupling_grad_vb_kernel<4>;
+    CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    kernel<<<(unsigned)blocks, 256, smem, c.st>>>(a);
+    count_launch(1);
+    LAUNCH_CHECK();
+    return;
+  }
   coupling_grad_kernel<<<(unsigned)std::min<int64_t>(items, 152 * 16), 256, 0, c.st>>>(
       g, w, c.h->dm64, c.h->adj_ado, M.n_exp, c.h->adj_entry_exp, items, alpha, c.G + c.L.v, c.G + c.L.re,
       c.G + c.L.im, c.G + c.L.nu);
@@ -144,12 +174,41 @@ static void grad_pair(AdjCtx &c, const double2 *g, const double2 *w, int branche
   LAUNCH_CHECK();
 }
 
-static void stage64(AdjCtx &c, const DevModel<double> &dm, const double2 *w, const double2 *y, double2 *out,
+// out = y + alpha L w (or L^H w); y null: zero; tp: scratch for the commutator's part
+// (may equal out if out is not y).
+static void stage64(AdjCtx &c, bool adjoint, const double2 *w, const double2 *y, double2 *out, double2 *tp,
                     double alpha, int branches) {
+  heom_hier *h = c.h;
+  if (h->adj_work) {
+    const F64Buf b{adjoint ? &h->f64_adj : &h->f64, w, y, out, tp, branches};
+    f64_stage(b, alpha, f64_shapes(b)[0].first, c.st);
+    LAUNCH_CHECK();
+    return;
+  }
   const int64_t total = (int64_t)branches * c.per;
-  stage_kernel<double><<<grid_for(total), 256, 0, c.st>>>(w, y, out, alpha, dm, total);
+  if (!y) {
+    CUDA_TRY(cudaMemsetAsync(out, 0, (size_t)total * 16, c.st));
+    y = out;
+  }
+  stage_kernel<double><<<grid_for(total), 256, 0, c.st>>>(w, y, out, alpha, adjoint ? h->dm_adj : h->dm64, total);
   count_launch(1);
   LAUNCH_CHECK();
+}
+
+// RK4 steps, dipole matrices and the basis change of the basis the gradient runs in.
+static void steps64(AdjCtx &c, double2 *y, double2 *wa, double2 *wb, int branches, double dt, int64_t n) {
+  if (c.h->adj_work)
+    rk4_work64(c.h, y, wa, wb, branches, dt, n, c.st);
+  else
+    rk4_steps<double>(c.h, y, wa, wb, branches, dt, n, c.st, HEOM_FP64);
+}
+
+static const double *mu_grad(heom_hier *h, int which) {
+  return h->adj_work ? mu_work<double>(h, which) : mu_of<double>(h, which);
+}
+
+static void to_grad_basis(AdjCtx &c, double2 *x, double2 *tmp) {
+  if (c.h->adj_work) work_in(c.h, x, x, tmp, 1, c.st);
 }
 
 static void axpy64(AdjCtx &c, double2 *y, const double2 *x, double a, int64_t n) {
@@ -163,26 +222,21 @@ static void axpy64(AdjCtx &c, double2 *y, const double2 *x, double a, int64_t n)
 // gradients.  Forward: w4 = y + dt/4 L y, w3 = y + dt/3 L w4, w2 = y + dt/2 L w3,
 // y' = y + dt L w2.
 static void back_step(AdjCtx &c, const double2 *y, double2 *lam, int B, double dt) {
-  const DevModel<double> &F = c.h->dm64, &Ad = c.h->dm_adj;
   const int64_t n = (int64_t)B * c.per;
-  const size_t bytes = (size_t)n * 16;
-  stage64(c, F, y, y, c.W4, dt / 4, B);
-  stage64(c, F, c.W4, y, c.W3, dt / 3, B);
-  stage64(c, F, c.W3, y, c.W2, dt / 2, B);
-  grad_pair(c, lam, c.W2, B, dt);                       // y' = y + dt L w2
-  CUDA_TRY(cudaMemsetAsync(c.A, 0, bytes, c.st));
-  stage64(c, Ad, lam, c.A, c.A, dt, B);                 // w2bar = dt L^H lam
+  stage64(c, false, y, y, c.W4, c.W4, dt / 4, B);
+  stage64(c, false, c.W4, y, c.W3, c.W3, dt / 3, B);
+  stage64(c, false, c.W3, y, c.W2, c.W2, dt / 2, B);
+  grad_pair(c, lam, c.W2, B, dt);                                // y' = y + dt L w2
+  stage64(c, true, lam, nullptr, c.A, c.A, dt, B);               // w2bar = dt L^H lam
   grad_pair(c, c.A, c.W3, B, dt / 2);
-  CUDA_TRY(cudaMemsetAsync(c.W2, 0, bytes, c.st));
-  stage64(c, Ad, c.A, c.W2, c.W2, dt / 2, B);           // w3bar = dt/2 L^H w2bar
+  stage64(c, true, c.A, nullptr, c.W2, c.W2, dt / 2, B);         // w3bar = dt/2 L^H w2bar
   grad_pair(c, c.W2, c.W4, B, dt / 3);
   axpy64(c, lam, c.A, 1.0, n);
   axpy64(c, lam, c.W2, 1.0, n);
-  CUDA_TRY(cudaMemsetAsync(c.W3, 0, bytes, c.st));
-  stage64(c, Ad, c.W2, c.W3, c.W3, dt / 3, B);          // w4bar = dt/3 L^H w3bar
+  stage64(c, true, c.W2, nullptr, c.W3, c.W3, dt / 3, B);        // w4bar = dt/3 L^H w3bar
   grad_pair(c, c.W3, y, B, dt / 4);
   axpy64(c, lam, c.W3, 1.0, n);
-  stage64(c, Ad, c.W3, lam, lam, dt / 4, B);            // + dt/4 L^H w4bar
+  stage64(c, true, c.W3, lam, lam, c.A, dt / 4, B);              // + dt/4 L^H w4bar
 }
 
 // Reverse sweep over a span of N RK4 steps from `start` (B branches):
@@ -200,7 +254,7 @@ static void backprop_span(AdjCtx &c, const double2 *start, int64_t N, int B, dou
   DeviceBuffer cur(sz);
   CUDA_TRY(cudaMemcpyAsync(cur.p, start, sz, cudaMemcpyDeviceToDevice, c.st));
   for (int64_t k = 1; k < n_ck; ++k) {
-    rk4_steps<double>(c.h, (double2 *)cur.p, c.W4, c.W3, B, dt, M, c.st, HEOM_FP64);
+    steps64(c, (double2 *)cur.p, c.W4, c.W3, B, dt, M);
     CUDA_TRY(cudaMemcpyAsync(ck[k - 1]->p, cur.p, sz, cudaMemcpyDeviceToDevice, c.st));
   }
   const int ring_n = (int)std::min<int64_t>(M, N);
@@ -212,7 +266,7 @@ static void backprop_span(AdjCtx &c, const double2 *start, int64_t N, int B, dou
     CUDA_TRY(cudaMemcpyAsync(ring[0]->p, src, sz, cudaMemcpyDeviceToDevice, c.st));
     for (int64_t u = 1; u < len; ++u) {
       CUDA_TRY(cudaMemcpyAsync(ring[u]->p, ring[u - 1]->p, sz, cudaMemcpyDeviceToDevice, c.st));
-      rk4_steps<double>(c.h, (double2 *)ring[u]->p, c.W4, c.W3, B, dt, 1, c.st, HEOM_FP64);
+      steps64(c, (double2 *)ring[u]->p, c.W4, c.W3, B, dt, 1);
     }
     for (int64_t t = s0 + len - 1; t >= s0; --t) {
       const double2 *y = (const double2 *)ring[t - s0]->p;
@@ -386,10 +440,14 @@ extern "C" heom_status heom_response_2d_grad(heom_hier *h, const heom_state *rho
     DeviceBuffer Tst((size_t)n1 * sz1), Tbar((size_t)n1 * sz1);
     CUDA_TRY(cudaMemsetAsync(Tbar.p, 0, Tbar.bytes, st));
     double2 *T = (double2 *)Tst.p, *Tb = (double2 *)Tbar.p;
-    kick_into<double>(h, (const double2 *)rho_eq->buf.p, T, 1, mu_of<double>(h, 2), st);
+    DeviceBuffer eqw(sz1);
+    double2 *eqp = (double2 *)eqw.p;
+    CUDA_TRY(cudaMemcpyAsync(eqp, rho_eq->buf.p, sz1, cudaMemcpyDeviceToDevice, st));
+    to_grad_basis(c, eqp, c.W4);
+    kick_into<double>(h, eqp, T, 1, mu_grad(h, 2), st);
     for (int j = 1; j < n1; ++j) {
       CUDA_TRY(cudaMemcpyAsync(T + (int64_t)j * per, T + (int64_t)(j - 1) * per, sz1, cudaMemcpyDeviceToDevice, st));
-      rk4_steps<double>(h, T + (int64_t)j * per, c.W4, c.W3, 1, dt, m, st, HEOM_FP64);
+      steps64(c, T + (int64_t)j * per, c.W4, c.W3, 1, dt, m);
     }
     const double c_re = 0.0, c_im = -1.0;   // i^3
     DeviceBuffer BR((size_t)cap * sz1), Y0((size_t)cap * sz1), lam((size_t)cap * sz1), tmp((size_t)cap * sz1),
@@ -403,22 +461,22 @@ extern "C" heom_status heom_response_2d_grad(heom_hier *h, const heom_state *rho
         // forward: second kick of both pathways, t2, third kick
         for (int j = 0; j < nj; ++j) {
           kick2_pair_kernel<double><<<grid_for(per), 256, 0, st>>>(T + (int64_t)(j0 + j) * per, br + (int64_t)j * per,
-                                                                  br + (int64_t)(nj + j) * per, h->mup64, h->mum64, d, per);
+                                                                  br + (int64_t)(nj + j) * per, mu_grad(h, 1), mu_grad(h, 2), d, per);
           count_launch(1);
           LAUNCH_CHECK();
         }
         CUDA_TRY(cudaMemcpyAsync(t1, br, (size_t)B * sz1, cudaMemcpyDeviceToDevice, st));   // F = G^{n2} BR
-        rk4_steps<double>(h, t1, c.W4, c.W3, B, dt, n2[it], st, HEOM_FP64);
-        kick_into<double>(h, t1, y0, B, mu_of<double>(h, 1), st);                                              // Y0 = mu+^x F
+        steps64(c, t1, c.W4, c.W3, B, dt, n2[it]);
+        kick_into<double>(h, t1, y0, B, mu_grad(h, 1), st);                                              // Y0 = mu+^x F
         // t3: traces at t = k m; lam starts with the source of the last sample
         CUDA_TRY(cudaMemsetAsync(lm, 0, (size_t)B * sz1, st));
         auto trace_src = [&](int64_t t, const double2 *y, double2 *l) {
           if (t % m) return;
           const int k = (int)(t / m);
           trace_adjoint_kernel<<<(unsigned)((dd + 255) / 256), 256, 0, st>>>(
-              l, y, RbI + (int64_t)j0 * n3 + k, n3, h->mu64, d, per, nj, c_re, c_im, c.G + c.L.mu);
+              l, y, RbI + (int64_t)j0 * n3 + k, n3, mu_grad(h, 0), d, per, nj, c_re, c_im, c.G + c.L.mu);
           trace_adjoint_kernel<<<(unsigned)((dd + 255) / 256), 256, 0, st>>>(
-              l + (int64_t)nj * per, y + (int64_t)nj * per, RbII + (int64_t)j0 * n3 + k, n3, h->mu64, d, per, nj,
+              l + (int64_t)nj * per, y + (int64_t)nj * per, RbII + (int64_t)j0 * n3 + k, n3, mu_grad(h, 0), d, per, nj,
               c_re, c_im, c.G + c.L.mu);
           count_launch(2);
           LAUNCH_CHECK();
@@ -427,26 +485,26 @@ extern "C" heom_status heom_response_2d_grad(heom_hier *h, const heom_state *rho
           // state at the last sample, for its trace source
           DeviceBuffer yN((size_t)B * sz1);
           CUDA_TRY(cudaMemcpyAsync(yN.p, y0, (size_t)B * sz1, cudaMemcpyDeviceToDevice, st));
-          rk4_steps<double>(h, (double2 *)yN.p, c.W4, c.W3, B, dt, N3, st, HEOM_FP64);
+          steps64(c, (double2 *)yN.p, c.W4, c.W3, B, dt, N3);
           trace_src(N3, (const double2 *)yN.p, lm);
           CUDA_TRY(cudaStreamSynchronize(st));
         }
         backprop_span(c, y0, N3, B, dt, Mck, lm, trace_src);
         // third kick: Fbar = mu-^x Y0bar; d/d mu+
         comm_grad(c, lm, t1, (int64_t)B * M.n_ado, 1.0, 0.0, 1.0, c.G + c.L.mup);
-        kick_into<double>(h, lm, t2b, B, mu_of<double>(h, 2), st);
+        kick_into<double>(h, lm, t2b, B, mu_grad(h, 2), st);
         // t2
         backprop_span(c, br, n2[it], B, dt, Mck, t2b, nullptr);
         // second kicks: I_j = mu+^x T_j, II_j = mu-^x (-T_j^dagger)
         double2 *Tj = T + (int64_t)j0 * per, *Tbj = Tb + (int64_t)j0 * per;
         const int64_t nI = (int64_t)nj * per;
         comm_grad(c, t2b, Tj, (int64_t)nj * M.n_ado, 1.0, 0.0, 1.0, c.G + c.L.mup);
-        kick_into<double>(h, t2b, t1, nj, mu_of<double>(h, 2), st);
+        kick_into<double>(h, t2b, t1, nj, mu_grad(h, 2), st);
         axpy64(c, Tbj, t1, 1.0, nI);
         neg_dagger_kernel<<<grid_for(nI), 256, 0, st>>>(Tj, t1, d, nI);                     // U = -T^dagger
         count_launch(1);
         comm_grad(c, t2b + nI, t1, (int64_t)nj * M.n_ado, 1.0, 0.0, 1.0, c.G + c.L.mum);
-        kick_into<double>(h, t2b + nI, t1, nj, mu_of<double>(h, 1), st);                                      // Ubar = mu+^x IIbar
+        kick_into<double>(h, t2b + nI, t1, nj, mu_grad(h, 1), st);   // Ubar = mu+^x IIbar
         neg_dagger_kernel<<<grid_for(nI), 256, 0, st>>>(t1, y0, d, nI);
         count_launch(1);
         LAUNCH_CHECK();
@@ -462,17 +520,36 @@ extern "C" heom_status heom_response_2d_grad(heom_hier *h, const heom_state *rho
       axpy64(c, l, Tb + (t / m) * per, 1.0, per);
     };
     backprop_span(c, T, N1, 1, dt, Mck, lm, trunk_src);
-    comm_grad(c, lm, (const double2 *)rho_eq->buf.p, M.n_ado, 1.0, 0.0, 1.0, c.G + c.L.mum);
+    comm_grad(c, lm, eqp, M.n_ado, 1.0, 0.0, 1.0, c.G + c.L.mum);
     double2 *eqbar = (double2 *)tmp.p;
-    kick_into<double>(h, lm, eqbar, 1, mu_of<double>(h, 1), st);                                             // (mu-^x)^H = mu+^x
+    kick_into<double>(h, lm, eqbar, 1, mu_grad(h, 1), st);   // (mu-^x)^H = mu+^x
     DeviceBuffer rho0(sz1);
     CUDA_TRY(cudaMemsetAsync(rho0.p, 0, sz1, st));
     const double one[2] = {1.0, 0.0};
     CUDA_TRY(cudaMemcpyAsync(rho0.p, one, 16, cudaMemcpyHostToDevice, st));
+    to_grad_basis(c, (double2 *)rho0.p, c.W4);
     backprop_span(c, (const double2 *)rho0.p, rho_eq->eq_steps, 1, rho_eq->eq_dt, Mck, eqbar, nullptr);
     std::vector<double> G(c.L.total);
     CUDA_TRY(cudaMemcpyAsync(G.data(), Gd.p, Gd.bytes, cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
+    if (h->adj_work) {   // back to the product basis: X' = U^T X U, so G = U G' U^T
+      auto back = [](double *g, const std::vector<double> &U, int n) {
+        std::vector<double> t((size_t)n * n, 0.0), r((size_t)n * n, 0.0);
+        for (int a = 0; a < n; ++a)
+          for (int k = 0; k < n; ++k)
+            for (int b = 0; b < n; ++b) t[(size_t)a * n + b] += U[(size_t)a * n + k] * g[(size_t)k * n + b];
+        for (int a = 0; a < n; ++a)
+          for (int b = 0; b < n; ++b)
+            for (int k = 0; k < n; ++k) r[(size_t)a * n + b] += t[(size_t)a * n + k] * U[(size_t)b * n + k];
+        std::copy(r.begin(), r.end(), g);
+      };
+      for (int64_t o : {c.L.H, c.L.mup, c.L.mum, c.L.mu}) back(G.data() + o, M.vb_U, d);
+      int64_t o = c.L.v;
+      for (int sm = 0; sm < M.n_modes; ++sm) {
+        back(G.data() + o, M.cb_U[sm], M.dims[sm]);
+        o += (int64_t)M.dims[sm] * M.dims[sm];
+      }
+    }
     // ---- chain rule to the twelve parameters
     for (int i = 0; i < 12; ++i) dtheta[i] = 0.0;
     for (Build &b : builds) {

@@ -145,7 +145,7 @@ struct heom_hier {
   // adjoint RHS tables (built on the first gradient call)
   // launch shapes picked by the autotuner: (kernel kind, elements) -> (block, grid)
   std::map<std::pair<int, int64_t>, std::pair<int, int>> tuned;
-  bool adj_ready = false;
+  bool adj_ready = false, adj_work = false;   // adj_work: the gradient runs in the coupling basis
   DevModel<double> dm_adj{};
   int *adj_ado = nullptr, *adj_entry_exp = nullptr;
   ~heom_hier() {
