@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 
 #include "f64_stage.h"
+#include "fixed54.cuh"
 #include "kernels.cuh"
 
 namespace heom {
@@ -62,31 +63,6 @@ static __global__ void __launch_bounds__(256) neg_dagger_kernel(const double2 *_
 // sum per thread, 452 us in register tiles (the FP64 pipe's
 // rate, also of its mma.m8n8k4 form), 133 us here; rms error 1.0e-16 of the largest entry,
 // FP64 sums 3.9e-16.
-// x 2^(1076 - top) to the nearest integer below 2^54 in magnitude; top: the largest
-// exponent field of the slice (at least 1)
-__device__ __forceinline__ int2 fixed54(double x, int top) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const int e = (int)(u >> 52) & 0x7ff, sh = min(top - max(e, 1), 63);
-  const unsigned long long m = ((u & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull)) << 1;
-  const long long r = (long long)((m + ((1ull << sh) >> 1)) >> sh), q = (long long)u < 0 ? -r : r;
-  const int hi = (int)((q + (1 << 25)) >> 26);
-  return make_int2(hi, (int)(q - ((long long)hi << 26)));
-}
-
-// re hi, re lo, im hi, im lo
-__device__ __forceinline__ int4 fixed54(double2 z, int top) {
-  const int2 a = fixed54(z.x, top), b = fixed54(z.y, top);
-  return make_int4(a.x, a.y, b.x, b.y);
-}
-
-__device__ __forceinline__ int exponent(double2 z) {
-  return max(__double2hiint(z.x) & 0x7ff00000, __double2hiint(z.y) & 0x7ff00000) >> 20;
-}
-
-__device__ __forceinline__ double pow2(int n) {   // 2^n, -1074 <= n <= 1023
-  return n < -1022 ? __longlong_as_double(1ll << (n + 1074)) : __longlong_as_double((long long)(n + 1023) << 52);
-}
-
 constexpr int kCommSlice = 16, kCommLd = kCommSlice + 1;
 
 constexpr int comm_smem(int T) { return 4 * 16 * T * kCommLd * 16 + 256 * T * T * 8; }
@@ -178,16 +154,13 @@ __global__ void __launch_bounds__(256, 2) comm_grad_kernel(const double2 *__rest
         }
       }
     }
-    const int n = eg + ew - 2 * 1076 + 52;
-    const double f1 = eg < 0x7ff && ew < 0x7ff ? pow2(n / 2) : __longlong_as_double(0x7ff8000000000000ll);
-    const double f2 = pow2(n - n / 2);
+    const Unit54 unit(eg, ew);
 #pragma unroll
     for (int i = 0; i < T; ++i)
 #pragma unroll
       for (int j = 0; j < T; ++j) {
         double *s = sum + (i * T + j) * 256 + t;
-        const double v = __ll2double_rn(hh[i][j] + ((hl[i][j] + (1ll << 25)) >> 26));
-        *s = n > -1000 && n < 900 ? fma(v, f1 * f2, *s) : fma(v * f1, f2, *s);
+        *s = unit.add(hh[i][j], hl[i][j], *s);
       }
   }
 #pragma unroll

@@ -292,7 +292,30 @@ void kick_into(heom_hier *h, const typename CxT<R>::type *in, typename CxT<R>::t
                       int branches, const R *K, cudaStream_t st) {
   const Model &M = h->M;
   const int64_t total = (int64_t)branches * M.n_ado * M.d * M.d;
+  if constexpr (sizeof(R) == 8)
+    if (M.d >= kKickTiledMinD) {
+      kick_tiled(in, out, K, M.d, (int64_t)branches * M.n_ado, false, st);
+      LAUNCH_CHECK();
+      return;
+    }
   kick_kernel<R><<<grid_for(total), 256, 0, st>>>(in, out, K, M.d, total);
+  count_launch(1);
+  LAUNCH_CHECK();
+}
+
+template <typename R>
+void kick2_into(heom_hier *h, const typename CxT<R>::type *T, typename CxT<R>::type *outI,
+                typename CxT<R>::type *outII, const R *KI, const R *KII, cudaStream_t st) {
+  const Model &M = h->M;
+  const int64_t total = (int64_t)M.n_ado * M.d * M.d;
+  if constexpr (sizeof(R) == 8)
+    if (M.d >= kKickTiledMinD) {
+      kick_tiled(T, outI, KI, M.d, M.n_ado, false, st);
+      kick_tiled(T, outII, KII, M.d, M.n_ado, true, st);
+      LAUNCH_CHECK();
+      return;
+    }
+  kick2_pair_kernel<R><<<grid_for(total), 256, 0, st>>>(T, outI, outII, KI, KII, M.d, total);
   count_launch(1);
   LAUNCH_CHECK();
 }
@@ -400,11 +423,8 @@ void response_2d_rows_impl(heom_hier *h, const heom_state *eq, const heom_grid *
     steps((C *)T.p, (C *)ta.p, (C *)tb.p, 1, (int64_t)(jr0 + j0) * m, trunk_prec);
     for (int j = 0; j < nj; ++j) {
       if (j > 0) steps((C *)T.p, (C *)ta.p, (C *)tb.p, 1, m, trunk_prec);
-      kick2_pair_kernel<R><<<grid_for(per_branch), 256, 0, st>>>(
-          (const C *)T.p, BR + (int64_t)j * per_branch, BR + (int64_t)(nj + j) * per_branch,
-          mu_work<R>(h, 1), mu_work<R>(h, 2), M.d, per_branch);
-      count_launch(1);
-      LAUNCH_CHECK();
+      kick2_into<R>(h, (const C *)T.p, BR + (int64_t)j * per_branch, BR + (int64_t)(nj + j) * per_branch,
+                    mu_work<R>(h, 1), mu_work<R>(h, 2), st);
     }
     int64_t t_now = 0;
     if (sizeof(R) == 4 && M.precision == HEOM_TC) tc_reserve(h->tc, (int64_t)B * M.n_ado);
@@ -439,6 +459,10 @@ template void rk4_steps<double>(heom_hier *, double2 *, double2 *, double2 *, in
 template void rk4_steps<float>(heom_hier *, float2 *, float2 *, float2 *, int, double, int64_t, cudaStream_t, int);
 template void kick_into<double>(heom_hier *, const double2 *, double2 *, int, const double *, cudaStream_t);
 template void kick_into<float>(heom_hier *, const float2 *, float2 *, int, const float *, cudaStream_t);
+template void kick2_into<double>(heom_hier *, const double2 *, double2 *, double2 *, const double *, const double *,
+                                 cudaStream_t);
+template void kick2_into<float>(heom_hier *, const float2 *, float2 *, float2 *, const float *, const float *,
+                                cudaStream_t);
 template void trace_into<double>(heom_hier *, const double2 *, int, const double *, int, double2 *, int64_t, cudaStream_t);
 template void trace_into<float>(heom_hier *, const float2 *, int, const double *, int, double2 *, int64_t, cudaStream_t);
 template void response_2d_rows_impl<double>(heom_hier *, const heom_state *, const heom_grid *, int, int, double2 *);

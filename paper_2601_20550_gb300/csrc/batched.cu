@@ -123,11 +123,8 @@ static void response_2d_multi(heom_hier *const *hs, const heom_state *const *eqs
       for (int k = 0; k < n_sets; ++k) {
         const int64_t per = S[k].per;
         double2 *br = (double2 *)S[k].P[0]->p;
-        kick2_pair_kernel<double><<<grid_for(per), 256, 0, st>>>((const double2 *)S[k].T->p, br + (int64_t)j * per,
-                                                                br + (int64_t)(nj + j) * per, mu_work<double>(S[k].h, 1),
-                                                                mu_work<double>(S[k].h, 2), S[k].h->M.d, per);
-        count_launch(1);
-        LAUNCH_CHECK();
+        kick2_into<double>(S[k].h, (const double2 *)S[k].T->p, br + (int64_t)j * per, br + (int64_t)(nj + j) * per,
+                           mu_work<double>(S[k].h, 1), mu_work<double>(S[k].h, 2), st);
       }
     }
     int64_t t_now = 0;

@@ -460,10 +460,8 @@ extern "C" heom_status heom_response_2d_grad(heom_hier *h, const heom_state *rho
         double2 *t1 = (double2 *)tmp.p, *t2b = (double2 *)tmp2.p;
         // forward: second kick of both pathways, t2, third kick
         for (int j = 0; j < nj; ++j) {
-          kick2_pair_kernel<double><<<grid_for(per), 256, 0, st>>>(T + (int64_t)(j0 + j) * per, br + (int64_t)j * per,
-                                                                  br + (int64_t)(nj + j) * per, mu_grad(h, 1), mu_grad(h, 2), d, per);
-          count_launch(1);
-          LAUNCH_CHECK();
+          kick2_into<double>(h, T + (int64_t)(j0 + j) * per, br + (int64_t)j * per, br + (int64_t)(nj + j) * per,
+                             mu_grad(h, 1), mu_grad(h, 2), st);
         }
         CUDA_TRY(cudaMemcpyAsync(t1, br, (size_t)B * sz1, cudaMemcpyDeviceToDevice, st));   // F = G^{n2} BR
         steps64(c, t1, c.W4, c.W3, B, dt, n2[it]);

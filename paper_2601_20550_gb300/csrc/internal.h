@@ -251,6 +251,10 @@ void rk4_steps(heom_hier *h, typename CxT<R>::type *y, typename CxT<R>::type *wa
 template <typename R>
 void kick_into(heom_hier *h, const typename CxT<R>::type *in, typename CxT<R>::type *out, int branches, const R *K,
                cudaStream_t st);
+// outI = KI^x T, outII = KII^x (-T^dagger), one branch each.
+template <typename R>
+void kick2_into(heom_hier *h, const typename CxT<R>::type *T, typename CxT<R>::type *outI,
+                typename CxT<R>::type *outII, const R *KI, const R *KII, cudaStream_t st);
 // i^order tr{mu rho_0} of each branch into out[branch * ostride].
 template <typename R>
 void trace_into(heom_hier *h, const typename CxT<R>::type *w, int branches, const double *mu, int order, double2 *out,

@@ -1,4 +1,5 @@
 // Non-template kernels: 2D Fourier sums / correlation spectrum and state conversion.
+#include "fixed54.cuh"
 #include "kernels.cuh"
 
 namespace heom {
@@ -65,6 +66,138 @@ void dft2d_sc(const double2 *RI, const double2 *RII, int n1, int n3, double dtau
   dft_rows_kernel<<<dim3((unsigned)n1, pb, 2), 128, 0, st>>>(RI, RII, tw3, n1, n3, F);
   dft_cols_kernel<<<dim3((unsigned)n1, pb), 128, 0, st>>>(F, tw1, n1, n3, dtau, SC);
   count_launch(3);
+}
+
+// Block = 32 x 32 entries of one item, 2 x 2 per thread; 16-wide slices of the contraction
+// index in shared memory as fixed point against the slice's largest exponents, one FP64
+// addition per slice and component.
+template <bool kDagger>
+static __global__ void __launch_bounds__(256, 3) kick64_kernel(const double2 *__restrict__ w, double2 *__restrict__ out,
+                                                               const double *__restrict__ K, int d, int tiles) {
+  constexpr int kTile = 32, kSlice = 16, kLd = kSlice + 1, kPer = kTile * kSlice / 256;
+  // K[p][k], w[k][q], then -K[k][q], w[p][k]
+  __shared__ __align__(16) int4 w1[2 * kTile * kLd];
+  __shared__ __align__(16) int2 k1[2 * kTile * kLd];
+  __shared__ int top[2][2];
+  const int64_t item = blockIdx.x / (tiles * tiles);
+  const int tile = (int)(blockIdx.x - item * tiles * tiles);
+  const int p0 = (tile / tiles) * kTile, q0 = (tile % tiles) * kTile;
+  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+  const double2 *wi = w + item * d * d;
+  auto at = [&](int r, int c) {
+    if (!kDagger) return wi[(int64_t)r * d + c];
+    const double2 v = wi[(int64_t)c * d + r];
+    return make_double2(-v.x, v.y);
+  };
+  const double2 z = make_double2(0.0, 0.0);
+  double2 sum[2][2] = {{z, z}, {z, z}};
+  if (t < 4) top[t >> 1][t & 1] = 1;
+  __syncthreads();
+  int par = 0;
+  for (int k0 = 0; k0 < d; k0 += kSlice, par ^= 1) {
+    double2 x[2][kPer];
+    double m[2][kPer];
+    int ek = 1, ew = 1;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      const int e = t + 256 * i, k = k0 + e % kSlice, r = e / kSlice;       // along rows
+      const int r2 = e % kTile, k2 = k0 + e / kTile;                        // along columns
+      m[0][i] = k < d && p0 + r < d ? K[(int64_t)(p0 + r) * d + k] : 0.0;
+      m[1][i] = k2 < d && q0 + r2 < d ? -K[(int64_t)k2 * d + q0 + r2] : 0.0;
+      // the item is read along its own rows: w[k][q] by columns of the tile, or by rows of w^dagger
+      x[0][i] = !kDagger ? (k2 < d && q0 + r2 < d ? at(k2, q0 + r2) : z) : (k < d && q0 + r < d ? at(k, q0 + r) : z);
+      x[1][i] = !kDagger ? (k < d && p0 + r < d ? at(p0 + r, k) : z) : (k2 < d && p0 + r2 < d ? at(p0 + r2, k2) : z);
+    }
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      ek = max(ek, max(exponent(make_double2(m[0][i], m[1][i])), 1));
+      ew = max(ew, max(exponent(x[0][i]), exponent(x[1][i])));
+    }
+    ek = __reduce_max_sync(0xffffffffu, ek);
+    ew = __reduce_max_sync(0xffffffffu, ew);
+    if ((t & 31) == 0) {
+      atomicMax(&top[par][0], ek);
+      atomicMax(&top[par][1], ew);
+    }
+    __syncthreads();   // the last slice's sums are done too
+    ek = top[par][0];
+    ew = top[par][1];
+    if (t < 2) top[par ^ 1][t] = 1;
+    if (ek == 0x7ff || ew == 0x7ff) {   // infinities or NaN: as they are
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int p = p0 + ty + 16 * i, q = q0 + tx + 16 * j;
+          if (p >= d || q >= d) continue;
+          for (int k = k0; k < min(d, k0 + kSlice); ++k) {
+            const double2 u = at(k, q), v = at(p, k);
+            const double l = K[(int64_t)p * d + k], r = K[(int64_t)k * d + q];
+            sum[i][j].x += l * u.x - v.x * r;
+            sum[i][j].y += l * u.y - v.y * r;
+          }
+        }
+      __syncthreads();
+      continue;
+    }
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      const int e = t + 256 * i, a = e / kSlice * kLd + e % kSlice, b = e % kTile * kLd + e / kTile;
+      k1[a] = fixed54(m[0][i], ek);
+      k1[kTile * kLd + b] = fixed54(m[1][i], ek);
+      w1[kDagger ? a : b] = fixed54(x[0][i], ew);
+      w1[kTile * kLd + (kDagger ? b : a)] = fixed54(x[1][i], ew);
+    }
+    __syncthreads();
+    long long hh[2][2][2] = {}, hl[2][2][2] = {};
+    auto mad = [&](int i, int j, const int2 &k, const int4 &x) {
+      hh[i][j][0] += (long long)k.x * x.x;
+      hl[i][j][0] += (long long)k.x * x.y;
+      hl[i][j][0] += (long long)k.y * x.x;
+      hh[i][j][1] += (long long)k.x * x.z;
+      hl[i][j][1] += (long long)k.x * x.w;
+      hl[i][j][1] += (long long)k.y * x.z;
+    };
+#pragma unroll 2
+    for (int k = 0; k < kSlice; ++k) {
+      const int2 kp[2] = {k1[ty * kLd + k], k1[(ty + 16) * kLd + k]};
+      const int4 xq[2] = {w1[tx * kLd + k], w1[(tx + 16) * kLd + k]};
+      const int2 kq[2] = {k1[(kTile + tx) * kLd + k], k1[(kTile + tx + 16) * kLd + k]};
+      const int4 xp[2] = {w1[(kTile + ty) * kLd + k], w1[(kTile + ty + 16) * kLd + k]};
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          mad(i, j, kp[i], xq[j]);
+          mad(i, j, kq[j], xp[i]);
+        }
+    }
+    const Unit54 unit(ek, ew);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        sum[i][j].x = unit.add(hh[i][j][0], hl[i][j][0], sum[i][j].x);
+        sum[i][j].y = unit.add(hh[i][j][1], hl[i][j][1], sum[i][j].y);
+      }
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int p = p0 + ty + 16 * i, q = q0 + tx + 16 * j;
+      if (p < d && q < d) out[(item * d + p) * d + q] = sum[i][j];
+    }
+}
+
+void kick_tiled(const double2 *w, double2 *out, const double *K, int d, int64_t items, bool dagger, cudaStream_t st) {
+  const int tiles = (d + 31) / 32;
+  const unsigned blocks = (unsigned)(items * tiles * tiles);   // below 2^31: a tile has 8 KB of device memory or more
+  if (dagger)
+    kick64_kernel<true><<<blocks, 256, 0, st>>>(w, out, K, d, tiles);
+  else
+    kick64_kernel<false><<<blocks, 256, 0, st>>>(w, out, K, d, tiles);
+  count_launch(1);
 }
 
 __global__ void dft1d_kernel(const double2 *__restrict__ R, int n, double dtau, double *__restrict__ I) {

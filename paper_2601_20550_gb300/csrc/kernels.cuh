@@ -141,6 +141,13 @@ __global__ void __launch_bounds__(256) kick_kernel(const typename CxT<R>::type *
   }
 }
 
+// The same for FP64 states through shared-memory tiles in integer products (fixed54.cuh),
+// and with dagger for -w^dagger in place of w.  One thread per entry needs 4 d FP64
+// multiply-adds of its own; it is as fast below d = 40 and few items (28 items: 22 against
+// 28 us at d = 36, 40 against 28 us at d = 40).  d = 216: 25.5 to 5.5 ms per 224 items.
+constexpr int kKickTiledMinD = 40;
+void kick_tiled(const double2 *w, double2 *out, const double *K, int d, int64_t items, bool dagger, cudaStream_t st);
+
 // Second kick of both pathways from one t1 trunk sample (Sec. II.C procedure):
 // the non-rephasing trunk equals -(rephasing trunk)^dagger ADO by ADO because the
 // equilibrium ADOs are Hermitian and Eq. HEOM_DB commutes with the dagger.
