@@ -251,17 +251,18 @@ void rk4_steps(heom_hier *h, typename CxT<R>::type *y, typename CxT<R>::type *wa
       if (!tc_supported(h->tc)) throw Fail{HEOM_EINVAL, "tensor-core path not prepared for this hierarchy"};
       tc_rk4_steps(h->tc, fy, fa, fb, branches, dt, nsteps, st);
     } else if (h->M.d >= kVbTiledMinD) {
-      // larger bases: the commutator tiled through shared memory, one block per
-      // 32 x 32 output tile of one item
-      const int tiles = (h->M.d + 31) / 32;
-      const int64_t nb = (int64_t)branches * h->M.n_ado * tiles * tiles;
-      if (nb > 0x7fffffffLL) throw Fail{HEOM_EINVAL, "too many tiles for one launch"};
+      // larger bases: the commutator tiled through shared memory (the same bits either way)
+      const int64_t items = (int64_t)branches * h->M.n_ado;
+      auto stage = [&](const float2 *w, float2 *out, double alpha) {
+        stage32(w, fy, out, (float)alpha, h->vb, items, st);
+      };
+      if (items * ((h->M.d + 31) / 32) * ((h->M.d + 31) / 32) > 0x7fffffffLL)
+        throw Fail{HEOM_EINVAL, "too many tiles for one launch"};
       for (int64_t s = 0; s < nsteps; ++s) {
-        stage_kernel_vb_tiled<<<(unsigned)nb, 256, 0, st>>>(fy, fy, fa, (float)(dt / 4), h->vb, tiles);
-        stage_kernel_vb_tiled<<<(unsigned)nb, 256, 0, st>>>(fa, fy, fb, (float)(dt / 3), h->vb, tiles);
-        stage_kernel_vb_tiled<<<(unsigned)nb, 256, 0, st>>>(fb, fy, fa, (float)(dt / 2), h->vb, tiles);
-        stage_kernel_vb_tiled<<<(unsigned)nb, 256, 0, st>>>(fa, fy, fy, (float)dt, h->vb, tiles);
-        count_launch(4);
+        stage(fy, fa, dt / 4);
+        stage(fa, fb, dt / 3);
+        stage(fb, fa, dt / 2);
+        stage(fa, fy, dt);
       }
     } else {
       const auto sh = tuned_shape(h, kTuneStageVb, total, st, {256, grid_for(total)}, grid_shapes(total),
@@ -292,12 +293,11 @@ void kick_into(heom_hier *h, const typename CxT<R>::type *in, typename CxT<R>::t
                       int branches, const R *K, cudaStream_t st) {
   const Model &M = h->M;
   const int64_t total = (int64_t)branches * M.n_ado * M.d * M.d;
-  if constexpr (sizeof(R) == 8)
-    if (M.d >= kKickTiledMinD) {
-      kick_tiled(in, out, K, M.d, (int64_t)branches * M.n_ado, false, st);
-      LAUNCH_CHECK();
-      return;
-    }
+  if (M.d >= kKickTiledMinD) {
+    kick_tiled(in, out, K, M.d, (int64_t)branches * M.n_ado, false, st);
+    LAUNCH_CHECK();
+    return;
+  }
   kick_kernel<R><<<grid_for(total), 256, 0, st>>>(in, out, K, M.d, total);
   count_launch(1);
   LAUNCH_CHECK();
@@ -308,13 +308,12 @@ void kick2_into(heom_hier *h, const typename CxT<R>::type *T, typename CxT<R>::t
                 typename CxT<R>::type *outII, const R *KI, const R *KII, cudaStream_t st) {
   const Model &M = h->M;
   const int64_t total = (int64_t)M.n_ado * M.d * M.d;
-  if constexpr (sizeof(R) == 8)
-    if (M.d >= kKickTiledMinD) {
-      kick_tiled(T, outI, KI, M.d, M.n_ado, false, st);
-      kick_tiled(T, outII, KII, M.d, M.n_ado, true, st);
-      LAUNCH_CHECK();
-      return;
-    }
+  if (M.d >= kKickTiledMinD) {
+    kick_tiled(T, outI, KI, M.d, M.n_ado, false, st);
+    kick_tiled(T, outII, KII, M.d, M.n_ado, true, st);
+    LAUNCH_CHECK();
+    return;
+  }
   kick2_pair_kernel<R><<<grid_for(total), 256, 0, st>>>(T, outI, outII, KI, KII, M.d, total);
   count_launch(1);
   LAUNCH_CHECK();

@@ -218,10 +218,7 @@ static void response_2d_multi_tc(heom_hier *const *hs, const heom_state *const *
       float2 *br = (float2 *)S[k].P[0]->p;
       for (int j = 0; j < nj; ++j) {
         if (j > 0) rk4_steps<float>(h, T, (float2 *)S[k].ta->p, (float2 *)S[k].tb->p, 1, dt, m, st, HEOM_FP32);
-        kick2_pair_kernel<float><<<grid_for(per), 256, 0, st>>>(T, br + (int64_t)j * per, br + (int64_t)(nj + j) * per,
-                                                               h->mup_vb32, h->mum_vb32, h->M.d, per);
-        count_launch(1);
-        LAUNCH_CHECK();
+        kick2_into<float>(h, T, br + (int64_t)j * per, br + (int64_t)(nj + j) * per, h->mup_vb32, h->mum_vb32, st);
       }
     }
     int64_t t_now = 0;

@@ -331,6 +331,238 @@ __global__ void __launch_bounds__(256) stage_kernel_vb_tiled(const float2 *__res
   }
 }
 
+// FP32 commutators K w - w K in register tiles: block = 64 x 64 entries of one item, 4 x 4
+// per thread (a warp: 16 rows, 32 columns), 32-wide slices of the contraction index through
+// a double buffer in shared memory (cp.async).  Along k the entries by row are read four
+// (K) or two (w) at a time, the entries by column two columns at a time: 24 shared loads
+// per 384 arithmetic instructions, against 10 per 24 with one column and four rows per
+// thread.  Every entry's operations and their order are those of stage_kernel_vb_tiled and
+// kick_kernel<float> (per term a product, a multiply-add and an addition), so the bits are
+// the same.
+constexpr int kC32Tile = 64, kC32Slice = 32;
+constexpr int kC32LdKr = 36, kC32LdWr = 68, kC32LdKc = 68, kC32LdWc = 132;   // in floats
+constexpr int kC32Kr = 0, kC32Wr = kC32Kr + kC32Tile * kC32LdKr, kC32Kc = kC32Wr + kC32Tile * kC32LdWr;
+constexpr int kC32Wc = kC32Kc + kC32Slice * kC32LdKc, kC32Buf = kC32Wc + kC32Slice * kC32LdWc;
+constexpr int kC32Smem = 2 * kC32Buf * 4;
+
+template <int kBytes>
+__device__ __forceinline__ void cp_async(float *dst, const void *src, bool ok) {   // zeros if not ok
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
+               "l"(src), "n"(kBytes), "r"(ok ? kBytes : 0));
+}
+
+// kOp: 0 out = K w - w K; 1 the same of -w^dagger; 2 RK4 stage of stage_kernel_vb
+template <int kOp>
+__global__ void __launch_bounds__(256, 2) comm32_kernel(const float2 *__restrict__ w, const float2 *y, float2 *out,
+                                                        const float *__restrict__ K, int d, int tiles, float alpha,
+                                                        const __grid_constant__ VbModel M) {
+  extern __shared__ __align__(16) float c32_smem[];
+  const int64_t dd = (int64_t)d * d, item = blockIdx.x / (tiles * tiles);
+  const int tile = (int)(blockIdx.x - item * tiles * tiles);
+  const int p0 = (tile / tiles) * kC32Tile, q0 = (tile % tiles) * kC32Tile;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int wp = (warp >> 1) * 16 + (lane >> 3), wq = (warp & 1) * 32 + (lane & 7) * 2;   // rows wp + 4 i
+  const float2 *wn = w + item * dd;
+  // w by rows: w[p][k] (kOp 1: w[q][k]); w by columns: w[k][q] (kOp 1: w[k][p])
+  const int r0 = kOp == 1 ? q0 : p0, c0 = kOp == 1 ? p0 : q0;
+  auto load = [&](int k0, float *b) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = (t >> 5) + 8 * i, k = k0 + lane;
+      const bool kp = p0 + r < d && k < d, wr = r0 + r < d && k < d;
+      cp_async<4>(b + kC32Kr + r * kC32LdKr + lane, K + (kp ? (p0 + r) * d + k : 0), kp);
+      cp_async<8>(b + kC32Wr + r * kC32LdWr + 2 * lane, wn + (wr ? (r0 + r) * d + k : 0), wr);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int c = t & 63, r = (t >> 6) + 4 * i, k = k0 + r;
+      const bool kq = q0 + c < d && k < d, wc = c0 + c < d && k < d;
+      cp_async<4>(b + kC32Kc + r * kC32LdKc + c, K + (kq ? k * d + q0 + c : 0), kq);
+      cp_async<8>(b + kC32Wc + r * kC32LdWc + 2 * c, wn + (wc ? k * d + c0 + c : 0), wc);
+    }
+    asm volatile("cp.async.commit_group;");
+  };
+  float2 sum[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) sum[i][j] = make_float2(0.f, 0.f);
+  const bool idle = p0 + (warp >> 1) * 16 >= d || q0 + (warp & 1) * 32 >= d;
+  load(0, c32_smem);
+  for (int k0 = 0, par = 0; k0 < d; k0 += kC32Slice, par ^= 1) {
+    if (k0 + kC32Slice < d) {
+      load(k0 + kC32Slice, c32_smem + (par ^ 1) * kC32Buf);
+      asm volatile("cp.async.wait_group 1;");
+    } else {
+      asm volatile("cp.async.wait_group 0;");
+    }
+    __syncthreads();
+    const float *b = c32_smem + par * kC32Buf;
+    const int end = idle ? 0 : min(kC32Slice, d - k0);
+    for (int k = 0; k < end; k += 4) {
+      float h[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float4 v = *(const float4 *)(b + kC32Kr + (wp + 4 * i) * kC32LdKr + k);
+        h[i][0] = v.x;
+        h[i][1] = v.y;
+        h[i][2] = v.z;
+        h[i][3] = v.w;
+      }
+#pragma unroll
+      for (int k2 = 0; k2 < 4; k2 += 2) {
+        float4 wr[4];   // two k of the four rows (kOp 1: of the four columns)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = kOp == 1 ? wq + (i & 1) + 16 * (i >> 1) : wp + 4 * i;
+          wr[i] = *(const float4 *)(b + kC32Wr + r * kC32LdWr + 2 * (k + k2));
+        }
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk) {
+          const float *kc = b + kC32Kc + (k + k2 + kk) * kC32LdKc + wq;
+          const float *wc = b + kC32Wc + (k + k2 + kk) * kC32LdWc;
+          const float2 ga = *(const float2 *)kc, gb = *(const float2 *)(kc + 16);
+          const float g[4] = {ga.x, ga.y, gb.x, gb.y};
+          float2 v[4], u[4];   // by row, by column
+#pragma unroll
+          for (int i = 0; i < 4; ++i) v[i] = kk ? make_float2(wr[i].z, wr[i].w) : make_float2(wr[i].x, wr[i].y);
+          if (kOp == 1) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) u[i] = *(const float2 *)(wc + 2 * (wp + 4 * i));
+          } else {
+            const float4 ua = *(const float4 *)(wc + 2 * wq), ub = *(const float4 *)(wc + 2 * wq + 32);
+            u[0] = make_float2(ua.x, ua.y);
+            u[1] = make_float2(ua.z, ua.w);
+            u[2] = make_float2(ub.x, ub.y);
+            u[3] = make_float2(ub.z, ub.w);
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float k1 = h[i][k2 + kk], k2_ = g[j];
+              if (kOp == 1) {
+                sum[i][j].x += __fmaf_rn(u[i].x, k2_, -__fmul_rn(k1, v[j].x));
+                sum[i][j].y += __fmaf_rn(k1, v[j].y, -__fmul_rn(u[i].y, k2_));
+              } else {
+                sum[i][j].x += __fmaf_rn(k1, u[j].x, -__fmul_rn(v[i].x, k2_));
+                sum[i][j].y += __fmaf_rn(k1, u[j].y, -__fmul_rn(v[i].y, k2_));
+              }
+            }
+        }
+      }
+    }
+    __syncthreads();
+  }
+  // through shared memory, so that a warp's accesses to memory are along rows
+  float2 *tilebuf = (float2 *)c32_smem;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      tilebuf[(wp + 4 * i) * kC32Tile + wq + (j & 1) + 16 * (j >> 1)] = sum[i][j];
+  __syncthreads();
+  const int b = q0 + (t & 63);
+  if (b >= d) return;
+  const int n = kOp == 2 ? (int)(item % M.n_ado) : 0;
+  const float2 *wb = wn - n * dd;
+  const float dec = kOp == 2 ? (float)M.decay[n] : 0.f;
+  constexpr int kRows = 8;
+  auto couple = [](float2 &o, float2 x, float p, float q) {
+    o.x += p * x.x + q * x.y;
+    o.y += p * x.y - q * x.x;
+  };
+#pragma unroll 1
+  for (int g = 0; g < 64 / 4 / kRows; ++g) {
+    const int row = (t >> 6) + 4 * kRows * g;   // rows row + 4 i
+    if (p0 + row >= d) break;
+    float2 o[kRows];
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) o[i] = tilebuf[(row + 4 * i) * kC32Tile + (t & 63)];
+    if (kOp == 2) {
+      int el[kRows];
+#pragma unroll
+      for (int i = 0; i < kRows; ++i) {
+        el[i] = min(p0 + row + 4 * i, d - 1) * d + b;
+        const float2 self = wn[el[i]];
+        o[i] = make_float2(o[i].y - dec * self.x, -o[i].x - dec * self.y);
+      }
+      for (int s = 0; s < M.n_modes; ++s) {
+        const int o0 = M.nb_off[n * M.n_modes + s], o1 = M.nb_off[n * M.n_modes + s + 1];
+        if (o0 == o1) continue;
+        const float lb = M.lam[s * d + b];
+        float f[kRows], gg[kRows];
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) {
+          const float la = M.lam[s * d + min(p0 + row + 4 * i, d - 1)];
+          f[i] = la - lb;
+          gg[i] = la + lb;
+        }
+        int q = o0;
+        for (; q + 1 < o1; q += 2) {
+          const float2 *xn = wb + (int64_t)M.nb_idx[q] * dd, *xn2 = wb + (int64_t)M.nb_idx[q + 1] * dd;
+          const float cA = M.nb_cA[q], cB = M.nb_cB[q], cA2 = M.nb_cA[q + 1], cB2 = M.nb_cB[q + 1];
+          float2 xv[kRows], xv2[kRows];
+#pragma unroll
+          for (int i = 0; i < kRows; ++i) {
+            xv[i] = xn[el[i]];
+            xv2[i] = xn2[el[i]];
+          }
+#pragma unroll
+          for (int i = 0; i < kRows; ++i) {
+            couple(o[i], xv[i], cB * gg[i], cA * f[i]);
+            couple(o[i], xv2[i], cB2 * gg[i], cA2 * f[i]);
+          }
+        }
+        if (q < o1) {
+          const float2 *xn = wb + (int64_t)M.nb_idx[q] * dd;
+          const float cA = M.nb_cA[q], cB = M.nb_cB[q];
+          float2 xv[kRows];
+#pragma unroll
+          for (int i = 0; i < kRows; ++i) xv[i] = xn[el[i]];
+#pragma unroll
+          for (int i = 0; i < kRows; ++i) couple(o[i], xv[i], cB * gg[i], cA * f[i]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+      const int a = p0 + row + 4 * i;
+      if (a >= d) break;
+      const int64_t e = item * dd + (int64_t)a * d + b;
+      if (kOp == 2) {
+        const float2 yv = y[e];
+        out[e] = make_float2(yv.x + alpha * o[i].x, yv.y + alpha * o[i].y);
+      } else {
+        out[e] = o[i];
+      }
+    }
+  }
+}
+
+template <int kOp>
+static void comm32(const float2 *w, const float2 *y, float2 *out, const float *K, int d, int64_t items, float alpha,
+                   const VbModel &M, cudaStream_t st) {
+  const int tiles = (d + kC32Tile - 1) / kC32Tile;
+  cudaFuncSetAttribute(comm32_kernel<kOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, kC32Smem);
+  comm32_kernel<kOp><<<(unsigned)(items * tiles * tiles), 256, kC32Smem, st>>>(w, y, out, K, d, tiles, alpha, M);
+  count_launch(1);
+}
+
+void kick_tiled(const float2 *w, float2 *out, const float *K, int d, int64_t items, bool dagger, cudaStream_t st) {
+  dagger ? comm32<1>(w, nullptr, out, K, d, items, 0.f, VbModel{}, st)
+         : comm32<0>(w, nullptr, out, K, d, items, 0.f, VbModel{}, st);
+}
+
+void stage32(const float2 *w, const float2 *y, float2 *out, float alpha, const VbModel &M, int64_t items,
+             cudaStream_t st) {
+  const int64_t tiles = (M.d + kC32Tile - 1) / kC32Tile;
+  if (M.d >= 36 && items * tiles * tiles >= 152) return comm32<2>(w, y, out, M.H, M.d, items, alpha, M, st);
+  const int t32 = (M.d + 31) / 32;
+  stage_kernel_vb_tiled<<<(unsigned)(items * t32 * t32), 256, 0, st>>>(w, y, out, alpha, M, t32);
+  count_launch(1);
+}
+
 __global__ void convert_f64_to_f32(const double2 *__restrict__ x, float2 *__restrict__ y, int64_t n) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = make_float2((float)x[i].x, (float)x[i].y);
