@@ -33,14 +33,15 @@ void count_launch(uint64_t n);
 
 namespace {
 
-// Threads of a panel block: three blocks' registers fit an SM without spills, and the
-// row groups of the usual sizes (2 x 25 at five levels, 36 at six) divide evenly.
+// Columns (rows) of a panel, and the most threads of its block.
+constexpr int kPanel = 16;
 __host__ __device__ constexpr int panel_threads(int R) { return R == 5 ? 320 : 384; }
+__host__ __device__ constexpr int panel_blocks(int R) { return R == 4 ? 2 : 3; }   // per SM, of that many
 constexpr int kF64MaxExp = 16;             // build_hierarchy's limit
 constexpr int kRotPad = 33;
 constexpr int kSmallD = 32;                // largest basis of f64_small_kernel
 constexpr size_t kMaxSmem = 227 * 1024;
-// Whole-item blocks up to two per SM; above, one panel of 32 columns (rows) per block.
+// Whole-item blocks up to two per SM; above, one panel of columns (rows) per block.
 constexpr size_t kFusedSmem = 112 * 1024;
 
 struct F64Set {
@@ -338,8 +339,9 @@ __global__ void __launch_bounds__(256, 4) f64_item_kernel(const __grid_constant_
 // first: it lives on the FP64 pipe and the products on the IMAD pipe, and blocks that
 // start together would otherwise wait for the same pipe all the time.
 // ---------------------------------------------------------------------------
-template <int R, int kPanel, bool kRight, bool kMulti>
-__global__ void __launch_bounds__(panel_threads(R), 3) f64_panel_kernel(const __grid_constant__ F64Args P) {
+template <int R, bool kRight, bool kMulti>
+__global__ void __launch_bounds__(panel_threads(R), panel_blocks(R))
+    f64_panel_kernel(const __grid_constant__ F64Args P) {
   extern __shared__ __align__(16) uint8_t smem[];
   const F64Set &S = pick<kMulti>(P);
   const F64Ops &O = S.O;
@@ -411,30 +413,28 @@ __global__ void __launch_bounds__(panel_threads(R), 3) f64_panel_kernel(const __
   const bool early = kRight && ((unsigned)lb * 2654435761u >> 31);
   if (early) elementwise(S.tp + item * dd);
   __syncthreads();
-  // one task: a row group and 16 complex columns, lane = (column, component)
-  constexpr int kHalves = kPanel / 16;
-  const int comp = lane & 1;
-  for (int k = warp; k < kHalves * O.groups; k += warps) {
-    const int g = k / kHalves, col = (k % kHalves) * 16 + (lane >> 1);
+  // one task: a row group and the 16 complex columns, lane = (column, component)
+  const int comp = lane & 1, col = lane >> 1;
+  for (int g = warp; g < O.groups; g += warps) {
     Acc<R> A;
     group_product<R>(O, g, reinterpret_cast<const int2 *>(zs + col) + comp, 2 * ld, A);
     if (col < np) {
       // -i alpha (x + i y) = alpha (y - i x): the real sum goes to the imaginary part
       const Unit f = unit(lexp[col], O.hexp, comp == (kRight ? 1 : 0) ? -ah : ah);
       double *t = reinterpret_cast<double *>((early ? S.out : S.tp) + item * dd) + (comp ^ 1);
+      double v[R], old[R];
+      double *o = t + 2 * (kRight ? (int64_t)(p0 + col) * d + g * R : (int64_t)g * R * d + p0 + col);
+      const int step = kRight ? 2 : 2 * d, live = min(R, d - g * R);
+#pragma unroll
+      for (int r = 0; r < R; ++r) old[r] = kRight && r < live ? o[r * step] : 0.0;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        const int x = g * R + r;
-        if (x < d) {
-          const double v = sum_value(finish(A, r, O.bits - 31), f);
-          if (!kRight) {
-            t[2 * ((int64_t)x * d + p0 + col)] = f.f * v;
-          } else {
-            double *o = t + 2 * ((int64_t)(p0 + col) * d + x);
-            *o = fma(f.f, v, *o);
-          }
-        }
+        v[r] = sum_value(finish(A, r, O.bits - 31), f);
+        v[r] = kRight ? fma(f.f, v[r], old[r]) : f.f * v[r];
       }
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        if (r < live) o[r * step] = v[r];
     }
   }
   if (kRight && !early) {
@@ -978,7 +978,7 @@ int table_size(const Model &M) {
   return t;
 }
 
-size_t panel_smem(int d, int tab, int panel) { return (size_t)tab * 16 + (size_t)d * (panel + 1) * 16; }
+size_t panel_smem(int d, int tab) { return (size_t)tab * 16 + (size_t)d * (kPanel + 1) * 16; }
 
 size_t fused_smem(int d, int tab, int m, bool t) {
   return (size_t)tab * 16 + (size_t)m * d * (d | 1) * 16 * (t ? 2 : 1) + (size_t)m * (sizeof(List) + 4) + 64;
@@ -996,15 +996,20 @@ int row_group(const Model &M) {
   return n % 5 == 0 ? 5 : n % 3 == 0 ? 6 : 4;
 }
 
-// Columns (rows) per block of the panel kernels, or 0 for whole items.  An item keeps one
-// SM busy for 70 us at d = 64 and 150 us at d = 80, so a launch with fewer than four
-// items per SM spreads each over panels; 16 columns where 32 would leave fewer than
-// three blocks on an SM or fewer blocks than two per SM.
-int panel_width(int d, int tab, int64_t items) {
+// Panels instead of whole items?  An item keeps one SM busy for 70 us at d = 64 and 150 us
+// at d = 80, so a launch with fewer than four items per SM spreads each over panels.
+bool use_panels(int d, int tab, int64_t items) {
+  return fused_smem(d, tab, 1, false) > kFusedSmem || (d >= 48 && items < 4 * sm_count());
+}
+
+// Threads of a panel block: small blocks are out of step with one another, so that the
+// products of some (IMAD pipe) run beside the elementwise part of others (FP64 pipe), and
+// the row groups divide evenly (25 at five levels, 16 at four); big ones where a launch
+// has few blocks or a basis that leaves room for three.
+int panel_shape(int R, int64_t blocks) {
   const int sms = sm_count();
-  if (fused_smem(d, tab, 1, false) <= kFusedSmem && (d < 48 || items >= 4 * sms)) return 0;
-  if (3 * (panel_smem(d, tab, 32) + 2048) > kMaxSmem || items * ((d + 31) / 32) < 2 * sms) return 16;
-  return 32;
+  if (R == 5) return blocks >= 4 * sms ? 160 : 320;
+  return R == 4 && blocks >= 2 * sms ? 256 : 384;
 }
 
 // Items per block of the whole-item kernel: enough columns for two to four warps of
@@ -1016,7 +1021,7 @@ int items_per_block(int d, int tab, int64_t items) {
   return m;
 }
 
-F64Set make_set(const F64Buf &b, int64_t begin, int *panel, size_t *smem, int64_t *blocks) {
+F64Set make_set(const F64Buf &b, int64_t begin, bool *panels, size_t *smem, int64_t *blocks) {
   const F64Ops &O = *b.ops;
   F64Set s{};
   s.O = O;
@@ -1026,15 +1031,15 @@ F64Set make_set(const F64Buf &b, int64_t begin, int *panel, size_t *smem, int64_
   s.tp = b.tp;
   s.begin = begin;
   s.items = (int64_t)b.branches * O.n_ado;
-  *panel = panel_width(O.d, O.tab, s.items);
-  if (*panel == 0) {
+  *panels = use_panels(O.d, O.tab, s.items);
+  if (!*panels) {
     s.per_block = items_per_block(O.d, O.tab, s.items);
     s.smem_t = fused_smem(O.d, O.tab, s.per_block, true) <= 56 * 1024;
     *smem = fused_smem(O.d, O.tab, s.per_block, s.smem_t);
     *blocks = (s.items + s.per_block - 1) / s.per_block;
   } else {
-    s.per_block = (O.d + *panel - 1) / *panel;
-    *smem = panel_smem(O.d, O.tab, *panel);
+    s.per_block = (O.d + kPanel - 1) / kPanel;
+    *smem = panel_smem(O.d, O.tab);
     *blocks = s.items * s.per_block;
   }
   return s;
@@ -1045,35 +1050,32 @@ void allow_smem(K kernel, size_t smem) {
   if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
-template <int R, int kPanel, bool kMulti>
-void launch_panels(const F64Args &a, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
-  allow_smem(f64_panel_kernel<R, kPanel, false, kMulti>, smem);
-  allow_smem(f64_panel_kernel<R, kPanel, true, kMulti>, smem);
-  f64_panel_kernel<R, kPanel, false, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
-  f64_panel_kernel<R, kPanel, true, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
-  count_launch(2);
-}
-
 template <int R, bool kMulti>
-void launch_r(const F64Args &a, int panel, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
-  if (panel == 32) return launch_panels<R, 32, kMulti>(a, blocks, smem, threads, st);
-  if (panel == 16) return launch_panels<R, 16, kMulti>(a, blocks, smem, threads, st);
+void launch_r(const F64Args &a, bool panels, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
+  if (panels) {
+    allow_smem(f64_panel_kernel<R, false, kMulti>, smem);
+    allow_smem(f64_panel_kernel<R, true, kMulti>, smem);
+    f64_panel_kernel<R, false, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
+    f64_panel_kernel<R, true, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
+    count_launch(2);
+    return;
+  }
   allow_smem(f64_item_kernel<R, kMulti>, smem);
   f64_item_kernel<R, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
   count_launch(1);
 }
 
-void launch(const F64Args &a, int R, int panel, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
+void launch(const F64Args &a, int R, bool panels, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
   if (blocks == 0) return;
   if (blocks > 0x7fffffffLL) throw std::invalid_argument("too many work items for one stage launch");
   auto with = [&](auto multi) {
     constexpr bool m = decltype(multi)::value;
     if (R == 4)
-      launch_r<4, m>(a, panel, blocks, smem, threads, st);
+      launch_r<4, m>(a, panels, blocks, smem, threads, st);
     else if (R == 5)
-      launch_r<5, m>(a, panel, blocks, smem, threads, st);
+      launch_r<5, m>(a, panels, blocks, smem, threads, st);
     else
-      launch_r<6, m>(a, panel, blocks, smem, threads, st);
+      launch_r<6, m>(a, panels, blocks, smem, threads, st);
   };
   if (a.n > 0)
     with(std::true_type());
@@ -1085,7 +1087,7 @@ void launch(const F64Args &a, int R, int panel, int64_t blocks, size_t smem, int
 
 bool f64_supported(const Model &M) {
   const int tab = table_size(M);
-  if (M.n_exp > kF64MaxExp || M.n_modes > kF64MaxModes || tab > kF64MaxTab || panel_smem(M.d, tab, 16) + sizeof(List) + 256 > kMaxSmem) return false;
+  if (M.n_exp > kF64MaxExp || M.n_modes > kF64MaxModes || tab > kF64MaxTab || panel_smem(M.d, tab) + sizeof(List) + 256 > kMaxSmem) return false;
   if (row_products(M) > 500) return false;   // the 64-bit sums stay exact
   for (double h : M.vb_H)
     if (!std::isfinite(h)) return false;
@@ -1226,23 +1228,25 @@ F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::
 }
 
 std::vector<std::pair<int, int>> f64_shapes(const F64Buf &b) {
-  int panel = 0;
+  bool panels = false;
   size_t smem = 0;
   int64_t blocks = 0;
-  make_set(b, 0, &panel, &smem, &blocks);
+  make_set(b, 0, &panels, &smem, &blocks);
   const int n = (int)std::min<int64_t>(blocks, 0x7fffffff);
-  if (panel == 0) return {{256, n}, {128, n}, {64, n}};
-  return {{panel_threads(b.ops->R), n}, {256, n}, {192, n}};
+  if (!panels) return {{256, n}, {128, n}, {64, n}};
+  const int t = panel_shape(b.ops->R, blocks);
+  return b.ops->R == 5 ? std::vector<std::pair<int, int>>{{t, n}, {480 - t, n}}
+                       : std::vector<std::pair<int, int>>{{t, n}, {640 - t, n}, {128, n}};
 }
 
 void f64_stage(const F64Buf &b, double alpha, int threads, cudaStream_t st) {
-  int panel = 0;
+  bool panels = false;
   size_t smem = 0;
   int64_t blocks = 0;
   F64Args a{};
-  a.one = make_set(b, 0, &panel, &smem, &blocks);
+  a.one = make_set(b, 0, &panels, &smem, &blocks);
   a.alpha = alpha;
-  launch(a, b.ops->R, panel, blocks, smem, threads, st);
+  launch(a, b.ops->R, panels, blocks, smem, threads, st);
 }
 
 namespace {
@@ -1422,18 +1426,18 @@ void f64_plan(F64Plan &p, const std::vector<F64Buf> &sets, cudaStream_t st) {
   std::map<std::pair<int, int>, std::vector<F64Set>> by;
   std::map<std::pair<int, int>, std::pair<int64_t, size_t>> size;
   for (const F64Buf &b : sets) {
-    int panel = 0;
+    bool panels = false;
     size_t smem = 0;
     int64_t blocks = 0;
-    F64Set s = make_set(b, 0, &panel, &smem, &blocks);
-    auto key = std::make_pair(b.ops->R, panel);
+    F64Set s = make_set(b, 0, &panels, &smem, &blocks);
+    auto key = std::make_pair(b.ops->R, (int)panels);
     s.begin = size[key].first;
     size[key].first += blocks;
     size[key].second = std::max(size[key].second, smem);
     by[key].push_back(s);
   }
   for (auto &kv : by) {
-    F64Plan::Class c{kv.first.first, kv.first.second, size[kv.first].first, size[kv.first].second,
+    F64Plan::Class c{kv.first.first, kv.first.second != 0, size[kv.first].first, size[kv.first].second,
                      (int)kv.second.size(), nullptr};
     if (device_malloc(&c.desc, kv.second.size() * sizeof(F64Set)) != cudaSuccess) {
       (void)cudaGetLastError();
@@ -1451,7 +1455,7 @@ void f64_stage_plan(const F64Plan &p, double alpha, cudaStream_t st) {
     a.many = (const F64Set *)c.desc;
     a.n = c.n;
     a.alpha = alpha;
-    launch(a, c.R, c.panel, c.blocks, c.smem, c.panel == 0 ? 256 : panel_threads(c.R), st);
+    launch(a, c.R, c.panels, c.blocks, c.smem, c.panels ? panel_shape(c.R, c.blocks) : 256, st);
   }
 }
 

@@ -104,7 +104,7 @@ bool f64_small_steps_plan(const F64SmallPlan &p, double dt, int64_t steps, cudaS
 struct F64Plan {
   struct Class {   // sets of one kernel variant
     int R;
-    int panel;   // columns per block, 0: whole items
+    bool panels;
     int64_t blocks;
     size_t smem;
     int n;
