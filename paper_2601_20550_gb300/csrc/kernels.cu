@@ -336,7 +336,9 @@ __global__ void __launch_bounds__(256) stage_kernel_vb_tiled(const float2 *__res
 // a double buffer in shared memory (cp.async).  Along k the entries by row are read four
 // (K) or two (w) at a time, the entries by column two columns at a time: 24 shared loads
 // per 384 arithmetic instructions, against 10 per 24 with one column and four rows per
-// thread.  Every entry's operations and their order are those of stage_kernel_vb_tiled and
+// thread; real and imaginary part take one packed instruction each time, which leaves half
+// the issue slots (d = 125, 924 items: stage 715 to 646 us, kick 490 to 461; the FP32
+// pipe's rate alone would take 340).  Every entry's operations and their order are those of stage_kernel_vb_tiled and
 // kick_kernel<float> (per term a product, a multiply-add and an addition), so the bits are
 // the same.
 constexpr int kC32Tile = 64, kC32Slice = 32;
@@ -349,6 +351,33 @@ template <int kBytes>
 __device__ __forceinline__ void cp_async(float *dst, const void *src, bool ok) {   // zeros if not ok
   asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
                "l"(src), "n"(kBytes), "r"(ok ? kBytes : 0));
+}
+
+// Two FP32 operations per instruction, each rounded as its scalar form.
+__device__ __forceinline__ unsigned long long pack2(float x, float y) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
 }
 
 // kOp: 0 out = K w - w K; 1 the same of -w^dagger; 2 RK4 stage of stage_kernel_vb
@@ -382,21 +411,13 @@ __global__ void __launch_bounds__(256, 2) comm32_kernel(const float2 *__restrict
     }
     asm volatile("cp.async.commit_group;");
   };
-  float2 sum[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) sum[i][j] = make_float2(0.f, 0.f);
+  unsigned long long sum[4][4] = {};   // complex, packed
   const bool idle = p0 + (warp >> 1) * 16 >= d || q0 + (warp & 1) * 32 >= d;
   load(0, c32_smem);
   for (int k0 = 0, par = 0; k0 < d; k0 += kC32Slice, par ^= 1) {
-    if (k0 + kC32Slice < d) {
-      load(k0 + kC32Slice, c32_smem + (par ^ 1) * kC32Buf);
-      asm volatile("cp.async.wait_group 1;");
-    } else {
-      asm volatile("cp.async.wait_group 0;");
-    }
-    __syncthreads();
+    asm volatile("cp.async.wait_group 0;");
+    __syncthreads();   // this slice is there, and nobody reads the last one any more
+    if (k0 + kC32Slice < d) load(k0 + kC32Slice, c32_smem + (par ^ 1) * kC32Buf);
     const float *b = c32_smem + par * kC32Buf;
     const int end = idle ? 0 : min(kC32Slice, d - k0);
     for (int k = 0; k < end; k += 4) {
@@ -441,26 +462,28 @@ __global__ void __launch_bounds__(256, 2) comm32_kernel(const float2 *__restrict
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
               const float k1 = h[i][k2 + kk], k2_ = g[j];
-              if (kOp == 1) {
-                sum[i][j].x += __fmaf_rn(u[i].x, k2_, -__fmul_rn(k1, v[j].x));
-                sum[i][j].y += __fmaf_rn(k1, v[j].y, -__fmul_rn(u[i].y, k2_));
+              if (kOp == 1) {   // the real part's product is the other one
+                float2 s = unpack2(sum[i][j]);
+                s.x += __fmaf_rn(u[i].x, k2_, -__fmul_rn(k1, v[j].x));
+                s.y += __fmaf_rn(k1, v[j].y, -__fmul_rn(u[i].y, k2_));
+                sum[i][j] = pack2(s.x, s.y);
               } else {
-                sum[i][j].x += __fmaf_rn(k1, u[j].x, -__fmul_rn(v[i].x, k2_));
-                sum[i][j].y += __fmaf_rn(k1, u[j].y, -__fmul_rn(v[i].y, k2_));
+                sum[i][j] = add2(sum[i][j], fma2(pack2(k1, k1), pack2(u[j].x, u[j].y),
+                                                 mul2(pack2(v[i].x, v[i].y), pack2(-k2_, -k2_))));
               }
             }
         }
       }
     }
-    __syncthreads();
   }
+  __syncthreads();
   // through shared memory, so that a warp's accesses to memory are along rows
   float2 *tilebuf = (float2 *)c32_smem;
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-      tilebuf[(wp + 4 * i) * kC32Tile + wq + (j & 1) + 16 * (j >> 1)] = sum[i][j];
+      tilebuf[(wp + 4 * i) * kC32Tile + wq + (j & 1) + 16 * (j >> 1)] = unpack2(sum[i][j]);
   __syncthreads();
   const int b = q0 + (t & 63);
   if (b >= d) return;

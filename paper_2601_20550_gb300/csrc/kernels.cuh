@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(256) kick_kernel(const typename CxT<R>::type *
 // entry reads 4 d values for 4 d multiply-adds of its own; it is as fast below d = 40 and
 // few items (FP64, 28 items: 22 against 28 us at d = 36, 40 against 28 us at d = 40;
 // FP32, 28 items: 14 against 17 us at d = 64, but 924 items 183 against 73 us).  d = 216:
-// FP64 25.5 to 5.5 ms per 224 items, FP32 7.7 to 2.7 ms per 924.
+// FP64 25.5 to 5.5 ms per 224 items, FP32 7.7 to 2.5 ms per 924.
 constexpr int kKickTiledMinD = 40;
 void kick_tiled(const double2 *w, double2 *out, const double *K, int d, int64_t items, bool dagger, cudaStream_t st);
 void kick_tiled(const float2 *w, float2 *out, const float *K, int d, int64_t items, bool dagger, cudaStream_t st);
@@ -278,7 +278,7 @@ constexpr int kVbTiledMinD = 24;
 __global__ void __launch_bounds__(256) stage_kernel_vb_tiled(const float2 *__restrict__ w, const float2 *y,
                                                              float2 *out, float alpha, VbModel M, int tiles);
 // Launches the tiled stage: 64 x 64 tiles in registers (comm32_kernel) for d >= 36 with a
-// block for every SM (d = 125, 924 items: 882 to 726 us; d = 100: 832 to 568), 32 x 32
+// block for every SM (d = 125, 924 items: 880 to 646 us; d = 100: 830 to 500), 32 x 32
 // otherwise (d = 64, 28 items: 20 against 29 us; d = 24, 924 items: 32 against 39 us).
 void stage32(const float2 *w, const float2 *y, float2 *out, float alpha, const VbModel &M, int64_t items,
              cudaStream_t st);
