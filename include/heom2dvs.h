@@ -220,9 +220,11 @@ heom_status heom_steady_state(heom_hier *h, double tol, int restart, int max_ite
 /*
  * Launch shapes chosen by the library's autotuner (no counterpart in the paper:
  * a tuning aid).  The first RK4 propagation of a given size on the FP64
- * (kind 0) or FP32 coupling-basis (kind 1) path times nine launch shapes of its
- * stage kernel (64/128/256 threads x 4/16/64 blocks per SM) on the real operands
- * and keeps the fastest; results do not depend on the shape.  On the
+ * (kind 0) or FP32 coupling-basis (kind 1) path times the launch shapes of its
+ * stage kernel on the real operands (two or three block sizes of the FP64 stages;
+ * 64/128/256 threads x 4/16/64 blocks per SM of the grid-stride kernels) and keeps
+ * the fastest; results do not depend on the shape.  FP64 hierarchies small enough
+ * for all steps in one launch have one shape; the tiled FP32 stages none.  On the
  * tensor-core path (kind 2) the tensor-core kernel keeps one shape (one
  * persistent 544-thread CTA per SM, bounded by its shared and tensor memory);
  * the coupling kernel that follows it is tuned over seventeen shapes (2, 4, 8 or
@@ -268,8 +270,9 @@ heom_status heom_response_2d_grad(heom_hier *h, const heom_state *rho_eq, const 
  * single-branch FP64 equilibrium) on one grid: outputs [n_sets][n_t2][n1][n3]
  * with the layouts of heom_response_2d (any output may be NULL).  When every
  * set is an HEOM_FP64 hierarchy, the sets advance together: each RK4 stage of
- * all sets and all their branches is one kernel launch (per-set models and
- * state pointers in a descriptor table), and each t3 scan is one CUDA-graph
+ * all sets and all their branches is one launch per kernel variant that they take
+ * (per-set tables and state pointers in a descriptor table; one launch for all
+ * steps if every basis has at most 32 states), and each t3 scan is one CUDA-graph
  * replay.  When every set is an HEOM_TC hierarchy (up to 16 sets), each RK4
  * stage of the t2 forks and t3 scans of all sets is one tensor-core launch and
  * one coupling-kernel launch (per-set operators and buffers in the launch's

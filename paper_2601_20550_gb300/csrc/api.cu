@@ -78,8 +78,8 @@ void stability_check(heom_hier *h, double dt) {
 // Launch-shape autotuner of the stage kernels.  The first launch of a kernel kind
 // at a given size times every candidate (grid_shapes: blocks of 64, 128 or 256
 // threads, 4, 16 or 64 blocks per SM, capped at one element per thread, for the
-// grid-stride kernels; three block sizes of the FP64 engine, whose grid follows from the
-// size) on the real operands -- three timed launches each after one untimed --
+// grid-stride kernels; two or three block sizes of the FP64 engine, whose grid follows
+// from the size) on the real operands -- three timed launches each after one untimed --
 // and keeps the fastest for this hierarchy; a size whose default launch already takes over
 // 50 ms keeps the default.  Candidate launches repeat the caller's first
 // stage, whose output is scratch that the step overwrites next, so tuning

@@ -1,5 +1,6 @@
 // Several parameter sets on one grid (heom_response_2d_batched): FP64 sets
-// advance together, one launch per RK4 stage across all sets and branches;
+// advance together, one launch per RK4 stage and kernel variant across all sets and
+// branches (small bases: one launch for all steps);
 // tensor-core sets likewise, one launch pair per stage.
 #include <algorithm>
 #include <cmath>

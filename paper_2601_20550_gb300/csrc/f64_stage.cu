@@ -337,7 +337,9 @@ __global__ void __launch_bounds__(256, 4) f64_item_kernel(const __grid_constant_
 // right one, which adds i alpha w H' and the elementwise rest of those rows.  Limbs
 // scaled per column (row).  Half of the right kernel's blocks take the elementwise part
 // first: it lives on the FP64 pipe and the products on the IMAD pipe, and blocks that
-// start together would otherwise wait for the same pipe all the time.
+// start together would otherwise wait for the same pipe all the time.  d = 125, 924 items:
+// 827 us (IMAD pipe 70 % busy) and 1540 us (FP64 pipe 64 %); one thread per element in the
+// product basis took 17.4 ms.
 // ---------------------------------------------------------------------------
 template <int R, bool kRight, bool kMulti>
 __global__ void __launch_bounds__(panel_threads(R), panel_blocks(R))
@@ -996,16 +998,24 @@ int row_group(const Model &M) {
   return n % 5 == 0 ? 5 : n % 3 == 0 ? 6 : 4;
 }
 
-// Panels instead of whole items?  An item keeps one SM busy for 70 us at d = 64 and 150 us
-// at d = 80, so a launch with fewer than four items per SM spreads each over panels.
+// Panels instead of whole items?  An item keeps one SM busy for 40 us at d = 36, 70 us at
+// d = 64 and 150 us at d = 80, so a launch with few items per SM spreads each over panels:
+// fewer than four per SM from d = 46 on, 1.5 at d = 36.  Two steps at d = 36, 28 items: 359
+// against 503 us, 196 items 580 against 709, 280 items 796 against 742; d = 45, 252 items:
+// 847 against 985, 588 items 1603 against 1548; one stage at d = 64, 3360 items: 1839
+// against 1737.
 bool use_panels(int d, int tab, int64_t items) {
-  return fused_smem(d, tab, 1, false) > kFusedSmem || (d >= 48 && items < 4 * sm_count());
+  return fused_smem(d, tab, 1, false) > kFusedSmem ||
+         (d > kSmallD && items < (int64_t)sm_count() * std::min(d - 30, 16) / 4);
 }
 
 // Threads of a panel block: small blocks are out of step with one another, so that the
 // products of some (IMAD pipe) run beside the elementwise part of others (FP64 pipe), and
 // the row groups divide evenly (25 at five levels, 16 at four); big ones where a launch
-// has few blocks or a basis that leaves room for three.
+// has few blocks or a basis that leaves room for three.  d = 125, 924 items: 160 threads
+// 827 + 1540 us, 320 854 + 1669 us; d = 64, 896 blocks: 256 threads 48 + 98 us, 384 53 +
+// 103 us; 112 blocks: 21 + 37 and 21 + 35 us; d = 216, 1920 blocks: 384 threads 460 + 596
+// us, 192 639 + 798 us.
 int panel_shape(int R, int64_t blocks) {
   const int sms = sm_count();
   if (R == 5) return blocks >= 4 * sms ? 160 : 320;
