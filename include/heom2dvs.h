@@ -272,7 +272,7 @@ heom_status heom_response_2d_grad(heom_hier *h, const heom_state *rho_eq, const 
  * set is an HEOM_FP64 hierarchy, the sets advance together: each RK4 stage of
  * all sets and all their branches is one launch per kernel variant that they take
  * (per-set tables and state pointers in a descriptor table; one launch for all
- * steps if every basis has at most 32 states), and each t3 scan is one CUDA-graph
+ * steps if every basis has at most 48 states), and each t3 scan is one CUDA-graph
  * replay.  When every set is an HEOM_TC hierarchy (up to 16 sets), each RK4
  * stage of the t2 forks and t3 scans of all sets is one tensor-core launch and
  * one coupling-kernel launch (per-set operators and buffers in the launch's

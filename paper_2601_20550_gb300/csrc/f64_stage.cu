@@ -39,7 +39,10 @@ __host__ __device__ constexpr int panel_threads(int R) { return R == 5 ? 320 : 3
 __host__ __device__ constexpr int panel_blocks(int R) { return R == 4 ? 2 : 3; }   // per SM, of that many
 constexpr int kF64MaxExp = 16;             // build_hierarchy's limit
 constexpr int kRotPad = 33;
-constexpr int kSmallD = 32;                // largest basis of f64_small_kernel
+// Largest basis of f64_small_kernel and rotate_item_kernel (row and column in six bits).
+// Two steps at d = 36, 7 ADOs: 142 us in one launch, 352 with a launch per stage; 84
+// items: 324 and 441 us.
+constexpr int kSmallD = 48;
 constexpr size_t kMaxSmem = 227 * 1024;
 // Whole-item blocks up to two per SM; above, one panel of columns (rows) per block.
 constexpr size_t kFusedSmem = 112 * 1024;
@@ -868,7 +871,7 @@ __global__ void __launch_bounds__(256) rotate_item_kernel(const double2 *x, doub
     const double2 t = reinterpret_cast<double2 *>(v)[(k / d) * ld + k % d];
     const int2 re = to_limbs(t.x, e1, 60, 30), im = to_limbs(t.y, e1, 60, 30);
     const float a = (float)(abs(re.x) + 1) * (1.f / (1 << 29)), b = (float)(abs(im.x) + 1) * (1.f / (1 << 29));
-    q += (unsigned)((a * a + b * b) * 262144.f) + 2u;   // up to 1024 elements: below 2^30
+    q += (unsigned)((a * a + b * b) * 262144.f) + 2u;   // up to 2304 elements: below 2^31
   }
   atomicAdd(&s_sum, q);
   __syncthreads();
@@ -1006,7 +1009,7 @@ int row_group(const Model &M) {
 // against 1737.
 bool use_panels(int d, int tab, int64_t items) {
   return fused_smem(d, tab, 1, false) > kFusedSmem ||
-         (d > kSmallD && items < (int64_t)sm_count() * std::min(d - 30, 16) / 4);
+         (d > 32 && items < (int64_t)sm_count() * std::min(d - 30, 16) / 4);
 }
 
 // Threads of a panel block: small blocks are out of step with one another, so that the

@@ -1,5 +1,5 @@
 """The FP64 engine (coupling basis, integer commutator) at the sizes where its variants
-change: bases up to 32 (all steps in one launch; one block, one cluster or the whole grid
+change: bases up to 48 (all steps in one launch; one block, one cluster or the whole grid
 per branch), whole items in shared memory, panels of 32 columns, ragged row groups and
 panels, several items per block, single-level modes.
 
@@ -51,6 +51,7 @@ def propagated(model, x, steps, dt=0.25):
     ((4, 4, 5), 1, 1, 1), ((3, 4, 7), 1, 1, 1), ((1, 9, 9), 1, 1, 1),     # 80, 84, 81
     ((5, 17), 1, 1, 1), ((4, 5, 5), 1, 1, 2), ((2, 8, 8), 1, 1, 1),       # panels: 85 (dense basis change), 100, 128
     ((3, 7, 8), 1, 1, 1),                                                 # 168: ragged last panel
+    ((5, 7), 1, 1, 1), ((3, 4, 4), 1, 1, 1), ((3, 4, 3), 2, 1, 3), ((7, 7), 1, 1, 2),   # 33 to 48 in one launch; 49
 ])
 def test_propagation(levels, depth, K, branches):
     model = model_of(levels, depth, K)
