@@ -23,6 +23,7 @@
 
 #include <cooperative_groups.h>
 
+#include "launch_math.h"
 #include "tc_stage.h"   // device_malloc, DeviceOom
 
 namespace cg = cooperative_groups;
@@ -329,8 +330,8 @@ __global__ void __launch_bounds__(256, 4) f64_item_kernel(const __grid_constant_
     const Unit f = unit(iexp[i], O.hexp, ah);
     const double2 y = S.y ? S.y[item * dd + el] : make_double2(0.0, 0.0);
     const double2 t = make_double2(fma(f.f, sum_value(c.y, f), y.x), fma(-f.f, sum_value(c.x, f), y.y));
-    const double2 *wb = S.w + (item - n) * dd;
-    S.out[item * dd + el] = couple(O, tab, lists[i], wb, wb + n * dd, dd, a, b, el, t, alpha * O.decay[n]);
+    S.out[item * dd + el] = couple(O, tab, lists[i], S.w + ado_offset(item - n, d), S.w + ado_offset(item, d), dd, a, b,
+                                   el, t, alpha * O.decay[n]);
   }
 }
 
@@ -402,7 +403,7 @@ __global__ void __launch_bounds__(panel_threads(R), panel_blocks(R))
   }
   // the elementwise rest of the panel's rows on top of from
   auto elementwise = [&](const double2 *from) {
-    const double2 *wb = S.w + (item - n) * dd;
+    const double2 *wb = S.w + ado_offset(item - n, d);
     const double2 *y = S.y ? S.y + item * dd : nullptr;
     const double adec = alpha * O.decay[n];
     for (int k = threadIdx.x; k < np * d; k += blockDim.x) {
@@ -502,9 +503,9 @@ __global__ void __launch_bounds__(512) f64_small_kernel(const __grid_constant__ 
   const int n_units = (kSync == 2 ? P.branches : 1) * O.n_ado * P.parts;
   const int u0 = min(n_units, (blk % P.bpb) * P.units);
   const int nu = min(P.units, n_units - u0);
-  const int first = kSync == 2 ? 0 : (blk / P.bpb) * O.n_ado;   // first item of the branch
-  const int i0 = first + u0 / P.parts;
-  const int ni = nu > 0 ? (first + (u0 + nu - 1) / P.parts - i0) + 1 : 0;      // items touched
+  const int64_t first = kSync == 2 ? 0 : (int64_t)(blk / P.bpb) * O.n_ado;   // first item of the branch
+  const int64_t i0 = first + u0 / P.parts;
+  const int ni = nu > 0 ? (u0 + nu - 1) / P.parts - u0 / P.parts + 1 : 0;      // items touched
   const int max_items = (P.units + P.parts - 1) / P.parts + (P.parts > 1 ? 1 : 0);
   double2 *tab = reinterpret_cast<double2 *>(smem);
   int4 *zs = reinterpret_cast<int4 *>(tab + O.tab);
@@ -518,12 +519,13 @@ __global__ void __launch_bounds__(512) f64_small_kernel(const __grid_constant__ 
   const int rows = (d + P.parts - 1) / P.parts;   // rows per part
   for (int i = warp; i < ni; i += warps) {
     SmallItem &I = items[i];
-    const int item = i0 + i, n = item % O.n_ado;
+    const int64_t item = i0 + i;
+    const int n = (int)(item % O.n_ado);
     const int *off = O.noff + n * nm;
     const int q0 = off[0], nq = off[nm] - q0;
     if (lane == 0) {
-      I.base = (int64_t)item * dd;
-      I.branch = (int64_t)(item - n) * dd;
+      I.base = ado_offset(item, d);
+      I.branch = ado_offset(item - n, d);
       I.decay = O.decay[n];
       I.n_nb = nq;
     }
@@ -544,7 +546,7 @@ __global__ void __launch_bounds__(512) f64_small_kernel(const __grid_constant__ 
   for (int k = threadIdx.x; k < nu * rows * d; k += blockDim.x) {
     const int u = k / (rows * d), r = k - u * rows * d, ug = u0 + u;
     const int a = (ug % P.parts) * rows + r / d, b = r % d;
-    elem[k] = (first + ug / P.parts - i0) << 12 | a << 6 | b;   // a may pass d in the last part: skipped
+    elem[k] = (ug / P.parts - u0 / P.parts) << 12 | a << 6 | b;   // a may pass d in the last part: skipped
   }
   for (int k = threadIdx.x; k < ni * dd; k += blockDim.x) {
     const int i = k / dd, el = k - i * dd;
@@ -552,7 +554,7 @@ __global__ void __launch_bounds__(512) f64_small_kernel(const __grid_constant__ 
   }
   __syncthreads();
   const int work = 2 * nu * rows * d, nz = ni * dd;
-  const int64_t z0 = (int64_t)i0 * dd;
+  const int64_t z0 = ado_offset(i0, d);
   int parity = 0;
   for (int64_t s = 0; s < G.steps; ++s)
     for (int q = 0; q < 4; ++q, parity ^= 1) {

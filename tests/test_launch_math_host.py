@@ -1,0 +1,38 @@
+"""Index arithmetic of the kernels and their launches (csrc/launch_math.h), compiled with
+the host compiler and compared with Python's integers at the sizes where 32 bits end."""
+import os
+import re
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2601_20550_gb300", "csrc")
+
+
+def run(tmp_path, body):
+    src, exe = tmp_path / "t.cpp", tmp_path / "t"
+    src.write_text('#include <cstdio>\n#include "launch_math.h"\nint main() {\n' + body + "\n}\n")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-fsanitize=undefined",
+                    "-fno-sanitize-recover=undefined", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    return subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()
+
+
+# hierarchies that fit one GPU and are accepted: 12 exponentials at depth 10 (42 GB a state),
+# d = 36 with 2042975 ADOs, and small bases with as many matrices
+@pytest.mark.parametrize("d,n_ado", [(64, 646646), (36, 2042975), (216, 24310), (6, 1 << 26), (1, 1 << 30)])
+def test_ado_offsets_pass_32_bits(tmp_path, d, n_ado):
+    ns = [0, 1, (1 << 31) // (d * d) - 1, (1 << 31) // (d * d), n_ado - 1]
+    out = run(tmp_path, "".join(f'  printf("%lld\\n", (long long)heom::ado_offset({n}, {d}));\n' for n in ns))
+    assert [int(v) for v in out] == [n * d * d for n in ns]
+
+
+def test_fp64_kernels_take_ado_offsets_from_there():
+    """No 32-bit index of an item (an ADO of a branch) in the FP64 kernels, and no 32-bit
+    product of an ADO index with d^2: an int dd appears only beside 64-bit indexes or within
+    one block's items."""
+    src = open(os.path.join(CSRC, "f64_stage.cu")).read()
+    for body in re.split(r"__global__", src)[1:]:
+        body = body.split("\n}\n", 1)[0]
+        assert not re.search(r"const int (first|i0|item)\b", body), body[:200]
+        if re.search(r"const int [^;]*\bdd = ", body):
+            assert not re.search(r"(?<![\w.])n \* dd\b", body), body[:200]
