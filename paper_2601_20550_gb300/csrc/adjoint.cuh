@@ -318,6 +318,7 @@ static __global__ void __launch_bounds__(256) coupling_grad_kernel(const double2
 // d = 64, 224 items: 1284 us with a warp reduction per neighbour and digit, 166 us here;
 // 28 items: 980 and 42 us (one block for all panels: 260 and 93 us).
 constexpr int kGradPanel = 16, kGradLd = kGradPanel + 1, kGradMaxN = 6;
+constexpr int kGradSmem = 226 * 1024;   // dynamic, beside 0.8 KB of static arrays
 
 struct CouplingGradArgs {
   const double2 *g, *w;

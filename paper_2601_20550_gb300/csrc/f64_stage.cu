@@ -23,14 +23,12 @@
 
 #include <cooperative_groups.h>
 
+#include "internal.h"
 #include "launch_math.h"
-#include "tc_stage.h"   // device_malloc, DeviceOom
 
 namespace cg = cooperative_groups;
 
 namespace heom {
-
-void count_launch(uint64_t n);
 
 namespace {
 
@@ -180,6 +178,11 @@ struct List {
   F64Entry e[2 * kF64MaxExp];
   int off[kF64MaxModes + 1];
 };
+
+// Dynamic shared memory that a launch may ask for, beside its kernel's own static arrays.
+constexpr size_t kStageSmem = kMaxSmem - sizeof(List) - 256;   // whole items, panels
+constexpr size_t kRotSmem = kMaxSmem - 512;
+constexpr size_t kSmallSmem = kMaxSmem - 1024;
 
 __device__ __forceinline__ void fill_list(const F64Ops &O, int n, List *L, int t, int nt) {
   const int *off = O.noff + n * O.n_modes;
@@ -1060,22 +1063,25 @@ F64Set make_set(const F64Buf &b, int64_t begin, bool *panels, size_t *smem, int6
   return s;
 }
 
+// The limit belongs to the kernel in its context, for every thread that launches it: always
+// the same value, never this launch's size.
 template <typename K>
-void allow_smem(K kernel, size_t smem) {
-  if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+void allow_smem(K kernel, size_t smem, size_t most) {
+  if (smem > 48 * 1024)
+    CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
 }
 
 template <int R, bool kMulti>
 void launch_r(const F64Args &a, bool panels, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
   if (panels) {
-    allow_smem(f64_panel_kernel<R, false, kMulti>, smem);
-    allow_smem(f64_panel_kernel<R, true, kMulti>, smem);
+    allow_smem(f64_panel_kernel<R, false, kMulti>, smem, kStageSmem);
+    allow_smem(f64_panel_kernel<R, true, kMulti>, smem, kStageSmem);
     f64_panel_kernel<R, false, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
     f64_panel_kernel<R, true, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
     count_launch(2);
     return;
   }
-  allow_smem(f64_item_kernel<R, kMulti>, smem);
+  allow_smem(f64_item_kernel<R, kMulti>, smem, kStageSmem);
   f64_item_kernel<R, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
   count_launch(1);
 }
@@ -1102,7 +1108,8 @@ void launch(const F64Args &a, int R, bool panels, int64_t blocks, size_t smem, i
 
 bool f64_supported(const Model &M) {
   const int tab = table_size(M);
-  if (M.n_exp > kF64MaxExp || M.n_modes > kF64MaxModes || tab > kF64MaxTab || panel_smem(M.d, tab) + sizeof(List) + 256 > kMaxSmem) return false;
+  if (M.n_exp > kF64MaxExp || M.n_modes > kF64MaxModes || tab > kF64MaxTab || panel_smem(M.d, tab) > kStageSmem)
+    return false;
   if (row_products(M) > 500) return false;   // the 64-bit sums stay exact
   for (double h : M.vb_H)
     if (!std::isfinite(h)) return false;
@@ -1288,7 +1295,7 @@ bool small_fit(F64SmallSet &p, SmallShape &sh) {
   const int rows = (O.d + p.parts - 1) / p.parts;
   const int64_t smem = O.tab * 16 + max_items * ((int64_t)O.d * (O.d | 1) * 16 + sizeof(SmallItem) + 8 + dd * 4) + dd * 8 +
                        2 * O.n_modes * O.d * 4 + (int64_t)p.units * rows * O.d * 4;
-  if (work > kSmallElems || smem > (int64_t)kMaxSmem - 1024 || n_units * dd > (1 << 30)) return false;
+  if (work > kSmallElems || smem > (int64_t)kSmallSmem || n_units * dd > (1 << 30)) return false;
   sh.smem = std::max(sh.smem, (size_t)smem);
   sh.threads = std::max(sh.threads, work <= 32 ? 64 : work <= 64 ? 128 : work <= 256 ? 256 : 512);
   sh.blocks += sh.sync == 2 ? p.bpb : p.branches * p.bpb;
@@ -1320,7 +1327,7 @@ bool launch_small(const F64SmallArgs &a, const SmallShape &sh, cudaStream_t st) 
   auto kernel = sh.sync == 0 ? f64_small_kernel<0, kMulti> : f64_small_kernel<1, kMulti>;
   if constexpr (!kMulti)
     if (sh.sync == 2) kernel = f64_small_kernel<2, false>;
-  allow_smem(kernel, sh.smem);
+  allow_smem(kernel, sh.smem, kSmallSmem);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)sh.blocks);
   cfg.blockDim = dim3((unsigned)sh.threads);
@@ -1329,7 +1336,7 @@ bool launch_small(const F64SmallArgs &a, const SmallShape &sh, cudaStream_t st) 
   cudaLaunchAttribute at{};
   cfg.attrs = &at;
   if (sh.sync == 1) {
-    if (sh.cluster > 8) cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (sh.cluster > 8) CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     at.id = cudaLaunchAttributeClusterDimension;
     at.val.clusterDim.x = (unsigned)sh.cluster;
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
@@ -1344,10 +1351,12 @@ bool launch_small(const F64SmallArgs &a, const SmallShape &sh, cudaStream_t st) 
     at.val.cooperative = 1;
     cfg.numAttrs = 1;
   }
-  if (cudaLaunchKernelEx(&cfg, kernel, a) != cudaSuccess) {
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a);
+  if (e == cudaErrorCooperativeLaunchTooLarge) {   // fewer SMs than the device's
     (void)cudaGetLastError();
     return false;
   }
+  CUDA_TRY(e);
   count_launch(1);
   return true;
 }
@@ -1475,7 +1484,7 @@ void f64_stage_plan(const F64Plan &p, double alpha, cudaStream_t st) {
 }
 
 bool rot_supported(const Model &M) {
-  if (M.n_modes > kF64MaxModes || (size_t)M.d * kRotPad * 16 + 512 > kMaxSmem) return false;
+  if (M.n_modes > kF64MaxModes || (size_t)M.d * kRotPad * 16 > kRotSmem) return false;
   for (int n : M.dims)
     if (n > kRotMaxN) return false;
   return true;
@@ -1525,8 +1534,8 @@ void rotate(const RotOps &r, bool forward, const double2 *x, double2 *out, doubl
     return;
   }
   const size_t smem = (size_t)r.d * kRotPad * 16;
-  allow_smem(rotate_kernel<false>, smem);
-  allow_smem(rotate_kernel<true>, smem);
+  allow_smem(rotate_kernel<false>, smem, kRotSmem);
+  allow_smem(rotate_kernel<true>, smem, kRotSmem);
   rotate_kernel<false><<<(unsigned)blocks, 256, smem, st>>>(x, tmp, u, r, panels);
   rotate_kernel<true><<<(unsigned)blocks, 256, smem, st>>>(tmp, out, u, r, panels);
   count_launch(2);

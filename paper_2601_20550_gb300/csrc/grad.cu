@@ -55,7 +55,7 @@ static void ensure_adjoint(heom_hier *h) {
   int nvl = 0;
   for (int s = 0; s < S; ++s) nvl += M.dims[s] * M.dims[s];
   if (nvl > kAdjMaxVl) throw Fail{HEOM_EINVAL, "mode bases too large for the gradient"};
-  bool work = h->f64.ready && (size_t)2 * M.d * kGradLd * 16 + 1024 <= 227 * 1024;
+  bool work = h->f64.ready && 2 * M.d * kGradLd * 16 <= kGradSmem;
   for (int n : M.dims) work = work && n <= kGradMaxN;
   std::vector<int> off((size_t)N * S + 1, 0), idx(M.nb_idx.size());
   std::vector<double> cA(M.nb_idx.size()), cB(M.nb_idx.size());
@@ -161,7 +161,8 @@ static void grad_pair(AdjCtx &c, const double2 *g, const double2 *w, int branche
     const int smem = 2 * M.d * kGradLd * 16;
     const auto kernel = *std::max_element(M.dims.begin(), M.dims.end()) > 4 ? coupling_grad_vb_kernel<kGradMaxN>
                                                                             : coupling_grad_vb_kernel<4>;
-    CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    // the kernel's limit is every thread's: always the same value
+    CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGradSmem));
     kernel<<<(unsigned)blocks, 256, smem, c.st>>>(a);
     count_launch(1);
     LAUNCH_CHECK();
