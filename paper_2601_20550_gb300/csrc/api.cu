@@ -91,8 +91,7 @@ static std::pair<int, int> tuned_shape(heom_hier *h, int kind, int64_t total, cu
                                        const std::pair<int, int> &dflt,
                                        const std::vector<std::pair<int, int>> &candidates,
                                        const std::function<void(int, int)> &launch) {
-  auto it = h->tuned.find({kind, total});
-  if (it != h->tuned.end()) return it->second;
+  if (const Shape *kept = kept_shape(h->tuned, kind, total, dflt, candidates)) return *kept;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return dflt;
   cudaEvent_t e0 = nullptr, e1 = nullptr;

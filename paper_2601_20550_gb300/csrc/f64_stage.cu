@@ -24,7 +24,6 @@
 #include <cooperative_groups.h>
 
 #include "internal.h"
-#include "launch_math.h"
 
 namespace cg = cooperative_groups;
 

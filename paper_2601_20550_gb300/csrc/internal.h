@@ -28,6 +28,7 @@
 #include "heom2dvs.h"
 #include "f64_stage.h"
 #include "kernels.cuh"
+#include "launch_math.h"
 #include "model.h"
 #include "tc_stage.h"
 
@@ -144,7 +145,7 @@ struct heom_hier {
   std::vector<heom_pair> desc_pairs;
   // adjoint RHS tables (built on the first gradient call)
   // launch shapes picked by the autotuner: (kernel kind, elements) -> (block, grid)
-  std::map<std::pair<int, int64_t>, std::pair<int, int>> tuned;
+  ShapeMap tuned;
   bool adj_ready = false, adj_work = false;   // adj_work: the gradient runs in the coupling basis
   DevModel<double> dm_adj{};
   int *adj_ado = nullptr, *adj_entry_exp = nullptr;

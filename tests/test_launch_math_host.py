@@ -36,3 +36,17 @@ def test_fp64_kernels_take_ado_offsets_from_there():
         assert not re.search(r"const int (first|i0|item)\b", body), body[:200]
         if re.search(r"const int [^;]*\bdd = ", body):
             assert not re.search(r"(?<![\w.])n \* dd\b", body), body[:200]
+
+
+def test_a_shape_kept_by_another_kernel_is_not_used(tmp_path):
+    """All steps in one launch (512 threads) and a launch per stage (at most 384) record their
+    shapes under one key; a stage takes a kept shape only if it is one of its own."""
+    out = run(tmp_path, """
+  heom::ShapeMap kept{{{0, 9072}, {512, 28}}, {{0, 100}, {128, 7}}, {{0, 200}, {256, 9}}};
+  const std::vector<heom::Shape> mine{{256, 7}, {128, 7}, {64, 7}};
+  printf("%d ", heom::kept_shape(kept, 0, 9072, mine[0], mine) != nullptr);
+  printf("%d ", heom::kept_shape(kept, 0, 100, mine[0], mine)->first);
+  printf("%d ", heom::kept_shape(kept, 0, 200, {256, 9}, mine)->second);
+  printf("%d ", heom::kept_shape(kept, 1, 100, mine[0], mine) != nullptr);
+  printf("%d", heom::kept_shape(kept, 0, 101, mine[0], mine) != nullptr);""")
+    assert out == ["0", "128", "9", "0", "0"]
