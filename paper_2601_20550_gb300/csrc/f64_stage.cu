@@ -167,9 +167,13 @@ __device__ __forceinline__ void group_product(const F64Ops &O, int g, const int2
 }
 
 // A sum as a 62-bit integer, units of 2^(2 low - 1).
+__device__ __forceinline__ long long finish(long long h, long long x, int low) {
+  return (h << 1) + ((x + (1LL << (low - 2))) >> (low - 1));
+}
+
 template <int R>
 __device__ __forceinline__ long long finish(const Acc<R> &A, int r, int low) {
-  return (A.h[r] << 1) + ((A.x[r] + (1LL << (low - 2))) >> (low - 1));
+  return finish(A.h[r], A.x[r], low);
 }
 
 // An ADO's coupling list in shared memory.
@@ -223,7 +227,7 @@ __device__ __forceinline__ double2 couple(const F64Ops &O, const double2 *tab, c
           const F64Entry &en = L.e[q + j];
           const bool first = q + j == q0;
           if (en.kind == 0) {
-            A = first ? x[j] : make_double2(A.x + x[j].x, A.y + x[j].y);
+            A = first ? x[j] : make_double2(__dadd_rn(A.x, x[j].x), __dadd_rn(A.y, x[j].y));
           } else {
             const double c = en.cA;
             A = first ? make_double2(c * x[j].x, c * x[j].y) : make_double2(fma(c, x[j].x, A.x), fma(c, x[j].y, A.y));
@@ -246,6 +250,16 @@ __device__ __forceinline__ double2 couple(const F64Ops &O, const double2 *tab, c
   return acc;
 }
 
+// y + alpha (L w)_{ab}: the elementwise rest (couple from zero, tab unscaled), the commutator
+// from its integer sums c (units of f), then alpha.  Whole items, their panels and the
+// small-hierarchy kernel compute an element with these operations in this order, on limbs
+// scaled by the item's largest exponent, so its bits depend neither on the launch nor on
+// what else is in the batch.
+__device__ __forceinline__ double2 element(double2 rest, longlong2 c, const Unit &f, double2 y, double alpha) {
+  return make_double2(fma(alpha, fma(f.f, sum_value(c.y, f), rest.x), y.x),
+                      fma(alpha, fma(-f.f, sum_value(c.x, f), rest.y), y.y));
+}
+
 // ---------------------------------------------------------------------------
 // Whole items per block: w's limbs (scaled per item) in shared memory with an odd row
 // stride, so that a warp reads 32 columns of a row or 32 rows of a column without bank
@@ -265,9 +279,8 @@ __global__ void __launch_bounds__(256, 4) f64_item_kernel(const __grid_constant_
   double2 *ts = reinterpret_cast<double2 *>(zs + m * isz);
   List *lists = reinterpret_cast<List *>(ts + (S.smem_t ? m * isz : 0));
   int *iexp = reinterpret_cast<int *>(lists + m);
-  const double alpha = P.alpha, ah = alpha * O.hsign;
   for (int i = threadIdx.x; i < m; i += blockDim.x) iexp[i] = 1;
-  fill_tab(O, alpha, tab);
+  fill_tab(O, 1.0, tab);
   __syncthreads();
   const double2 *w = S.w + i0 * dd;
   {
@@ -329,25 +342,34 @@ __global__ void __launch_bounds__(256, 4) f64_item_kernel(const __grid_constant_
     const int64_t item = i0 + i;
     const int n = (int)(item % O.n_ado);
     const longlong2 c = *reinterpret_cast<const longlong2 *>(S.smem_t ? ts + i * isz + a * ld + b : S.tp + item * dd + el);
-    const Unit f = unit(iexp[i], O.hexp, ah);
-    const double2 y = S.y ? S.y[item * dd + el] : make_double2(0.0, 0.0);
-    const double2 t = make_double2(fma(f.f, sum_value(c.y, f), y.x), fma(-f.f, sum_value(c.x, f), y.y));
-    S.out[item * dd + el] = couple(O, tab, lists[i], S.w + ado_offset(item - n, d), S.w + ado_offset(item, d), dd, a, b,
-                                   el, t, alpha * O.decay[n]);
+    const double2 zero = make_double2(0.0, 0.0);
+    const double2 rest = couple(O, tab, lists[i], S.w + ado_offset(item - n, d), S.w + ado_offset(item, d), dd, a, b, el,
+                                zero, O.decay[n]);
+    S.out[item * dd + el] =
+        element(rest, c, unit(iexp[i], O.hexp, O.hsign), S.y ? S.y[item * dd + el] : zero, P.alpha);
   }
 }
 
 // ---------------------------------------------------------------------------
-// One panel per block, for bases whose items do not fit and for launches with few
-// items: kPanel columns of w in the left kernel (tp = -i alpha H' w), kPanel rows in the
-// right one, which adds i alpha w H' and the elementwise rest of those rows.  Limbs
-// scaled per column (row).  Half of the right kernel's blocks take the elementwise part
-// first: it lives on the FP64 pipe and the products on the IMAD pipe, and blocks that
-// start together would otherwise wait for the same pipe all the time.  d = 125, 924 items:
-// 827 us (IMAD pipe 70 % busy) and 1540 us (FP64 pipe 64 %); one thread per element in the
-// product basis took 17.4 ms.
+// One panel per block: kPanel columns of w in the left kernel (tp = H' w), kPanel rows in
+// the right one, which takes w H' off and adds the elementwise rest of those rows.  Half of
+// the right kernel's blocks take the elementwise part first: it lives on the FP64 pipe and
+// the products on the IMAD pipe, and blocks that start together would otherwise wait for
+// the same pipe all the time.
+//
+// kItem: bases whose items fit a block (launches with few of them), with the arithmetic of
+// f64_item_kernel: limbs scaled by the whole item's largest exponent, which every block
+// finds for itself (d^2 loads that hit L2: 5 to 8 % of a launch of a few hundred items; one
+// cluster per item that shares it: as fast for 10 items, 2 to 12 % slower from 80 on); the
+// commutator's integers in tp; blocks that take the elementwise part first keep it in
+// shared memory.
+//
+// Otherwise: limbs scaled per column (row), tp = -i alpha H' w in FP64, on which the right
+// kernel adds in either order; ADO and panel decide, so that an element's additions have
+// one order wherever its branch stands.  d = 125, 924 items: 827 us and 1540 us; one thread
+// per element in the product basis took 17.4 ms.
 // ---------------------------------------------------------------------------
-template <int R, bool kRight, bool kMulti>
+template <int R, bool kRight, bool kMulti, bool kItem>
 __global__ void __launch_bounds__(panel_threads(R), panel_blocks(R))
     f64_panel_kernel(const __grid_constant__ F64Args P) {
   extern __shared__ __align__(16) uint8_t smem[];
@@ -361,14 +383,16 @@ __global__ void __launch_bounds__(panel_threads(R), panel_blocks(R))
   constexpr int ld = kRight ? kPanel + 1 : kPanel;
   double2 *tab = reinterpret_cast<double2 *>(smem);
   int4 *zs = reinterpret_cast<int4 *>(tab + O.tab);      // [d][ld]
-  __shared__ int lexp[kPanel];
+  double2 *rest = reinterpret_cast<double2 *>(zs + d * ld);   // kItem, early blocks: [kPanel][d | 1]
+  __shared__ int lexp[kPanel], turn;
   __shared__ List list;
   const double alpha = P.alpha, ah = alpha * O.hsign;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   if (threadIdx.x < kPanel) lexp[threadIdx.x] = 1;
   const int n = (int)(item % O.n_ado);
   if (kRight) {
-    fill_tab(O, alpha, tab);
+    if (threadIdx.x == 0) turn = (int)(((unsigned)n * (unsigned)d + (unsigned)p0) * 2654435761u >> 31);
+    fill_tab(O, kItem ? 1.0 : alpha, tab);
     fill_list(O, n, &list, threadIdx.x, blockDim.x);
   }
   __syncthreads();
@@ -382,7 +406,7 @@ __global__ void __launch_bounds__(panel_threads(R), panel_blocks(R))
       e = max(e, exp_field(v));
       reinterpret_cast<double2 *>(zs)[c * ld + col_t] = v;
     }
-    atomicMax(lexp + col_t, e);
+    if (!kItem) atomicMax(lexp + col_t, e);
   } else {
     for (int a = warp; a < kPanel; a += warps) {
       int e = 0;
@@ -391,48 +415,92 @@ __global__ void __launch_bounds__(panel_threads(R), panel_blocks(R))
         e = max(e, exp_field(v));
         reinterpret_cast<double2 *>(zs)[c * ld + a] = v;
       }
-      e = __reduce_max_sync(0xffffffffu, e);
-      if (lane == 0) lexp[a] = max(e, 1);
+      if (!kItem) {
+        e = __reduce_max_sync(0xffffffffu, e);
+        if (lane == 0) lexp[a] = max(e, 1);
+      }
     }
   }
+  if (kItem) {
+    int top = 0;
+#pragma unroll 4
+    for (int k = threadIdx.x; k < (int)dd; k += blockDim.x) top = max(top, exp_field(w[k]));
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (lane == 0) atomicMax(lexp, top);
+  }
   __syncthreads();
-  const int emax = lexp[col_t];
+  const int emax = lexp[kItem ? 0 : col_t];
   for (int c = row_t; c < d; c += rows_t) {
     int4 *p = zs + c * ld + col_t;
     const double2 v = *reinterpret_cast<double2 *>(p);
     const int2 re = to_limbs(v.x, emax, O.bits, O.bits - 31), im = to_limbs(v.y, emax, O.bits, O.bits - 31);
     *p = make_int4(re.x, re.y, im.x, im.y);
   }
-  // the elementwise rest of the panel's rows on top of from
-  auto elementwise = [&](const double2 *from) {
-    const double2 *wb = S.w + ado_offset(item - n, d);
+  const bool early = kRight && turn;
+  // the elementwise rest of the panel's rows: with the commutator in tp into out, or (kItem,
+  // early) alone into shared memory
+  auto elementwise = [&]() {
+    const double2 *wb = S.w + (item - n) * dd, *from = S.tp + item * dd;
     const double2 *y = S.y ? S.y + item * dd : nullptr;
-    const double adec = alpha * O.decay[n];
+    const double dec = kItem ? O.decay[n] : alpha * O.decay[n];
     for (int k = threadIdx.x; k < np * d; k += blockDim.x) {
       const int ar = k / d, el = p0 * d + k;
-      double2 acc = from[el];
-      if (y) {
-        const double2 yv = y[el];
-        acc = make_double2(acc.x + yv.x, acc.y + yv.y);
+      double2 acc = zero;
+      if (!kItem) {
+        acc = from[el];
+        if (y) {
+          const double2 yv = y[el];
+          acc = make_double2(acc.x + yv.x, acc.y + yv.y);
+        }
       }
-      S.out[item * dd + el] = couple(O, tab, list, wb, w, dd, p0 + ar, k - ar * d, el, acc, adec);
+      acc = couple(O, tab, list, wb, w, dd, p0 + ar, k - ar * d, el, acc, dec);
+      if (kItem && early)
+        rest[ar * (d | 1) + k - ar * d] = acc;
+      else if (kItem)
+        S.out[item * dd + el] = element(acc, *reinterpret_cast<const longlong2 *>(from + el),
+                                        unit(emax, O.hexp, O.hsign), y ? y[el] : zero, alpha);
+      else
+        S.out[item * dd + el] = acc;
     }
   };
-  const bool early = kRight && ((unsigned)lb * 2654435761u >> 31);
-  if (early) elementwise(S.tp + item * dd);
+  if (early) elementwise();
   __syncthreads();
   // one task: a row group and the 16 complex columns, lane = (column, component)
   const int comp = lane & 1, col = lane >> 1;
   for (int g = warp; g < O.groups; g += warps) {
     Acc<R> A;
     group_product<R>(O, g, reinterpret_cast<const int2 *>(zs + col) + comp, 2 * ld, A);
-    if (col < np) {
+    const int step = kRight ? 2 : 2 * d, live = col < np ? min(R, d - g * R) : 0;
+    const int64_t at = 2 * (kRight ? (int64_t)(p0 + col) * d + g * R : (int64_t)g * R * d + p0 + col);
+    if (kItem) {
+      long long *o = reinterpret_cast<long long *>(S.tp + item * dd) + at + comp, v[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[r] = kRight && r < live ? o[r * step] : 0;
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[r] = kRight ? v[r] - finish(A, r, O.bits - 31) : finish(A, r, O.bits - 31);
+      if (early) {
+        // element(): the real sum goes to the imaginary part, and out may be tp
+        __syncwarp();
+        const Unit f = unit(emax, O.hexp, comp ? O.hsign : -O.hsign);
+        const double *e = reinterpret_cast<const double *>(rest + col * (d | 1) + g * R) + (comp ^ 1);
+        const double *y = S.y ? reinterpret_cast<const double *>(S.y + item * dd) + at + (comp ^ 1) : nullptr;
+        double *out = reinterpret_cast<double *>(S.out + item * dd) + at + (comp ^ 1), yv[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) yv[r] = y && r < live ? y[2 * r] : 0.0;
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          if (r < live) out[2 * r] = fma(alpha, fma(f.f, sum_value(v[r], f), e[2 * r]), yv[r]);
+      } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          if (r < live) o[r * step] = v[r];
+      }
+    } else if (col < np) {
       // -i alpha (x + i y) = alpha (y - i x): the real sum goes to the imaginary part
       const Unit f = unit(lexp[col], O.hexp, comp == (kRight ? 1 : 0) ? -ah : ah);
       double *t = reinterpret_cast<double *>((early ? S.out : S.tp) + item * dd) + (comp ^ 1);
       double v[R], old[R];
-      double *o = t + 2 * (kRight ? (int64_t)(p0 + col) * d + g * R : (int64_t)g * R * d + p0 + col);
-      const int step = kRight ? 2 : 2 * d, live = min(R, d - g * R);
+      double *o = t + at;
 #pragma unroll
       for (int r = 0; r < R; ++r) old[r] = kRight && r < live ? o[r * step] : 0.0;
 #pragma unroll
@@ -447,7 +515,7 @@ __global__ void __launch_bounds__(panel_threads(R), panel_blocks(R))
   }
   if (kRight && !early) {
     __syncthreads();
-    elementwise(S.tp + item * dd);
+    elementwise();
   }
 }
 
@@ -638,9 +706,10 @@ __global__ void __launch_bounds__(512) f64_small_kernel(const __grid_constant__ 
             x2 += (long long)g.y * t.x;
           }
           const Unit f = unit(ie[it], O.hexp, comp ? -O.hsign : O.hsign);
-          const double cm = sum_value(((h1 - h2) << 1) + ((x1 - x2 + (1LL << (low - 2))) >> (low - 1)), f);
-          // acc = -gamma w + sum_s [ +- f_s A_s(other component) + g_s B_s ] +- f C
-          double acc = -I->decay * wv, A = 0.0, B = 0.0;
+          const double cm = sum_value(finish(h1, x1, low) - finish(h2, x2, low), f);
+          // acc = -gamma w + sum_s [ +- f_s A_s(other component) + g_s B_s ] +- f C, the
+          // operations of stage_element in their order
+          double acc = fma(-I->decay, wv, 0.0), A = 0.0, B = 0.0;
           int m = 0;
           bool any = false, both = false;
           auto close = [&]() {
@@ -658,7 +727,7 @@ __global__ void __launch_bounds__(512) f64_small_kernel(const __grid_constant__ 
             const F64Entry &en = I->e[j];
             const double o = comp ? v.x : v.y;
             if (en.kind == 0) {
-              A = any ? A + o : o;
+              A = any ? __dadd_rn(A, o) : o;
             } else {
               A = any ? fma(en.cA, o, A) : en.cA * o;
               if (en.kind == 2) {
@@ -989,6 +1058,8 @@ int table_size(const Model &M) {
 
 size_t panel_smem(int d, int tab) { return (size_t)tab * 16 + (size_t)d * (kPanel + 1) * 16; }
 
+size_t item_panel_smem(int d, int tab) { return panel_smem(d, tab) + (size_t)kPanel * (d | 1) * 16; }
+
 size_t fused_smem(int d, int tab, int m, bool t) {
   return (size_t)tab * 16 + (size_t)m * d * (d | 1) * 16 * (t ? 2 : 1) + (size_t)m * (sizeof(List) + 4) + 64;
 }
@@ -1005,15 +1076,24 @@ int row_group(const Model &M) {
   return n % 5 == 0 ? 5 : n % 3 == 0 ? 6 : 4;
 }
 
-// Panels instead of whole items?  An item keeps one SM busy for 40 us at d = 36, 70 us at
-// d = 64 and 150 us at d = 80, so a launch with few items per SM spreads each over panels:
-// fewer than four per SM from d = 46 on, 1.5 at d = 36.  Two steps at d = 36, 28 items: 359
-// against 503 us, 196 items 580 against 709, 280 items 796 against 742; d = 45, 252 items:
-// 847 against 985, 588 items 1603 against 1548; one stage at d = 64, 3360 items: 1839
-// against 1737.
-bool use_panels(int d, int tab, int64_t items) {
-  return fused_smem(d, tab, 1, false) > kFusedSmem ||
-         (d > 32 && items < (int64_t)sm_count() * std::min(d - 30, 16) / 4);
+// Panels instead of whole items?  An item keeps one SM busy for 40 us at d = 36 and 160 us at
+// d = 64, so a launch with few items spreads each over panels; from d = 69 on an SM holds two
+// whole items at most, and panels, which an SM holds more of, are faster for any number.  Us
+// per stage, items / panels (15 exponents' neighbours), by number of items: d = 36, 160
+// items: 61 / 50, 240: 63 / 64, 480: 96 / 104; d = 45, 480: 139 / 131, 960: 224 / 221, 1280:
+// 281 / 286; d = 48, 640: 189 / 187, 960: 248 / 259; d = 60, 1920: 822 / 818, 2560: 1058 /
+// 1067; d = 64, 80: 172 / 69, 480: 355 / 257, 1920: 960 / 937, 2560: 1231 / 1233; d = 72,
+// 3840: 3749 / 2523; d = 80, 80: 297 / 102, 3840: 3996 / 3338.
+enum Variant { kItems = 0, kItemPanels = 1, kPanels = 2 };
+
+Variant variant_of(int d, int tab, int64_t items) {
+  const size_t one = fused_smem(d, tab, 1, false);
+  if (one > kFusedSmem) return kPanels;
+  if (d <= 32) return kItems;
+  if (3 * (one + 1024) > kMaxSmem + 1024) return kItemPanels;
+  // items per SM: 1.5 at d = 36, 4.6 at d = 48, 16.5 at d = 64
+  const int64_t x = d - 30, per_sm_280 = std::max<int64_t>(70 * std::min<int64_t>(x, 15), 4 * x * x);
+  return items * 280 < sm_count() * per_sm_280 ? kItemPanels : kItems;
 }
 
 // Threads of a panel block: small blocks are out of step with one another, so that the
@@ -1038,7 +1118,7 @@ int items_per_block(int d, int tab, int64_t items) {
   return m;
 }
 
-F64Set make_set(const F64Buf &b, int64_t begin, bool *panels, size_t *smem, int64_t *blocks) {
+F64Set make_set(const F64Buf &b, int64_t begin, Variant *variant, size_t *smem, int64_t *blocks) {
   const F64Ops &O = *b.ops;
   F64Set s{};
   s.O = O;
@@ -1048,15 +1128,15 @@ F64Set make_set(const F64Buf &b, int64_t begin, bool *panels, size_t *smem, int6
   s.tp = b.tp;
   s.begin = begin;
   s.items = (int64_t)b.branches * O.n_ado;
-  *panels = use_panels(O.d, O.tab, s.items);
-  if (!*panels) {
+  *variant = variant_of(O.d, O.tab, s.items);
+  if (*variant == kItems) {
     s.per_block = items_per_block(O.d, O.tab, s.items);
     s.smem_t = fused_smem(O.d, O.tab, s.per_block, true) <= 56 * 1024;
     *smem = fused_smem(O.d, O.tab, s.per_block, s.smem_t);
     *blocks = (s.items + s.per_block - 1) / s.per_block;
   } else {
     s.per_block = (O.d + kPanel - 1) / kPanel;
-    *smem = panel_smem(O.d, O.tab);
+    *smem = *variant == kItemPanels ? item_panel_smem(O.d, O.tab) : panel_smem(O.d, O.tab);
     *blocks = s.items * s.per_block;
   }
   return s;
@@ -1070,32 +1150,35 @@ void allow_smem(K kernel, size_t smem, size_t most) {
     CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
 }
 
+template <int R, bool kMulti, bool kItem>
+void launch_panels(const F64Args &a, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
+  allow_smem(f64_panel_kernel<R, false, kMulti, kItem>, smem, kStageSmem);
+  allow_smem(f64_panel_kernel<R, true, kMulti, kItem>, smem, kStageSmem);
+  f64_panel_kernel<R, false, kMulti, kItem><<<(unsigned)blocks, threads, smem, st>>>(a);
+  f64_panel_kernel<R, true, kMulti, kItem><<<(unsigned)blocks, threads, smem, st>>>(a);
+  count_launch(2);
+}
+
 template <int R, bool kMulti>
-void launch_r(const F64Args &a, bool panels, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
-  if (panels) {
-    allow_smem(f64_panel_kernel<R, false, kMulti>, smem, kStageSmem);
-    allow_smem(f64_panel_kernel<R, true, kMulti>, smem, kStageSmem);
-    f64_panel_kernel<R, false, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
-    f64_panel_kernel<R, true, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
-    count_launch(2);
-    return;
-  }
+void launch_r(const F64Args &a, Variant variant, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
+  if (variant == kItemPanels) return launch_panels<R, kMulti, true>(a, blocks, smem, threads, st);
+  if (variant == kPanels) return launch_panels<R, kMulti, false>(a, blocks, smem, threads, st);
   allow_smem(f64_item_kernel<R, kMulti>, smem, kStageSmem);
   f64_item_kernel<R, kMulti><<<(unsigned)blocks, threads, smem, st>>>(a);
   count_launch(1);
 }
 
-void launch(const F64Args &a, int R, bool panels, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
+void launch(const F64Args &a, int R, Variant variant, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
   if (blocks == 0) return;
   if (blocks > 0x7fffffffLL) throw std::invalid_argument("too many work items for one stage launch");
   auto with = [&](auto multi) {
     constexpr bool m = decltype(multi)::value;
     if (R == 4)
-      launch_r<4, m>(a, panels, blocks, smem, threads, st);
+      launch_r<4, m>(a, variant, blocks, smem, threads, st);
     else if (R == 5)
-      launch_r<5, m>(a, panels, blocks, smem, threads, st);
+      launch_r<5, m>(a, variant, blocks, smem, threads, st);
     else
-      launch_r<6, m>(a, panels, blocks, smem, threads, st);
+      launch_r<6, m>(a, variant, blocks, smem, threads, st);
   };
   if (a.n > 0)
     with(std::true_type());
@@ -1169,6 +1252,10 @@ F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::
     return r;
   };
   std::vector<int> foff(1, 0), fc, doff(1, 0), soff(1, 0);
+  std::vector<int2> hd(d <= kSmallD ? (size_t)d * d : 0);   // the same limbs, dense
+  auto dense = [&](int a, int c, const int2 &v) {
+    if (a < d && !hd.empty()) hd[(size_t)a * d + c] = v;
+  };
   std::vector<int4> fh, dh, sh;
   const bool aligned = R == M.dims.back();   // a group is the last mode's digits
   auto last_digit_kept = [&](int a, int c) { return a % R == c % R; };
@@ -1184,6 +1271,8 @@ F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::
         for (int p = 0; p < (R + 1) / 2; ++p) {
           const int2 u = a0 + 2 * p < a1 ? limbs(a0 + 2 * p, c) : make_int2(0, 0);
           const int2 v = 2 * p + 1 >= R ? make_int2(c, 0) : a0 + 2 * p + 1 < a1 ? limbs(a0 + 2 * p + 1, c) : make_int2(0, 0);
+          dense(a0 + 2 * p, c, u);
+          if (2 * p + 1 < R) dense(a0 + 2 * p + 1, c, v);
           fh.push_back(make_int4(u.x, u.y, v.x, v.y));
         }
       } else {
@@ -1198,7 +1287,10 @@ F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::
         if (last_digit_kept(a0, c)) {
           const int2 v = limbs(a0, c);
           dh.push_back(make_int4(v.x, v.y, c, 0));
-          for (int r = 0; r < R; ++r) single[r].erase(std::find(single[r].begin(), single[r].end(), c + r));
+          for (int r = 0; r < R; ++r) {
+            single[r].erase(std::find(single[r].begin(), single[r].end(), c + r));
+            dense(a0 + r, c + r, v);
+          }
         }
     }
     doff.push_back((int)dh.size());
@@ -1206,6 +1298,7 @@ F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::
       for (int c : single[r]) {
         const int2 v = limbs(a0 + r, c);
         sh.push_back(make_int4(v.x, v.y, c, 0));
+        dense(a0 + r, c, v);
       }
       soff.push_back((int)sh.size());
     }
@@ -1224,12 +1317,7 @@ F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::
                                   (M.cb_lam[s][a] + M.cb_lam[s][b]) + (M.cb_lam_lo[s][a] + M.cb_lam_lo[s][b])));
     for (int a = 0; a < d; ++a) dig[(size_t)s * d + a] = (uint16_t)((a / M.stride[s]) % M.dims[s]);
   }
-  if (d <= kSmallD) {
-    std::vector<int2> hd((size_t)d * d);
-    for (int a = 0; a < d; ++a)
-      for (int c = 0; c < d; ++c) hd[(size_t)a * d + c] = digits_differ(M, a, c) <= 2 ? limbs(a, c) : make_int2(0, 0);
-    O.hd = up(hd, allocs);
-  }
+  if (!hd.empty()) O.hd = up(hd, allocs);
   O.foff = up(foff, allocs);
   O.fc = up(fc, allocs);
   O.fh = up(fh, allocs);
@@ -1249,25 +1337,25 @@ F64Ops f64_build(const Model &M, const std::vector<int32_t> &nb_off, const std::
 }
 
 std::vector<std::pair<int, int>> f64_shapes(const F64Buf &b) {
-  bool panels = false;
+  Variant variant = kItems;
   size_t smem = 0;
   int64_t blocks = 0;
-  make_set(b, 0, &panels, &smem, &blocks);
+  make_set(b, 0, &variant, &smem, &blocks);
   const int n = (int)std::min<int64_t>(blocks, 0x7fffffff);
-  if (!panels) return {{256, n}, {128, n}, {64, n}};
+  if (variant == kItems) return {{256, n}, {128, n}, {64, n}};
   const int t = panel_shape(b.ops->R, blocks);
   return b.ops->R == 5 ? std::vector<std::pair<int, int>>{{t, n}, {480 - t, n}}
                        : std::vector<std::pair<int, int>>{{t, n}, {640 - t, n}, {128, n}};
 }
 
 void f64_stage(const F64Buf &b, double alpha, int threads, cudaStream_t st) {
-  bool panels = false;
+  Variant variant = kItems;
   size_t smem = 0;
   int64_t blocks = 0;
   F64Args a{};
-  a.one = make_set(b, 0, &panels, &smem, &blocks);
+  a.one = make_set(b, 0, &variant, &smem, &blocks);
   a.alpha = alpha;
-  launch(a, b.ops->R, panels, blocks, smem, threads, st);
+  launch(a, b.ops->R, variant, blocks, smem, threads, st);
 }
 
 namespace {
@@ -1449,18 +1537,18 @@ void f64_plan(F64Plan &p, const std::vector<F64Buf> &sets, cudaStream_t st) {
   std::map<std::pair<int, int>, std::vector<F64Set>> by;
   std::map<std::pair<int, int>, std::pair<int64_t, size_t>> size;
   for (const F64Buf &b : sets) {
-    bool panels = false;
+    Variant variant = kItems;
     size_t smem = 0;
     int64_t blocks = 0;
-    F64Set s = make_set(b, 0, &panels, &smem, &blocks);
-    auto key = std::make_pair(b.ops->R, (int)panels);
+    F64Set s = make_set(b, 0, &variant, &smem, &blocks);
+    const auto key = std::make_pair(b.ops->R, (int)variant);
     s.begin = size[key].first;
     size[key].first += blocks;
     size[key].second = std::max(size[key].second, smem);
     by[key].push_back(s);
   }
   for (auto &kv : by) {
-    F64Plan::Class c{kv.first.first, kv.first.second != 0, size[kv.first].first, size[kv.first].second,
+    F64Plan::Class c{kv.first.first, kv.first.second, size[kv.first].first, size[kv.first].second,
                      (int)kv.second.size(), nullptr};
     if (device_malloc(&c.desc, kv.second.size() * sizeof(F64Set)) != cudaSuccess) {
       (void)cudaGetLastError();
@@ -1478,7 +1566,7 @@ void f64_stage_plan(const F64Plan &p, double alpha, cudaStream_t st) {
     a.many = (const F64Set *)c.desc;
     a.n = c.n;
     a.alpha = alpha;
-    launch(a, c.R, c.panels, c.blocks, c.smem, c.panels ? panel_shape(c.R, c.blocks) : 256, st);
+    launch(a, c.R, (Variant)c.variant, c.blocks, c.smem, c.variant == kItems ? 256 : panel_shape(c.R, c.blocks), st);
   }
 }
 

@@ -103,8 +103,7 @@ bool f64_small_steps_plan(const F64SmallPlan &p, double dt, int64_t steps, cudaS
 // One stage of several hierarchies: a plan (device descriptors) per set of buffers.
 struct F64Plan {
   struct Class {   // sets of one kernel variant
-    int R;
-    bool panels;
+    int R, variant;
     int64_t blocks;
     size_t smem;
     int n;
