@@ -991,7 +991,7 @@ const T *up(const std::vector<T> &v, std::vector<void *> &allocs) {
     throw DeviceOom();
   }
   allocs.push_back(p);
-  if (!v.empty()) cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
+  if (!v.empty()) CUDA_TRY(cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
   return (const T *)p;
 }
 
@@ -1066,8 +1066,8 @@ size_t fused_smem(int d, int tab, int m, bool t) {
 
 int sm_count() {
   int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  CUDA_TRY(cudaGetDevice(&dev));
+  CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   return sms;
 }
 
@@ -1502,8 +1502,8 @@ void f64_small_plan(F64SmallPlan &p, const std::vector<F64SmallBuf> &sets, cudaS
     (void)cudaGetLastError();
     throw DeviceOom();
   }
-  cudaMemcpyAsync(p.desc, v.data(), v.size() * sizeof(F64SmallSet), cudaMemcpyHostToDevice, st);
-  cudaStreamSynchronize(st);
+  CUDA_TRY(cudaMemcpyAsync(p.desc, v.data(), v.size() * sizeof(F64SmallSet), cudaMemcpyHostToDevice, st));
+  CUDA_TRY(cudaStreamSynchronize(st));
   p.n = (int)v.size();
   p.sync = sh.sync;
   p.blocks = sh.blocks;
@@ -1555,9 +1555,9 @@ void f64_plan(F64Plan &p, const std::vector<F64Buf> &sets, cudaStream_t st) {
       throw DeviceOom();
     }
     p.classes.push_back(c);
-    cudaMemcpyAsync(c.desc, kv.second.data(), kv.second.size() * sizeof(F64Set), cudaMemcpyHostToDevice, st);
+    CUDA_TRY(cudaMemcpyAsync(c.desc, kv.second.data(), kv.second.size() * sizeof(F64Set), cudaMemcpyHostToDevice, st));
   }
-  cudaStreamSynchronize(st);
+  CUDA_TRY(cudaStreamSynchronize(st));
 }
 
 void f64_stage_plan(const F64Plan &p, double alpha, cudaStream_t st) {

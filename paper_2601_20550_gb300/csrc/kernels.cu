@@ -1,10 +1,8 @@
 // Non-template kernels: 2D Fourier sums / correlation spectrum and state conversion.
 #include "fixed54.cuh"
-#include "kernels.cuh"
+#include "internal.h"
 
 namespace heom {
-
-void count_launch(uint64_t n);
 
 __global__ void __launch_bounds__(256) dft_twiddle_kernel(double2 *__restrict__ tw, int n1, int n3) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -567,7 +565,7 @@ template <int kOp>
 static void comm32(const float2 *w, const float2 *y, float2 *out, const float *K, int d, int64_t items, float alpha,
                    const VbModel &M, cudaStream_t st) {
   const int tiles = (d + kC32Tile - 1) / kC32Tile;
-  cudaFuncSetAttribute(comm32_kernel<kOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, kC32Smem);
+  CUDA_TRY(cudaFuncSetAttribute(comm32_kernel<kOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, kC32Smem));
   comm32_kernel<kOp><<<(unsigned)(items * tiles * tiles), 256, kC32Smem, st>>>(w, y, out, K, d, tiles, alpha, M);
   count_launch(1);
 }
