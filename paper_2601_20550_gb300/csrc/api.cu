@@ -287,12 +287,21 @@ void rk4_steps(heom_hier *h, typename CxT<R>::type *y, typename CxT<R>::type *wa
   if (h->f64.ready) work_out(h, dy, dy, da, branches, st);
 }
 
+// Tiles?  The FP64 ones (kick64_kernel) take both factors as fixed point against the largest
+// entry of a tile's slice.  A state in the coupling basis has that accuracy anyway; in the
+// product basis, where users see populations and coherences over many decades, every product
+// is rounded by itself (kick_kernel).
+static bool tiled_kick(const heom_hier *h, const double *K) {
+  return h->M.d >= kKickTiledMinD && K != h->mu64 && K != h->mup64 && K != h->mum64;
+}
+static bool tiled_kick(const heom_hier *h, const float *) { return h->M.d >= kKickTiledMinD; }
+
 template <typename R>
 void kick_into(heom_hier *h, const typename CxT<R>::type *in, typename CxT<R>::type *out,
                       int branches, const R *K, cudaStream_t st) {
   const Model &M = h->M;
   const int64_t total = (int64_t)branches * M.n_ado * M.d * M.d;
-  if (M.d >= kKickTiledMinD) {
+  if (tiled_kick(h, K)) {
     kick_tiled(in, out, K, M.d, (int64_t)branches * M.n_ado, false, st);
     LAUNCH_CHECK();
     return;
@@ -307,7 +316,7 @@ void kick2_into(heom_hier *h, const typename CxT<R>::type *T, typename CxT<R>::t
                 typename CxT<R>::type *outII, const R *KI, const R *KII, cudaStream_t st) {
   const Model &M = h->M;
   const int64_t total = (int64_t)M.n_ado * M.d * M.d;
-  if (M.d >= kKickTiledMinD) {
+  if (tiled_kick(h, KI)) {
     kick_tiled(T, outI, KI, M.d, M.n_ado, false, st);
     kick_tiled(T, outII, KII, M.d, M.n_ado, true, st);
     LAUNCH_CHECK();

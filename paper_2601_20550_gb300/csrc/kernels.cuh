@@ -142,7 +142,8 @@ __global__ void __launch_bounds__(256) kick_kernel(const typename CxT<R>::type *
 }
 
 // The same through shared-memory tiles, and with dagger for -w^dagger in place of w: FP64
-// in integer products (fixed54.cuh), FP32 with kick_kernel<float>'s bits.  One thread per
+// in integer products (fixed54.cuh), for coupling-basis states only: entries below 2^-55 of
+// a slice's largest are zero to it; FP32 with kick_kernel<float>'s bits.  One thread per
 // entry reads 4 d values for 4 d multiply-adds of its own; it is as fast below d = 40 and
 // few items (FP64, 28 items: 22 against 28 us at d = 36, 40 against 28 us at d = 40;
 // FP32, 28 items: 14 against 17 us at d = 64, but 924 items 183 against 73 us).  d = 216:
