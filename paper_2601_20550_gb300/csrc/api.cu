@@ -159,8 +159,8 @@ void work_in(heom_hier *h, const double2 *x, double2 *out, double2 *tmp, int bra
   } else if (h->rot.ready) {
     rotate(h->rot, true, x, out, tmp, items, st);
   } else {
-    sim_left_kernel<double2><<<grid_for(elems), 256, 0, st>>>(x, tmp, h->U64, h->M.d, elems);
-    sim_right_kernel<double2><<<grid_for(elems), 256, 0, st>>>(tmp, out, h->U64, h->M.d, elems);
+    sim_left_kernel<double2><<<grid_for(elems), 256, 0, st>>>(x, tmp, h->Uw64, h->M.d, elems);
+    sim_right_kernel<double2><<<grid_for(elems), 256, 0, st>>>(tmp, out, h->Uw64, h->M.d, elems);
     count_launch(2);
   }
   LAUNCH_CHECK();
@@ -173,8 +173,8 @@ void work_out(heom_hier *h, const double2 *x, double2 *out, double2 *tmp, int br
   } else if (h->rot.ready) {
     rotate(h->rot, false, x, out, tmp, items, st);
   } else {
-    sim_left_kernel<double2><<<grid_for(elems), 256, 0, st>>>(x, tmp, h->UT64, h->M.d, elems);
-    sim_right_kernel<double2><<<grid_for(elems), 256, 0, st>>>(tmp, out, h->UT64, h->M.d, elems);
+    sim_left_kernel<double2><<<grid_for(elems), 256, 0, st>>>(x, tmp, h->UTw64, h->M.d, elems);
+    sim_right_kernel<double2><<<grid_for(elems), 256, 0, st>>>(tmp, out, h->UTw64, h->M.d, elems);
     count_launch(2);
   }
   LAUNCH_CHECK();
@@ -562,6 +562,13 @@ void ensure_device(heom_hier *h) {
     std::vector<double> mm(mp.size());
     for (int a = 0; a < M.d; ++a)
       for (int b = 0; b < M.d; ++b) mm[(size_t)a * M.d + b] = mp[(size_t)b * M.d + a];
+    if (!h->rot.ready) {
+      const std::vector<double> U = mode_product(M, M.cb_U);
+      for (int a = 0; a < M.d; ++a)
+        for (int b = 0; b < M.d; ++b) UT[(size_t)a * M.d + b] = U[(size_t)b * M.d + a];
+      h->Uw64 = h->up(U);
+      h->UTw64 = h->up(UT);
+    }
     h->mu_w64 = h->up(f64_matrix(M, M.mu));
     h->mup_w64 = h->up(mp);
     h->mum_w64 = h->up(mm);

@@ -542,7 +542,8 @@ extern "C" heom_status heom_response_2d_grad(heom_hier *h, const heom_state *rho
             for (int k = 0; k < n; ++k) r[(size_t)a * n + b] += t[(size_t)a * n + k] * U[(size_t)b * n + k];
         std::copy(r.begin(), r.end(), g);
       };
-      for (int64_t o : {c.L.H, c.L.mup, c.L.mum, c.L.mu}) back(G.data() + o, M.vb_U, d);
+      const std::vector<double> U = mode_product(M, M.cb_U);
+      for (int64_t o : {c.L.H, c.L.mup, c.L.mum, c.L.mu}) back(G.data() + o, U, d);
       int64_t o = c.L.v;
       for (int sm = 0; sm < M.n_modes; ++sm) {
         back(G.data() + o, M.cb_U[sm], M.dims[sm]);

@@ -130,7 +130,8 @@ struct heom_hier {
   double *mu_trace = nullptr;   // FP64 mu for traces
   TcOperators tc{};             // tensor-core operator tiles (HEOM_TC)
   VbModel vb{};                 // coupling-eigenbasis model (FP32 paths)
-  double *U64 = nullptr, *UT64 = nullptr;        // coupling eigenbasis U and U^T
+  double *U64 = nullptr, *UT64 = nullptr;        // coupling eigenbasis U and U^T (complex64 states)
+  double *Uw64 = nullptr, *UTw64 = nullptr;      // the FP64 path's, with the digits of its tables (f64.ready, not rot.ready)
   float *mu_vb32 = nullptr, *mup_vb32 = nullptr, *mum_vb32 = nullptr;
   double *mu_vb64 = nullptr;                     // mu in the coupling basis (traces of complex64 states)
   double *mu_w64 = nullptr, *mup_w64 = nullptr, *mum_w64 = nullptr;   // mu, mu+, mu- there (FP64 path)

@@ -403,6 +403,21 @@ static std::vector<double> similarity(const std::vector<double> &U, const std::v
   return out;
 }
 
+std::vector<double> mode_product(const Model &M, const std::vector<std::vector<double>> &Us) {
+  const int d = M.d;
+  std::vector<double> U((size_t)d * d, 0.0);
+  for (int a = 0; a < d; ++a)
+    for (int b = 0; b < d; ++b) {
+      double v = 1.0;
+      for (int s = 0; s < M.n_modes && v != 0.0; ++s) {
+        int as = (a / M.stride[s]) % M.dims[s], bs = (b / M.stride[s]) % M.dims[s];
+        v *= Us[s][(size_t)as * M.dims[s] + bs];
+      }
+      U[(size_t)a * d + b] = v;
+    }
+  return U;
+}
+
 void build_coupling_basis(Model &M) {
   const int d = M.d;
   std::vector<std::vector<double>> Us;
@@ -428,16 +443,7 @@ void build_coupling_basis(Model &M) {
     M.cb_lam_lo.push_back(wlo);
     M.cb_U_lo.push_back(lo);
   }
-  M.vb_U.assign((size_t)d * d, 0.0);
-  for (int a = 0; a < d; ++a)
-    for (int b = 0; b < d; ++b) {
-      double v = 1.0;
-      for (int s = 0; s < M.n_modes && v != 0.0; ++s) {
-        int as = (a / M.stride[s]) % M.dims[s], bs = (b / M.stride[s]) % M.dims[s];
-        v *= Us[s][(size_t)as * M.dims[s] + bs];
-      }
-      M.vb_U[(size_t)a * d + b] = v;
-    }
+  M.vb_U = mode_product(M, Us);
   M.vb_H = similarity(M.vb_U, M.H, d);
   M.vb_mu = similarity(M.vb_U, M.mu, d);
   M.vb_mu_plus = similarity(M.vb_U, M.mu_plus, d);

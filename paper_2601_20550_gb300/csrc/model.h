@@ -42,7 +42,9 @@ struct Model {
   std::vector<std::vector<double>> cb_lam, cb_lam_lo, cb_U, cb_U_lo;
 };
 
-// Coupling-eigenbasis quantities (fills vb_* of M).
+// Kronecker product of one matrix per mode.
+std::vector<double> mode_product(const Model &M, const std::vector<std::vector<double>> &Us);
+// Coupling-eigenbasis quantities (fills vb_* and cb_* of M).
 void build_coupling_basis(Model &M);
 
 void jacobi_eigh(std::vector<double> &A, int n, std::vector<double> &w, std::vector<double> &Z);
