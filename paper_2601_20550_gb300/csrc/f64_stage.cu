@@ -1170,7 +1170,7 @@ void launch_r(const F64Args &a, Variant variant, int64_t blocks, size_t smem, in
 
 void launch(const F64Args &a, int R, Variant variant, int64_t blocks, size_t smem, int threads, cudaStream_t st) {
   if (blocks == 0) return;
-  if (blocks > 0x7fffffffLL) throw std::invalid_argument("too many work items for one stage launch");
+  (void)grid_blocks(blocks);   // refuses what one launch cannot hold
   auto with = [&](auto multi) {
     constexpr bool m = decltype(multi)::value;
     if (R == 4)
@@ -1608,25 +1608,25 @@ RotOps rot_build(const Model &M, std::vector<void *> &allocs) {
 }
 
 void rotate(const RotOps &r, bool forward, const double2 *x, double2 *out, double2 *tmp, int64_t items, cudaStream_t st) {
-  if (items <= 0) return;
-  const int panels = (r.d + 31) / 32;
-  const int64_t blocks = items * panels;
-  if (blocks > 0x7fffffffLL) throw std::invalid_argument("too many work items for one launch");
+  const int panels = (r.d + 31) / 32, dd = r.d * r.d;
   const int2 *u = forward ? r.fwd : r.bwd;
-  if (r.d <= kSmallD) {
-    const int dd = r.d * r.d;
-    rotate_item_kernel<<<(unsigned)items, dd <= 64 ? 64 : dd <= 128 ? 128 : 256, r.d * (r.d | 1) * 16, st>>>(
-        x, out, u, r);
-    count_launch(1);
-    return;
+  const size_t smem = (size_t)r.d * (r.d <= kSmallD ? r.d | 1 : kRotPad) * 16;
+  if (r.d > kSmallD) {
+    allow_smem(rotate_kernel<false>, smem, kRotSmem);
+    allow_smem(rotate_kernel<true>, smem, kRotSmem);
   }
-  const size_t smem = (size_t)r.d * kRotPad * 16;
-  allow_smem(rotate_kernel<false>, smem, kRotSmem);
-  allow_smem(rotate_kernel<true>, smem, kRotSmem);
-  rotate_kernel<false><<<(unsigned)blocks, 256, smem, st>>>(x, tmp, u, r, panels);
-  rotate_kernel<true><<<(unsigned)blocks, 256, smem, st>>>(tmp, out, u, r, panels);
-  count_launch(2);
+  for (int64_t n = 0; items > 0; items -= n, x += ado_offset(n, r.d), out += ado_offset(n, r.d)) {
+    if (r.d <= kSmallD) {
+      n = launch_share(items, 1);
+      rotate_item_kernel<<<grid_blocks(n), dd <= 64 ? 64 : dd <= 128 ? 128 : 256, smem, st>>>(x, out, u, r);
+      count_launch(1);
+      continue;
+    }
+    n = launch_share(items, panels);
+    rotate_kernel<false><<<grid_blocks(n * panels), 256, smem, st>>>(x, tmp, u, r, panels);
+    rotate_kernel<true><<<grid_blocks(n * panels), 256, smem, st>>>(tmp, out, u, r, panels);
+    count_launch(2);
+  }
 }
-
 
 }  // namespace heom

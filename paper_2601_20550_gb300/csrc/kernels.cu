@@ -190,7 +190,7 @@ static __global__ void __launch_bounds__(256, 3) kick64_kernel(const double2 *__
 
 void kick_tiled(const double2 *w, double2 *out, const double *K, int d, int64_t items, bool dagger, cudaStream_t st) {
   const int tiles = (d + 31) / 32;
-  const unsigned blocks = (unsigned)(items * tiles * tiles);   // below 2^31: a tile has 8 KB of device memory or more
+  const unsigned blocks = grid_blocks(items * tiles * tiles);
   if (dagger)
     kick64_kernel<true><<<blocks, 256, 0, st>>>(w, out, K, d, tiles);
   else
@@ -566,7 +566,7 @@ static void comm32(const float2 *w, const float2 *y, float2 *out, const float *K
                    const VbModel &M, cudaStream_t st) {
   const int tiles = (d + kC32Tile - 1) / kC32Tile;
   CUDA_TRY(cudaFuncSetAttribute(comm32_kernel<kOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, kC32Smem));
-  comm32_kernel<kOp><<<(unsigned)(items * tiles * tiles), 256, kC32Smem, st>>>(w, y, out, K, d, tiles, alpha, M);
+  comm32_kernel<kOp><<<grid_blocks(items * tiles * tiles), 256, kC32Smem, st>>>(w, y, out, K, d, tiles, alpha, M);
   count_launch(1);
 }
 
@@ -580,7 +580,7 @@ void stage32(const float2 *w, const float2 *y, float2 *out, float alpha, const V
   const int64_t tiles = (M.d + kC32Tile - 1) / kC32Tile;
   if (M.d >= 36 && items * tiles * tiles >= 152) return comm32<2>(w, y, out, M.H, M.d, items, alpha, M, st);
   const int t32 = (M.d + 31) / 32;
-  stage_kernel_vb_tiled<<<(unsigned)(items * t32 * t32), 256, 0, st>>>(w, y, out, alpha, M, t32);
+  stage_kernel_vb_tiled<<<grid_blocks(items * t32 * t32), 256, 0, st>>>(w, y, out, alpha, M, t32);
   count_launch(1);
 }
 

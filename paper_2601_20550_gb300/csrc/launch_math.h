@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cstdint>
 #include <map>
+#include <stdexcept>
 #include <utility>
 #include <vector>
 
@@ -19,6 +20,17 @@ namespace heom {
 // First element of d x d matrix n of a state.  A branch may hold more than 2^31 elements
 // (d = 64, 646646 ADOs: 42 GB).
 HEOM_HD int64_t ado_offset(int64_t n, int d) { return n * ((int64_t)d * d); }
+
+// Blocks of a launch along x.
+constexpr int64_t kMaxBlocks = 0x7fffffff;
+
+inline unsigned grid_blocks(int64_t blocks) {
+  if (blocks < 0 || blocks > kMaxBlocks) throw std::invalid_argument("too many work items for one launch");
+  return (unsigned)blocks;
+}
+
+// Items that one launch takes of the rest, at per_item blocks each.
+inline int64_t launch_share(int64_t rest, int per_item) { return std::min(rest, kMaxBlocks / per_item); }
 
 // Launch shapes (threads per block, blocks) kept per (kernel kind, elements).
 using Shape = std::pair<int, int>;

@@ -50,3 +50,33 @@ def test_a_shape_kept_by_another_kernel_is_not_used(tmp_path):
   printf("%d ", heom::kept_shape(kept, 1, 100, mine[0], mine) != nullptr);
   printf("%d", heom::kept_shape(kept, 0, 101, mine[0], mine) != nullptr);""")
     assert out == ["0", "128", "9", "0", "0"]
+
+
+def test_blocks_of_a_launch(tmp_path):
+    """A grid beyond 2^31 - 1 blocks is refused, not truncated; work that can be split is taken
+    in launches that hold whole items and end."""
+    out = run(tmp_path, """
+  printf("%u ", heom::grid_blocks(0x7fffffffLL));
+  for (int64_t b : {0x80000000LL, 0x100000000LL, -1LL}) {
+    bool refused = false;
+    try { heom::grid_blocks(b); } catch (const std::invalid_argument &) { refused = true; }
+    printf("%d ", refused);
+  }
+  for (int per : {1, 3, 14})
+    for (int64_t items : {0LL, 5LL, 0x7fffffffLL, 2800000000LL, 9000000000LL}) {
+      int64_t rest = items, done = 0, n = 0;
+      int launches = 0;
+      for (; rest > 0; rest -= n, done += n, ++launches) {
+        n = heom::launch_share(rest, per);
+        heom::grid_blocks(n * per);
+      }
+      printf("%d ", done == items && launches == (items + 0x7fffffffLL / per - 1) / (0x7fffffffLL / per));
+    }""")
+    assert out == ["2147483647", "1", "1", "1"] + ["1"] * 15
+
+
+def test_tiled_launches_check_their_grids():
+    for name in ("kernels.cu", "f64_stage.cu"):
+        src = open(os.path.join(CSRC, name)).read()
+        assert not re.search(r"<<<\(unsigned\)\(items", src), name
+        assert not re.search(r"blocks = \(unsigned\)", src), name
