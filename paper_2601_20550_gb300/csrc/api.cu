@@ -819,7 +819,8 @@ heom_status heom_equilibrate(heom_hier *h, double dt_fs, double t_max_fs, double
     std::vector<double> hn(M.n_ado);
     int64_t done = 0;
     bool converged = false;
-    work_in(h, rho, rho, (double2 *)a.p, 1, h->stream);   // the residual's norms do not depend on the basis
+    // the residual's norms do not depend on the basis
+    if (nmax > 0) work_in(h, rho, rho, (double2 *)a.p, 1, h->stream);
     while (done < nmax && !converged) {
       int64_t chunk = std::min<int64_t>(100, nmax - done);
       rk4_work64(h, rho, (double2 *)a.p, (double2 *)b.p, 1, dt_fs, chunk, h->stream);
@@ -842,7 +843,7 @@ heom_status heom_equilibrate(heom_hier *h, double dt_fs, double t_max_fs, double
       if (!std::isfinite(res) || !std::isfinite(n0)) throw Fail{HEOM_ENONFINITE, "equilibrium residual is not finite"};
       converged = std::sqrt(res) <= tol * std::sqrt(n0);
     }
-    work_out(h, rho, rho, (double2 *)a.p, 1, h->stream);
+    if (nmax > 0) work_out(h, rho, rho, (double2 *)a.p, 1, h->stream);
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     if (converged) return HEOM_OK;
     g_last_error = "equilibrium tolerance not reached by t_max";

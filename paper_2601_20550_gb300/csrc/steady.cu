@@ -101,7 +101,12 @@ extern "C" heom_status heom_steady_state(heom_hier *h, double tol, int restart, 
     // products stay), x goes back to the product basis at the end
     work_in(h, x, x, wp, 1, st);
     auto back = [&]() {
-      work_out(h, x, x, wp, 1, st);
+      if (its == 0) {   // x is |0><0| still
+        CUDA_TRY(cudaMemsetAsync(x, 0, (size_t)n * 16, st));
+        CUDA_TRY(cudaMemcpyAsync(x, one, 16, cudaMemcpyHostToDevice, st));
+      } else {
+        work_out(h, x, x, wp, 1, st);
+      }
       CUDA_TRY(cudaStreamSynchronize(st));
     };
     while (its < max_iter) {
