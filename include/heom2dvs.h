@@ -164,6 +164,10 @@ int heom_state_branches(const heom_state *s);
  * Advance every branch of rho by n_steps RK4 steps of Eq. HEOM_DB (Sec. III).
  * The RK4 polynomial is evaluated in nested (Horner) form, identical to the
  * classic four-stage tableau for this linear, time-independent equation.
+ * FP64 states are propagated in the coupling eigenbasis: rounding errors are of the
+ * order 2^-53 of the largest entry of an ADO and of what its neighbours bring, not of
+ * each entry (a population of 1e-9 beside one of 1 keeps about eight digits).  A
+ * branch's result is the same bits alone, in any batch and in any row block.
  * Errors: HEOM_EINVAL, HEOM_EUNSTABLE (dt fails the stability pre-check),
  * HEOM_ECUDA.
  */
@@ -171,7 +175,8 @@ heom_status heom_propagate(heom_hier *h, heom_state *rho, double dt_fs, int64_t 
 
 /*
  * Apply the hyperoperator K^x (K = mu, mu_plus or mu_minus: which = 0, 1, 2) to
- * every ADO of every branch in place (the dipole kicks of Sec. II.C).
+ * every ADO of every branch in place (the dipole kicks of Sec. II.C).  FP64: every
+ * product is rounded by itself, so each entry is accurate relative to its own terms.
  */
 heom_status heom_kick(heom_hier *h, heom_state *rho, int which);
 
@@ -201,7 +206,7 @@ heom_status heom_response_2d(heom_hier *h, const heom_state *rho_eq, const heom_
  * Stationary hierarchy by a Krylov solve instead of propagation (the steady
  * state that the equilibration of Sec. II.C.1 approaches): restarted
  * GMRES(restart) from x = |0><0| on A x = 0 with A = L (the right-hand side of
- * Eq. HEOM_DB, FP64, product basis) when steps_per_matvec = 0, or A = G^k - 1
+ * Eq. HEOM_DB, FP64, in the coupling eigenbasis) when steps_per_matvec = 0, or A = G^k - 1
  * with G one RK4 step of dt_fs and k = steps_per_matvec.  Both have the steady
  * state as null vector; the second compresses the spectrum of a stiff hierarchy
  * (fast coherences, slow population transfer) into a range GMRES handles in a
@@ -272,8 +277,9 @@ heom_status heom_response_2d_grad(heom_hier *h, const heom_state *rho_eq, const 
  * set is an HEOM_FP64 hierarchy, the sets advance together: each RK4 stage of
  * all sets and all their branches is one launch per kernel variant that they take
  * (per-set tables and state pointers in a descriptor table; one launch for all
- * steps if every basis has at most 48 states), and each t3 scan is one CUDA-graph
- * replay.  When every set is an HEOM_TC hierarchy (up to 16 sets), each RK4
+ * steps if every basis has at most 48 states and every set's branches at most 1536
+ * elements per block, a block or a cluster of blocks per branch), and each t3 scan is
+ * one CUDA-graph replay.  When every set is an HEOM_TC hierarchy (up to 16 sets), each RK4
  * stage of the t2 forks and t3 scans of all sets is one tensor-core launch and
  * one coupling-kernel launch (per-set operators and buffers in the launch's
  * descriptor; a CTA reloads H' when its next item belongs to another set).  In
@@ -366,7 +372,9 @@ heom_status heom_trace_dev(heom_hier *h, const void *state, int branches, int pr
  * have its device tables (any earlier device call on it, e.g. heom_state_create).
  * Every call shares the one scratch array: calls that overlap on the GPU (other
  * streams, other threads, other hierarchies) race and must be serialised by the
- * caller.  No RK4 stability pre-check is made.
+ * caller.  No RK4 stability pre-check is made.  The stages run in the product
+ * basis, one thread per element: the result equals heom_propagate_dev's to rounding,
+ * not bit for bit, and small entries keep their own digits.
  */
 #define HEOM_NOALLOC_MAX_BYTES (16LL * 1024 * 1024)
 heom_status heom_propagate_noalloc(heom_hier *h, void *state, int branches, double dt_fs,

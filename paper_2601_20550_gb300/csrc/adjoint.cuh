@@ -57,7 +57,7 @@ static __global__ void __launch_bounds__(256) neg_dagger_kernel(const double2 *_
 // GB300 issues 2 FP64 operations per clock and SM, on the FP64 tensor instruction too, but
 // 32 multiply-adds of 32 x 32 + 64 bits, so the sums run in integers: the entries of a
 // 16-wide slice as 54-bit fixed point against the slice's largest exponent, in limbs of 28
-// and 26 bits, three products each (low x low is below 2^-56 of the largest), 64 exact
+// and 26 bits, three products each (low x low, 2^-58 of the largest, dropped), 64 exact
 // products per sum, then one FP64 addition.  Block = (16 T)^2 entries of G over a share of
 // the (item, slice) units, T x T per thread.  At d = 64, 224 items: 649 us with one FP64
 // sum per thread, 452 us in register tiles (the FP64 pipe's

@@ -2,16 +2,23 @@
 //
 // What bounds it.  GB300 issues 2 FP64 operations per clock and SM, 1/64 of its FP32
 // rate.  The commutator's 2 x 2 x d multiply-adds per element were nine tenths of the
-// stage on that pipe.  Here they run as exact integer products on the IMAD pipe (32
-// IMAD.WIDE per clock and SM): w (per item, or per column and row) and H' are scaled by
-// powers of two to 57 bits and cut into two signed limbs, 31 bits above 26, and
-//   sum_c h z = 2^52 sum h1 z1 + 2^26 sum (h1 z0 + h0 z1)   (+ h0 z0, dropped: below
-//   2^-60 of the largest value of the sum)
+// stage on that pipe.  Here they run as integer products on the IMAD pipe (32 IMAD.WIDE
+// per clock and SM): w (per item, or per column and row) and H' are rounded to 57-bit fixed
+// point and cut into two signed limbs, 31 bits above 26, and
+//   sum_c h z = 2^52 sum h1 z1 + 2^26 sum (h1 z0 + h0 z1)   (+ 2^0 sum h0 z0, dropped: each
+//   term at most 2^-62 of the largest value that the sum can take, so 2^-56.8 for the 37
+//   products of a row at four levels, 2^-54 for the 250 that 57 bits allow)
 // is accumulated without rounding in two 64-bit integers, three IMAD.WIDE per product;
 // only H''s structural non-zeros are multiplied (37 of 64 columns at four levels, 61 of
 // 125 at five).  The sums are rounded once when they turn back into FP64.  The
 // elementwise rest takes ~38 FP64 operations per element and stage and shares the SM
 // with the integer phase of other resident blocks.
+//
+// Accuracy is that of FP64 relative to the largest entry of an ADO (of a column or row of
+// it in the panels of large bases), not entry by entry: the change of basis alone mixes an
+// ADO's entries.  One mode of six levels, 40 steps from the ground state: the populations of
+// levels 1 to 5, 2e-7 to 2e-10, have absolute errors near 1e-17, relative ones of 1e-10 to
+// 6e-8 (2e-14 and less with stage_kernel<double> in the product basis).
 #include "f64_stage.h"
 
 #include <algorithm>
@@ -42,7 +49,8 @@ constexpr int kRotPad = 33;
 // items: 324 and 441 us.
 constexpr int kSmallD = 48;
 constexpr size_t kMaxSmem = 227 * 1024;
-// Whole-item blocks up to two per SM; above, one panel of columns (rows) per block.
+// Bases whose items fit a block, two of them per SM (up to 83 states), take the items'
+// arithmetic; larger ones always go by panels of columns and rows.
 constexpr size_t kFusedSmem = 112 * 1024;
 
 struct F64Set {
@@ -366,8 +374,9 @@ __global__ void __launch_bounds__(256, 4) f64_item_kernel(const __grid_constant_
 //
 // Otherwise: limbs scaled per column (row), tp = -i alpha H' w in FP64, on which the right
 // kernel adds in either order; ADO and panel decide, so that an element's additions have
-// one order wherever its branch stands.  d = 125, 924 items: 827 us and 1540 us; one thread
-// per element in the product basis took 17.4 ms.
+// one order wherever its branch stands.  d = 125, 924 items: 830 us (IMAD pipe 74 % busy)
+// and 1544 us (FP64 pipe 72 %, IMAD 52 %); one thread per element in the product basis took
+// 17.4 ms.
 // ---------------------------------------------------------------------------
 template <int R, bool kRight, bool kMulti, bool kItem>
 __global__ void __launch_bounds__(panel_threads(R), panel_blocks(R))
@@ -1100,9 +1109,9 @@ Variant variant_of(int d, int tab, int64_t items) {
 // products of some (IMAD pipe) run beside the elementwise part of others (FP64 pipe), and
 // the row groups divide evenly (25 at five levels, 16 at four); big ones where a launch
 // has few blocks or a basis that leaves room for three.  d = 125, 924 items: 160 threads
-// 827 + 1540 us, 320 854 + 1669 us; d = 64, 896 blocks: 256 threads 48 + 98 us, 384 53 +
-// 103 us; 112 blocks: 21 + 37 and 21 + 35 us; d = 216, 1920 blocks: 384 threads 460 + 596
-// us, 192 639 + 798 us.
+// 827 + 1540 us, 320 854 + 1669 us; d = 64, both launches, 896 blocks: 256 threads 140
+// us, 384 159 us; 112 blocks: 57 and 53 us; d = 216, 1920 blocks: 384 threads 460 + 596 us,
+// 192 639 + 798 us.
 int panel_shape(int R, int64_t blocks) {
   const int sms = sm_count();
   if (R == 5) return blocks >= 4 * sms ? 160 : 320;

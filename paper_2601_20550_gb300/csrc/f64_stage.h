@@ -4,8 +4,9 @@
 // (rho' = U^T rho U, U the Kronecker product of the per-mode eigenvectors of V_s):
 // the system-bath terms are elementwise there, and H' = U^T H_S' U keeps H_S''s
 // structure (elements between states that differ in three or more modes vanish).
-// The commutator [H', w] runs in exact integer arithmetic on the IMAD pipe (see
-// f64_stage.cu); everything else is FP64.
+// The commutator [H', w] runs in 57-bit fixed point on the IMAD pipe, its sums in integers
+// (see f64_stage.cu, also for the accuracy); everything else is FP64.  An item's result is
+// the same bits in every kernel that takes its basis, so it does not depend on the batch.
 #pragma once
 
 #include <cstdint>

@@ -1,8 +1,9 @@
-// FP64 products as exact integer sums: 54-bit fixed point against a common exponent, in
-// limbs of 28 and 26 bits (q = hi 2^26 + lo), so that up to 64 products hi x hi and 128
-// products hi x lo sum exactly in 64 bits.  GB300 issues 2 FP64 operations per clock and
-// SM but 32 multiply-adds of 32 x 32 + 64 bits: three per product (lo x lo stays below
-// 2^-56 of the largest).
+// FP64 products as integer sums: 54-bit fixed point against a common exponent, in limbs of
+// 28 and 26 bits (q = hi 2^26 + lo), so that up to 64 products hi x hi and 128 products
+// hi x lo sum without rounding in 64 bits.  GB300 issues 2 FP64 operations per clock and SM
+// but 32 multiply-adds of 32 x 32 + 64 bits: three per product (lo x lo, at most 2^-58 of
+// the largest product each, is dropped).  Errors are relative to the largest of the values
+// that share the exponent.
 #pragma once
 
 #include <cuda_runtime.h>
