@@ -28,8 +28,8 @@ namespace heom {
 struct MultiSet {
   heom_hier *h;
   const heom_state *eq;
-  int64_t per;                                          // n_ado d^2
-  std::unique_ptr<DeviceBuffer> eqW, T, ta, tb, P[4];   // equilibrium, trunk and its scratch; branch sets
+  int64_t per;                                     // n_ado d^2
+  std::unique_ptr<DeviceBuffer> T, ta, tb, P[4];   // trunk and its scratch; branch sets
 };
 
 // Plans of RK4 steps on the buffers (y, wa, wb) of every set: all steps in one launch if
@@ -94,8 +94,6 @@ static void response_2d_multi(heom_hier *const *hs, const heom_state *const *eqs
     S[k].T.reset(new DeviceBuffer(S[k].per * 16));
     S[k].ta.reset(new DeviceBuffer(S[k].per * 16));
     S[k].tb.reset(new DeviceBuffer(S[k].per * 16));
-    S[k].eqW.reset(new DeviceBuffer(S[k].per * 16));
-    work_in(hs[k], (const double2 *)eqs[k]->buf.p, (double2 *)S[k].eqW->p, (double2 *)S[k].ta->p, 1, st);
   }
   // t1 rows per chunk: both pathways of J rows, 3 or 4 branch sets per parameter set
   const int nbuf = nt2 > 1 ? 4 : 3;
@@ -116,8 +114,11 @@ static void response_2d_multi(heom_hier *const *hs, const heom_state *const *eqs
     multi_step_setup(S, fork, 0, 1, 2, B, st);                       // y = BR, scratch Y, WA
     multi_step_setup(S, scan, 1, 2, nbuf == 4 ? 3 : 0, B, st);       // y = Y, scratch WA, WB
     PhaseRange phase("heom: t1 trunk (sets)");
-    for (int k = 0; k < n_sets; ++k)
-      kick_into<double>(S[k].h, (const double2 *)S[k].eqW->p, (double2 *)S[k].T->p, 1, mu_work<double>(S[k].h, 2), st);
+    for (int k = 0; k < n_sets; ++k) {   // the equilibrium passes through the trunk's scratch
+      double2 *T = (double2 *)S[k].T->p, *ta = (double2 *)S[k].ta->p, *tb = (double2 *)S[k].tb->p;
+      work_in(S[k].h, (const double2 *)S[k].eq->buf.p, ta, tb, 1, st);
+      kick_into<double>(S[k].h, ta, T, 1, mu_work<double>(S[k].h, 2), st);
+    }
     multi_rk4(trunk, dt, (int64_t)j0 * m, st);
     for (int j = 0; j < nj; ++j) {
       if (j > 0) multi_rk4(trunk, dt, m, st);
